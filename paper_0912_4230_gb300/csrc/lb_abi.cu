@@ -47,6 +47,7 @@ struct lb_ctx {
   cudaStream_t stream = nullptr;
   unsigned N = 0, nblk = 0;
   dim3 sgrid, sblock;  // launch shape of the per-cell step kernel
+  bool linear = false;  // ... which takes the cells in the order of n (sgrid.x blocks)
   unsigned nwarps = 0;   // flux slots (one per warp of the step launch)
   bool use_tma = false;  // row-pipelined step kernel in use
   bool tma_ok = false;   // ... and available for this lattice
@@ -210,13 +211,35 @@ const StorageOps *ops_of(int storage) {
   }
 }
 
-// Launch shape of the per-cell step kernel: rows of BX threads (a multiple
-// of 32, up to the lattice width), BY rows per block.
-void cell_shape(const lb_domain &dom, dim3 *grid, dim3 *block) {
+// Launch shape of the per-cell step kernel by rows: BX threads (a multiple of
+// 32, up to the lattice width), BY rows per block.
+void row_shape(const lb_domain &dom, dim3 *grid, dim3 *block) {
   unsigned bx = 32;
   while (bx < unsigned(STEP_BLOCK) && bx < unsigned(dom.nx)) bx *= 2;
   *block = dim3(bx, STEP_BLOCK / bx, 1);
   *grid = dim3((dom.nx + bx - 1) / bx, (dom.ny + block->y - 1) / block->y, dom.nz);
+}
+// ... over the cells in order of n (never more blocks than by rows, which hold
+// STEP_BLOCK cells or fewer each, so the flux slots cover it too).
+// Where all warps of the launch are resident at once (152 SMs of 24 warps; FP64
+// 12) blocks of one warp spread them evenly: 254 warps of FP64 work are 2 on
+// the busiest SM instead of 4.
+void linear_shape(const lb_domain &dom, bool fp64, dim3 *grid, dim3 *block) {
+  const size_t N = size_t(dom.nx) * dom.ny * dom.nz;
+  const unsigned threads = N <= size_t(152) * 32 * (fp64 ? 12 : 24) ? 32 : STEP_BLOCK;
+  *block = dim3(threads, 1, 1);
+  *grid = dim3(unsigned((N + threads - 1) / threads), 1, 1);
+}
+// The default: by rows where that leaves no thread idle, else linear.
+bool cell_shape(const lb_domain &dom, bool fp64, dim3 *grid, dim3 *block) {
+  row_shape(dom, grid, block);
+  dim3 lg, lb;
+  linear_shape(dom, fp64, &lg, &lb);
+  if (lb.x == unsigned(STEP_BLOCK) && dom.nx % int(block->x) == 0 && dom.ny % int(block->y) == 0)
+    return false;
+  *grid = lg;
+  *block = lb;
+  return true;
 }
 
 // Flux slots: one pair per warp of the widest launch any step kernel may
@@ -300,7 +323,7 @@ Layout layout_of(const lb_domain &dom, const lb_params &prm, const StorageOps &o
   L.create_stage = N * 4 + (k_rows ? 6 * N * 4 : 0) + N + 64 + 256;
   L.init_stage = N * 4 * (4 + S) + (f_scale ? size_t(Q) * N * 4 : 0) + N * 4 + N + 256;
   dim3 g, b;
-  cell_shape(dom, &g, &b);
+  row_shape(dom, &g, &b);  // at least as many blocks as any other shape by default
   L.batch_share = size_t(g.x) * g.y * g.z * sizeof(uint64_t);
   return L;
 }
@@ -309,6 +332,15 @@ Layout layout_of(const lb_domain &dom, const lb_params &prm, const StorageOps &o
 // packed arena) accounts for it; dev_alloc takes at least 16 bytes.
 size_t granule(size_t b) { return b == 0 ? 0 : (std::max<size_t>(b, 16) + 255) / 256 * 256; }
 
+// Step index t and, for the time-dependent viscosity law, its factor at t (one
+// value for all cells, formed here in FP64 instead of by every thread).
+template <class Real>
+void set_time(const lb_ctx *c, StepArgs<Real> &a, long long t) {
+  a.t = t;
+  if (c->prm.visc_law == 2)
+    a.nu_t = Real(c->prm.nu_g * (1.0 + c->prm.a * std::exp(c->prm.alpha * double(t))));
+}
+
 template <class Real>
 void fill_args(const lb_ctx *c, StepArgs<Real> &a) {
   std::memset(&a, 0, sizeof a);
@@ -316,6 +348,9 @@ void fill_args(const lb_ctx *c, StepArgs<Real> &a) {
   a.ny = c->dom.ny;
   a.nz = c->dom.nz;
   a.N = c->N;
+  a.linear = c->linear ? 1 : 0;
+  a.by_nx = FastDiv::of(unsigned(c->dom.nx));
+  a.by_ny = FastDiv::of(unsigned(c->dom.ny));
   a.f_wall = c->f_wall;
   a.f_press = c->f_press;
   a.f_vel = c->f_vel;
@@ -342,11 +377,10 @@ void fill_args(const lb_ctx *c, StepArgs<Real> &a) {
   a.rhohat = static_cast<const Real *>(c->rhohat);
   for (int i = 0; i < 3; ++i) a.G[i] = Real(c->prm.G[i]);
   a.tau = Real(c->prm.tau);
+  a.itau = Real(1.0 / c->prm.tau);
+  a.nu0 = (a.tau - Real(0.5)) * Real(1.0 / 3.0);
   a.tau0 = Real(c->prm.tau0);
   a.tau1 = Real(c->prm.tau1);
-  a.nu_g = Real(c->prm.nu_g);
-  a.a_h = Real(c->prm.a);
-  a.alpha = Real(c->prm.alpha);
   a.beta = Real(c->prm.beta);
   a.visc_law = c->prm.visc_law;
   a.A = Real(c->prm.A);
@@ -357,7 +391,7 @@ void fill_args(const lb_ctx *c, StepArgs<Real> &a) {
     a.D = Real((c->prm.tau_D - 0.5) / 3.0);
     a.C_in = Real(c->prm.C_in);
   }
-  a.t = c->t;
+  set_time(c, a, c->t);
   a.flux = c->flux ? 1 : 0;
   a.flux_slots = c->flux_slots;
   a.state = c->state;
@@ -459,7 +493,7 @@ int step_feat(const lb_ctx *c);
 int enqueue_step(lb_ctx *c, cudaStream_t s, bool last) {
   return with_args(c, [&](void *args, auto &a) {
     using Real = std::remove_reference_t<decltype(a.G[0])>;
-    a.t = c->t + 1;
+    set_time(c, a, c->t + 1);
     a.reduce = (c->prm.check_every > 0 && a.t % c->prm.check_every == 0) ? 1 : 0;
     a.fields = last ? c->fields : nullptr;
     if (c->fs) {
@@ -529,7 +563,10 @@ int capture_pair(lb_ctx *c, cudaGraphExec_t *out, StepFn &&step) {
 }
 
 // features of the per-cell step kernel this lattice needs
-int step_feat(const lb_ctx *c) { return (c->open_faces ? FEAT_OPEN : 0) | (c->S > 1 ? FEAT_SPEC : 0); }
+int step_feat(const lb_ctx *c) {
+  return (c->open_faces ? FEAT_OPEN : 0) | (c->S > 1 ? FEAT_SPEC : 0) |
+         (c->prm.A != 0.0 ? FEAT_TENS : 0);
+}
 
 // One warp waits, with the step kernels' bounded wait, on a shared-memory
 // barrier that nothing completes; on giving up it sets the timeout bit of the
@@ -661,7 +698,7 @@ int lb_create(const lb_domain *dom, const float *porosity, const float *K6, cons
   }
   c->N = unsigned(N64);
   c->nblk = (c->N + BLOCK - 1) / BLOCK;
-  cell_shape(*dom, &c->sgrid, &c->sblock);
+  c->linear = cell_shape(*dom, ops->fp64, &c->sgrid, &c->sblock);
   c->nwarps = slot_warps(*dom);  // flux slots for every launch shape the autotuner may pick
   c->solute = prm->solute != 0;
   c->fs = prm->free_surface != 0;
@@ -843,7 +880,9 @@ int lb_create(const lb_domain *dom, const float *porosity, const float *K6, cons
   if (prm->kernel == 2 && !c->use_tma)
     return bail(fail(c, LB_EUNSUPPORTED, "row-pipelined kernel: this lattice shape or storage"));
   if (prm->kernel == 3) {
-    const unsigned bx = c->sblock.x;
+    dim3 rg, rb3;
+    row_shape(*dom, &rg, &rb3);
+    const unsigned bx = rb3.x;
     if (c->fs || !ops->pipe_config || !pipe_shape(c, bx, &c->pipe))
       return bail(fail(c, LB_EUNSUPPORTED, "row-staged kernel: this lattice or storage"));
   }
@@ -958,7 +997,7 @@ int lb_init(lb_ctx *c, const float *rho0, const float *u0, const float *C0,
   return with_args(c, [&](void *args, auto &a) {
     using Real = std::remove_reference_t<decltype(a.G[0])>;
     a.link = c->link;  // solid cells are always skipped at init
-    a.t = 0;
+    set_time(c, a, 0);
     a.fields = c->fields;
     InitArgs<Real> in{};
     in.rho0 = d_rho;
@@ -1023,6 +1062,12 @@ int lb_set_graphs(lb_ctx *c, int32_t enable) {
 
 namespace {
 
+// A lattice's blocks of STEP_BLOCK threads in a batch work list.
+dim3 batch_grid(const lb_ctx *c) {
+  if (!c->linear) return c->sgrid;
+  return dim3((c->N + STEP_BLOCK - 1) / STEP_BLOCK, 1, 1);
+}
+
 template <class Real>
 int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   lb_ctx *c0 = ctxs[0];
@@ -1031,19 +1076,22 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   CK(c0, cudaGetDevice(&dev));
   CK(c0, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const unsigned wave = unsigned(6 * sms);  // resident blocks of the per-cell kernel
-  // a lattice whose own launch fills the GPU steps alone (its per-cell launch);
-  // the smaller ones share the persistent launches, their blocks concatenated
+  // the lattices share persistent launches, their blocks concatenated, so that
+  // only the last wave of a whole step is partly filled. Large ones too: 15
+  // lattices of 32^3 .. 128^3 (FP32) step in 0.244 ms; with those of at least 1,
+  // 2, 4 or 8 waves in launches of their own 0.302, 0.285, 0.261, 0.252 ms.
   std::vector<int> alone, shared;
-  for (int i = 0; i < n; ++i) {
-    const dim3 g = ctxs[i]->sgrid;
-    (g.x * g.y * g.z >= wave || ctxs[i]->open_faces || ctxs[i]->S > 1 ? alone : shared)
-        .push_back(i);
+  for (int i = 0; i < n; ++i)
+    (ctxs[i]->open_faces || ctxs[i]->S > 1 ? alone : shared).push_back(i);
+  if (shared.size() == 1) {  // nothing to share with
+    alone.push_back(shared[0]);
+    shared.clear();
   }
   const int ns = int(shared.size());
   std::vector<unsigned> begin(size_t(ns) + 1);
   unsigned total = 0;
   for (int j = 0; j < ns; ++j) {
-    const dim3 g = ctxs[shared[j]]->sgrid;
+    const dim3 g = batch_grid(ctxs[shared[j]]);
     begin[j] = total;
     total += g.x * g.y * g.z;
   }
@@ -1053,7 +1101,7 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   if (ns > 0) {
     std::vector<uint64_t> work(total);
     for (int j = 0; j < ns; ++j) {
-      const dim3 g = ctxs[shared[j]]->sgrid;
+      const dim3 g = batch_grid(ctxs[shared[j]]);
       unsigned b = begin[j];
       for (unsigned bz = 0; bz < g.z; ++bz)
         for (unsigned by = 0; by < g.y; ++by)
@@ -1075,7 +1123,7 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   auto one_step = [&](cudaStream_t st, bool last) -> int {
     auto step_args = [&](lb_ctx *c, StepArgs<Real> &a) {
       fill_args(c, a);
-      a.t = c->t + 1;
+      set_time(c, a, c->t + 1);
       a.reduce = (c->prm.check_every > 0 && a.t % c->prm.check_every == 0) ? 1 : 0;
       a.fields = last ? c->fields : nullptr;
     };
@@ -1092,9 +1140,9 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
         lb_ctx *c = ctxs[shared[j]];
         BatchEntry<Real> &e = tab->e[j - g0];
         step_args(c, e.a);
-        e.gx = c->sgrid.x;
-        e.gy = c->sgrid.y;
-        e.bx = c->sblock.x;
+        e.gx = batch_grid(c).x;
+        e.gy = batch_grid(c).y;
+        e.bx = c->linear ? unsigned(STEP_BLOCK) : c->sblock.x;
       }
       const unsigned blocks = begin[g1] - begin[g0];
       CK(c0, c0->ops->batch_step(c0->kmode, c0->solute, tab.get(), d_work, unsigned(g0),
@@ -1177,7 +1225,7 @@ int lb_autotune(lb_ctx *c, int32_t reps, int32_t *choice) {
   if (reps < 1) reps = 1;
   if (choice) *choice = 0;
   if (c->fs || c->prm.A != 0.0) return LB_OK;  // fixed launches (free surface, surface tension)
-  enum Kind { CELL, ROWS, STAGED };
+  enum Kind { CELL, LINEAR, ROWS, STAGED };
   struct Cand {
     Kind kind;
     unsigned bx;
@@ -1185,6 +1233,7 @@ int lb_autotune(lb_ctx *c, int32_t reps, int32_t *choice) {
   };
   std::vector<Cand> cands;
   for (unsigned bx = 32; bx <= unsigned(STEP_BLOCK); bx *= 2) cands.push_back({CELL, bx, {}});
+  if (c->dom.nx % 32 != 0 || c->linear) cands.push_back({LINEAR, unsigned(STEP_BLOCK), {}});
   if (c->tma_ok) cands.push_back({ROWS, 0, {}});
   for (unsigned bx = 32; bx <= unsigned(STEP_BLOCK); bx *= 2) {
     Cand cd{STAGED, bx, {}};
@@ -1198,14 +1247,16 @@ int lb_autotune(lb_ctx *c, int32_t reps, int32_t *choice) {
   int rc = LB_OK;
   for (size_t i = 0; i < cands.size() && rc == LB_OK; ++i) {
     const Cand &cd = cands[i];
-    const dim3 blk(cd.bx, STEP_BLOCK / std::max(cd.bx, 1u), 1);
-    const dim3 grd(cd.bx ? (c->dom.nx + blk.x - 1) / blk.x : 1,
-                   cd.bx ? (c->dom.ny + blk.y - 1) / blk.y : 1, c->dom.nz);
+    dim3 blk(cd.bx, STEP_BLOCK / std::max(cd.bx, 1u), 1);
+    dim3 grd(cd.bx ? (c->dom.nx + blk.x - 1) / blk.x : 1,
+             cd.bx ? (c->dom.ny + blk.y - 1) / blk.y : 1, c->dom.nz);
+    if (cd.kind == LINEAR) linear_shape(c->dom, c->ops->fp64, &grd, &blk);
     // side-effect free timing launches: input buffer -> output buffer without
     // swapping, no flux accumulation, no checks, no field export
     auto launch = [&]() -> int {
       return with_args(c, [&](void *args, auto &a) {
-        a.t = c->t + 1;
+        set_time(c, a, c->t + 1);
+        a.linear = cd.kind == LINEAR ? 1 : 0;
         a.flux = 0;
         a.reduce = 0;
         a.fields = nullptr;
@@ -1246,6 +1297,8 @@ int lb_autotune(lb_ctx *c, int32_t reps, int32_t *choice) {
   drop_graphs(c);  // the captured launches used the previous shape
   c->use_tma = w.kind == ROWS;
   c->pipe = w.kind == STAGED ? w.ps : lb_ctx::PipeShape{};
+  if (w.kind == LINEAR || w.kind == CELL) c->linear = w.kind == LINEAR;
+  if (w.kind == LINEAR) linear_shape(c->dom, c->ops->fp64, &c->sgrid, &c->sblock);
   if (w.kind == CELL) {
     c->sblock = dim3(w.bx, STEP_BLOCK / w.bx, 1);
     c->sgrid = dim3((c->dom.nx + w.bx - 1) / w.bx, (c->dom.ny + c->sblock.y - 1) / c->sblock.y,

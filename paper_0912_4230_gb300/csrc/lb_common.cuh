@@ -225,10 +225,30 @@ struct DevState {
   unsigned pad;
 };
 
+// Division of n < 2^31 by a fixed d >= 1 as a high product and a shift
+// (Granlund and Montgomery): mul = ceil(2^(31+l) / d) with 2^(l-1) < d <= 2^l;
+// d = 1 is marked by mul = 0.
+struct FastDiv {
+  unsigned mul, shift;
+  static FastDiv of(unsigned d) {
+    if (d <= 1) return {0u, 0u};
+    unsigned l = 0;
+    while ((1ull << l) < d) ++l;
+    return {unsigned(((1ull << (31 + l)) + d - 1) / d), l - 1};
+  }
+  __host__ __device__ unsigned div(unsigned n) const {
+    return mul ? unsigned((uint64_t(n) * mul) >> 32) >> shift : n;
+  }
+};
+
 template <class Real>
 struct StepArgs {
   int nx, ny, nz;
   unsigned N;
+  // per-cell launches: 1 = a thread per cell in the order of n (block b holds
+  // cells b STEP_BLOCK ..), 0 = rows of blockDim.x threads (step_kernel)
+  int linear;
+  FastDiv by_nx, by_ny;
   // face-kind masks over the 6 faces (bit layout of faces_crossed)
   unsigned f_wall;                   // fluid wall faces
   unsigned f_press, f_vel;           // fluid pressure / velocity faces (others periodic)
@@ -252,7 +272,9 @@ struct StepArgs {
   const Real *face;      // per face (2 axis + side): [0, 6) 3 x pressure, [6, 24) velocity xyz,
                          // [24, 30) 3 x pressure minus its rounding to Real
   Real G[3];
-  Real tau, tau0, tau1, nu_g, a_h, alpha, beta;
+  Real tau, tau0, tau1, beta;
+  Real itau, nu0;       // 1/tau and nu of the constant law
+  Real nu_t;            // law 2: nu_g (1 + a e^{alpha t}) at this step's t
   int visc_law;
   Real A, wall_rho;
   Real forch;           // multiplier of the Ergun coefficient (KM_FORCH)

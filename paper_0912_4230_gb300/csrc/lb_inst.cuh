@@ -53,7 +53,10 @@ struct Instance {
       switch (feat) {
         case 0: return step_t<K, L, 0>(a, grid, block, s);
         case FEAT_OPEN: return step_t<K, L, FEAT_OPEN>(a, grid, block, s);
+        case FEAT_TENS: return step_t<K, L, FEAT_TENS>(a, grid, block, s);
         case FEAT_SPEC: return L ? step_t<K, L, FEAT_SPEC>(a, grid, block, s) : cudaErrorInvalidValue;
+        case FEAT_SPEC | FEAT_TENS:  // open faces and surface tension exclude each other
+          return L ? step_t<K, L, FEAT_SPEC | FEAT_TENS>(a, grid, block, s) : cudaErrorInvalidValue;
         default:
           return L ? step_t<K, L, FEAT_OPEN | FEAT_SPEC>(a, grid, block, s) : cudaErrorInvalidValue;
       }

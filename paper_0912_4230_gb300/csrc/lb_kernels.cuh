@@ -20,9 +20,11 @@ namespace lbgb {
 
 // Compile-time features of the per-cell step kernel, each a separate
 // instantiation so that lattices without them keep the plain code:
-// pressure / velocity faces of the fluid lattice, and further solute species
-// (1 .. S-1, advanced by the same thread after the fluid and species 0).
-enum : int { FEAT_OPEN = 1, FEAT_SPEC = 2 };
+// pressure / velocity faces of the fluid lattice, further solute species
+// (1 .. S-1, advanced by the same thread after the fluid and species 0), and
+// surface tension (A != 0; its terms would otherwise cost a predicated
+// instruction or two per direction in every lattice).
+enum : int { FEAT_OPEN = 1, FEAT_SPEC = 2, FEAT_TENS = 4 };
 
 // the first direction of each pair of opposite directions (its partner is opp)
 __host__ __device__ constexpr int pair_first(int k) {
@@ -42,6 +44,73 @@ template <int N>
 struct Unroll<N, N> {
   template <class F>
   __device__ __forceinline__ static void run(F &&) {}
+};
+
+// Additions and products that the compiler does not contract into an fma, so
+// that every kernel forms the same values whatever surrounds them.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// Values of the fluid and the solute lattice side by side. The collision
+// does the same operations on f_q and h_q, so with FP32 collision the two
+// share one packed instruction (fma / add / sub .rn.f32x2 of sm_100+, each
+// half rounded as the scalar instruction): the step kernels are bound by
+// instruction issue and load latency, and this halves the issue slots of the
+// moments and the collision. FP64 has no packed form; without the solute
+// lattice only f is there.
+template <class Real, bool SOLUTE>
+struct Lat {
+  Real f, h;
+  __device__ __forceinline__ static Lat mk(Real f, Real h) { return Lat{f, SOLUTE ? h : Real(0)}; }
+  __device__ __forceinline__ Real lo() const { return f; }
+  __device__ __forceinline__ Real hi() const { return SOLUTE ? h : Real(0); }
+  __device__ __forceinline__ static Lat fma(Lat a, Lat b, Lat c) {
+    return mk(::fma(a.f, b.f, c.f), SOLUTE ? ::fma(a.h, b.h, c.h) : Real(0));
+  }
+  __device__ __forceinline__ static Lat add(Lat a, Lat b) {
+    return mk(add_rn(a.f, b.f), SOLUTE ? add_rn(a.h, b.h) : Real(0));
+  }
+  __device__ __forceinline__ static Lat sub(Lat a, Lat b) {
+    return mk(sub_rn(a.f, b.f), SOLUTE ? sub_rn(a.h, b.h) : Real(0));
+  }
+};
+template <>
+struct Lat<float, true> {
+  unsigned long long v;
+  __device__ __forceinline__ static Lat mk(float f, float h) {
+    Lat r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(f), "f"(h));
+    return r;
+  }
+  __device__ __forceinline__ float lo() const {
+    float a;
+    asm("{ .reg .f32 t; mov.b64 {%0, t}, %1; }" : "=f"(a) : "l"(v));
+    return a;
+  }
+  __device__ __forceinline__ float hi() const {
+    float b;
+    asm("{ .reg .f32 t; mov.b64 {t, %0}, %1; }" : "=f"(b) : "l"(v));
+    return b;
+  }
+  __device__ __forceinline__ static Lat fma(Lat a, Lat b, Lat c) {
+    Lat r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+  }
+  __device__ __forceinline__ static Lat add(Lat a, Lat b) {
+    Lat r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+  }
+  __device__ __forceinline__ static Lat sub(Lat a, Lat b) {
+    Lat r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+  }
 };
 
 template <class Real>
@@ -168,8 +237,8 @@ __device__ __forceinline__ Real tau_of(const StepArgs<Real> &a, Real C) {
     return a.tau0 + (a.tau1 - a.tau0) * cl;
   }
   if (a.visc_law == 2) {
-    const Real nu = a.nu_g * (Real(1) + a.a_h * exp(a.alpha * Real(a.t))) *
-                    exp(a.beta * (Real(1) - C));
+    // nu_t = nu_g (1 + a e^{alpha t}), the same for every cell
+    const Real nu = a.nu_t * exp(a.beta * (Real(1) - C));
     return Real(3) * nu + Real(0.5);
   }
   return a.tau;
@@ -179,6 +248,24 @@ __device__ __forceinline__ Real tau_of(const StepArgs<Real> &a, Real C) {
 // instruction sequence in FP32, exact division in FP64.
 __device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+
+// Reciprocal of a quantity of order one (density, porosity, relaxation time,
+// 1 + drag): the hardware's approximation and Newton-Raphson steps, r <- r + r
+// (1 - x r), one in FP32 (from 1 ulp) and two in FP64 (from 2^-20), without
+// the range checks and slow path of the exact reciprocal. FP64 arithmetic is
+// 1/64 of FP32's rate on this chip, so a reciprocal of 5 instead of ~10
+// instructions counts there.
+__device__ __forceinline__ float rcp1(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ double rcp1(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
 
 // Inside an iteration that corrects its own errors (the Forchheimer Newton
 // solve) FP32 takes the hardware's single-instruction approximations (at
@@ -210,7 +297,7 @@ __device__ __forceinline__ double sqrt_iter(double x) { return sqrt(x); }
 // closed form of an isotropic medium with the r^2-weighted a and b; three
 // iterations in FP32 and four in FP64 reach the root to rounding for K from
 // 1e-4 to 1e2, 100:1 anisotropy and cF up to 20.
-template <int KMODE, class Real, class KV>
+template <int KMODE, bool EXACT = false, class Real, class KV>
 __device__ __forceinline__ void velocity_solve_kv(KV kv, Real eps, Real nu, const Real (&V)[3],
                                                   const Real (&G)[3], Real cF, Real (&Vp)[3],
                                                   Real (&Fe)[3]) {
@@ -261,9 +348,22 @@ __device__ __forceinline__ void velocity_solve_kv(KV kv, Real eps, Real nu, cons
   } else if (KMODE == KM_DIAG) {
     const Real kx = kv(0), ky = kv(1), kz = kv(2);
     const Real hs = Real(0.5) * en;
-    Vp[0] = r0 * rcp(Real(1) + hs * kx);
-    Vp[1] = r1 * rcp(Real(1) + hs * ky);
-    Vp[2] = r2 * rcp(Real(1) + hs * kz);
+    const Real lx = Real(1) + hs * kx, ly = Real(1) + hs * ky, lz = Real(1) + hs * kz;
+    if constexpr (EXACT) {
+      Vp[0] = r0 * rcp(lx);
+      Vp[1] = r1 * rcp(ly);
+      Vp[2] = r2 * rcp(lz);
+    } else if constexpr (sizeof(Real) == 8) {
+      // one FP64 reciprocal for the three (k <= 1e45, so the product is finite)
+      const Real lxy = lx * ly, i3 = rcp1(lxy * lz), iz = i3 * lz;
+      Vp[0] = r0 * (iz * ly);
+      Vp[1] = r1 * (iz * lx);
+      Vp[2] = r2 * (i3 * lxy);
+    } else {
+      Vp[0] = r0 * rcp1(lx);
+      Vp[1] = r1 * rcp1(ly);
+      Vp[2] = r2 * rcp1(lz);
+    }
     Fe[0] = -en * kx * Vp[0] + eps * G[0];
     Fe[1] = -en * ky * Vp[1] + eps * G[1];
     Fe[2] = -en * kz * Vp[2] + eps * G[2];
@@ -276,7 +376,8 @@ __device__ __forceinline__ void velocity_solve_kv(KV kv, Real eps, Real nu, cons
     // adjugate of the symmetric matrix Lambda
     const Real c00 = l11 * l22 - l12 * l12, c01 = l02 * l12 - l01 * l22, c02 = l01 * l12 - l02 * l11;
     const Real c11 = l00 * l22 - l02 * l02, c12 = l01 * l02 - l00 * l12, c22 = l00 * l11 - l01 * l01;
-    const Real idet = Real(1) / (l00 * c00 + l01 * c01 + l02 * c02);
+    const Real det = l00 * c00 + l01 * c01 + l02 * c02;
+    const Real idet = EXACT ? Real(1) / det : rcp1(det);
     Vp[0] = (c00 * r0 + c01 * r1 + c02 * r2) * idet;
     Vp[1] = (c01 * r0 + c11 * r1 + c12 * r2) * idet;
     Vp[2] = (c02 * r0 + c12 * r1 + c22 * r2) * idet;
@@ -320,8 +421,9 @@ __device__ __forceinline__ void colour_gradient(const Real *__restrict__ rh, uns
 // direction they are w_q b_q with
 //   b_q = K + cu (B3 + B45 cu + P9 cF) + P3 cF [+ S2 (c_q.F)^2],
 // cu = c_q.V', cF = c_q.F_e (K0 in place of K for the rest direction), taken
-// as scale (b_q - shift): scale 1 and shift 0 give the deviation above;
-// 16-bit storage folds its scale and the cell's reference into them.
+// taken as scale (b_q - shift). Used by the initialisation (feq_dev), the
+// free surface and 16-bit storage; the FP32/FP64 porous step folds further
+// (collide_tail).
 template <class Real>
 struct FluidCollide {
   Real drho, rho, ie, uu, uF, itau, omt, pre, stc, Fn, iFn;
@@ -353,22 +455,17 @@ struct FluidCollide {
     }
     return b;
   }
-  // b_q and b_qbar of a pair of opposite directions: the even part K +
-  // cu (B45 cu + P9 cF) [+ S2 (c.F)^2] is shared, the odd part B3 cu + P3 cF
-  // changes sign (cu = c_q.V', cF = c_q.F_e). Every step is an explicit
-  // fma, product or sum, so every kernel rounds it alike.
+  // Even and odd part of b_q for a pair of opposite directions: K + cu (B45 cu
+  // + P9 cF) [+ S2 (c.F)^2] and B3 cu + P3 cF (cu = c_q.V', cF = c_q.F_e)
   template <int q>
-  __device__ __forceinline__ void br_pair(Real &bq, Real &bo) const {
-    const Real cu = Real(cx(q)) * Vp[0] + Real(cy(q)) * Vp[1] + Real(cz(q)) * Vp[2];
+  __device__ __forceinline__ void even_odd(Real cu, Real &ev, Real &od) const {
     const Real cF = Real(cx(q)) * Fe[0] + Real(cy(q)) * Fe[1] + Real(cz(q)) * Fe[2];
-    Real ev = fma(cu, fma(B45, cu, P9 * cF), K);
+    ev = fma(cu, fma(B45, cu, P9 * cF), K);
     if (st) {
       const Real cs = Real(cx(q)) * F[0] + Real(cy(q)) * F[1] + Real(cz(q)) * F[2];
       ev = fma(S2 * cs, cs, ev);
     }
-    const Real od = fma(B3, cu, P3 * cF);
-    bq = ev + od;
-    bo = ev - od;
+    od = fma(B3, cu, P3 * cF);
   }
   // f^eq_q - w_q (with the surface-tension part), for initialisation
   template <int q>
@@ -418,6 +515,25 @@ __device__ __forceinline__ float st_threshold<float>() { return 1e-20f; }
 template <>
 __device__ __forceinline__ double st_threshold<double>() { return 1e-30; }
 
+// Flags a warp whose mass or solute sum is not finite. The sums themselves
+// (10 shuffles and additions of each) are only formed when some lane's value
+// is large or not a number; below 1e36 the sum of 32 is finite.
+template <class Real>
+__device__ __forceinline__ void finite_check(DevState *state, Real drho, Real sC) {
+  // (FP64: by the high words, on the integer pipe; the FP64 one is the
+  // bottleneck of those kernels)
+  bool fine;
+  if constexpr (sizeof(Real) == 8)
+    fine = (__double2hiint(drho) & 0x7fffffff) < 0x47700000 &&
+           (__double2hiint(sC) & 0x7fffffff) < 0x47700000;
+  else
+    fine = fabs(drho) < Real(1e36) && fabs(sC) < Real(1e36);
+  if (__any_sync(0xffffffffu, !fine)) {
+    const Real m = warp_sum(drho), c = warp_sum(sC);
+    if ((threadIdx.x & 31u) == 0 && !(isfinite(m) && isfinite(c))) atomicOr(&state->status, 1u);
+  }
+}
+
 // Per-warp FP64 reductions of a step. Solute fluxes through inlet/outlet
 // faces are accumulated into one FP64 slot pair per warp of the launch
 // (each warp owns its slots across steps, so the running sums are
@@ -435,10 +551,7 @@ __device__ __forceinline__ void warp_reductions(const StepArgs<Real> &a, unsigne
       a.flux_slots[2 * size_t(warp_gid) + 1] += double(so);
     }
   }
-  if (a.reduce) {
-    const Real m = warp_sum(drho), c = warp_sum(sC);
-    if (lane == 0 && !(isfinite(m) && isfinite(c))) atomicOr(&a.state->status, 1u);
-  }
+  if (a.reduce) finite_check(a.state, drho, sC);
 }
 
 // Stream of a cell on a pressure or velocity face of the fluid lattice into
@@ -516,46 +629,163 @@ __device__ __noinline__ Pops<typename S::Real> gather_open_faces(
   return d;
 }
 
-// Fluid moments of the arriving populations: drho += sum_q (f_q - w_q) and
-// V = j / rho with j = sum_q c_q (f_q - w_q), rho = 1 + drho. With E the
-// values are e_q = (f_q - w_q)/w_q (16-bit storage) and carry their weights
-// here.
-template <bool E = false, class Real, class FV>
-__device__ __forceinline__ void fluid_moments(FV fv, Real &drho, Real (&V)[3]) {
-  Real j0 = Real(0), j1 = Real(0), j2 = Real(0);
-  Unroll<0, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const Real v = fv(qc);
-    if constexpr (E) {
-      constexpr Real w = wq<Real>(q);
-      drho = fma(w, v, drho);
-      if (cx(q)) j0 = fma(Real(cx(q)) * w, v, j0);
-      if (cy(q)) j1 = fma(Real(cy(q)) * w, v, j1);
-      if (cz(q)) j2 = fma(Real(cz(q)) * w, v, j2);
-    } else {
-      drho += v;
-      if (cx(q)) j0 += Real(cx(q)) * v;
-      if (cy(q)) j1 += Real(cy(q)) * v;
-      if (cz(q)) j2 += Real(cz(q)) * v;
-    }
-  });
-  const Real irho = rcp(Real(1) + drho);
-  V[0] = j0 * irho;
-  V[1] = j1 * irho;
-  V[2] = j2 * irho;
+// Reciprocals up to the velocity: with 16-bit storage the correctly rounded
+// one. In a tight medium the drag balances the body force, F_e is the small
+// difference of the two, and its FP32 rounding is as large as the last bit of
+// a 16-bit remainder.
+template <class S>
+__device__ __forceinline__ typename S::Real rcp_as(typename S::Real x) {
+  if constexpr (S::kShift)
+    return rcp(x);
+  else
+    return rcp1(x);
 }
+
+// Moments of the arriving populations: drho = sum_q (f_q - w_q), V = j / rho
+// with j = sum_q c_q (f_q - w_q), rho = 1 + drho, and the solute total sC =
+// sum_q h_q. FP32 / FP64 storage takes opposite directions together: their
+// sums feed drho and sC, their differences j, and both are kept in sd for
+// the collision (sd[k] the sum and sd[9 + k] the difference of pair k, sd[18]
+// the rest direction). 16-bit storage gives the values per unit weight, e_q =
+// (f_q - w_q)/w_q and h_q/w_q, and sums them with their weights in the order
+// of q (sd unused): two roundings that differ in one bit end in different
+// 16-bit remainders.
+template <class S, bool SOLUTE, class FV, class HV>
+__device__ __forceinline__ void moments(FV fv, HV hv, typename S::Real &drho,
+                                        typename S::Real &sC, typename S::Real (&V)[3],
+                                        Lat<typename S::Real, SOLUTE> (&sd)[Q]) {
+  using Real = typename S::Real;
+  using L = Lat<Real, SOLUTE>;
+  auto in = [&](auto qc) { return L::mk(fv(qc), hv(qc)); };
+  L tot = L::mk(Real(0), Real(0)), axis = tot;
+  Real jd[3] = {Real(0), Real(0), Real(0)}, ja[3] = {Real(0), Real(0), Real(0)};
+  if constexpr (S::kShift) {
+    Unroll<0, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      constexpr Real w = wq<Real>(q);
+      tot = L::fma(L::mk(w, w), in(qc), tot);
+      if (cx(q)) jd[0] = fma(Real(cx(q)) * w, fv(qc), jd[0]);
+      if (cy(q)) jd[1] = fma(Real(cy(q)) * w, fv(qc), jd[1]);
+      if (cz(q)) jd[2] = fma(Real(cz(q)) * w, fv(qc), jd[2]);
+    });
+  } else {
+    Unroll<0, 9>::run([&](auto kc) {
+      constexpr int k = decltype(kc)::value, q = pair_first(k), o = opp(q);
+      constexpr bool ax = inv_wq(q) == 18;
+      const L p = in(std::integral_constant<int, q>{}), m = in(std::integral_constant<int, o>{});
+      sd[k] = L::add(p, m);
+      sd[9 + k] = L::sub(p, m);
+      if constexpr (ax)
+        axis = q == 5 ? sd[k] : L::add(axis, sd[k]);
+      else
+        tot = q == 1 ? sd[k] : L::add(tot, sd[k]);
+      const Real dif = sd[9 + k].lo();
+      auto take = [&](int i, int c, bool start) {
+        if (ax)
+          ja[i] = dif;
+        else
+          jd[i] = start ? dif : (c > 0 ? add_rn(jd[i], dif) : sub_rn(jd[i], dif));
+      };
+      if (cx(q)) take(0, cx(q), q == 1);
+      if (cy(q)) take(1, cy(q), q == 1);
+      if (cz(q)) take(2, cz(q), q == 7);
+    });
+    sd[18] = in(std::integral_constant<int, 0>{});
+    tot = L::add(L::add(tot, axis), sd[18]);
+  }
+  drho = tot.lo();
+  sC = tot.hi();
+  const Real ir = rcp_as<S>(add_rn(Real(1), drho));
+#pragma unroll
+  for (int i = 0; i < 3; ++i) V[i] = mul_rn(S::kShift ? jd[i] : add_rn(ja[i], jd[i]), ir);
+}
+
+template <class Real>
+struct Lat1 {
+  __device__ __forceinline__ static Real add(Real a, Real b) { return add_rn(a, b); }
+  __device__ __forceinline__ static Real sub(Real a, Real b) { return sub_rn(a, b); }
+};
+
+// sum_i c_qi a_i for the axes of direction q, by additions
+template <int q, class A, class F>
+__device__ __forceinline__ A along(const A (&a)[3], F) {
+  constexpr int c[3] = {cx(q), cy(q), cz(q)};
+  constexpr int i = c[0] ? 0 : (c[1] ? 1 : 2);                      // first axis
+  constexpr int k = (c[0] && c[1]) ? 1 : ((c[2] && i != 2) ? 2 : -1);  // second, or none
+  if constexpr (k < 0) {
+    static_assert(c[i] == 1, "pair_first lists the positive axis directions");
+    return a[i];
+  } else if constexpr (c[i] == 1 && c[k] == 1) {
+    return F::add(a[i], a[k]);
+  } else if constexpr (c[i] == 1) {
+    return F::sub(a[i], a[k]);
+  } else {
+    static_assert(c[k] == 1, "one of a pair's directions has a positive component");
+    return F::sub(a[k], a[i]);
+  }
+}
+
+// x / fl(1/3) in FP32, correctly rounded: the quotient by multiplication with
+// 3, the rounded reciprocal of fl(1/3), and one step of Markstein's correction.
+__device__ __forceinline__ float div_third(float x) {
+  const float q = x * 3.0f;
+  return fmaf(fmaf(-wq<float>(0), q, x), 3.0f, q);
+}
+
+// Solute collision of one lattice (Eq. equild, BGK) for itd = 1/tau_D, per
+// cell. Weighted rows: with e = itd sC / 36 and H = 3 e V*, h~_q = (1 - itd) h_q
+// + (e + c_q.H) for the diagonals, twice the bracket for the axes, and the
+// rest direction takes itd sC - 24 e, so the equilibrium adds no solute beyond
+// one rounding.
+template <class Real>
+struct SoluteRows {
+  Real e, H[3], rest;
+  __device__ __forceinline__ void fold(Real sC, Real itd, Real v0, Real v1, Real v2) {
+    e = mul_rn(mul_rn(itd, wq<Real>(1)), sC);
+    const Real e3 = mul_rn(Real(3), e);
+    H[0] = mul_rn(e3, v0);
+    H[1] = mul_rn(e3, v1);
+    H[2] = mul_rn(e3, v2);
+    rest = fma(Real(-24), e, mul_rn(itd, sC));
+  }
+};
 
 // The per-cell arithmetic after streaming: concentration and viscosity,
 // colour gradient, V' and the Darcy force, fluid and solute collision,
-// stores and exported fields. fv(q) and hv(q) give the arriving f_q - w_q and
-// h_q (16-bit storage: (f_q - w_q)/w_q and h_q/w_q), kv(r) the rows of K^-1;
-// drho, rho, V are the fluid moments, sC the solute total of the arriving h.
+// stores and exported fields. drho, V are the fluid moments, sC the solute
+// total of the arriving h, sd their sums and differences (16-bit storage: fv(q)
+// and hv(q) give (f_q - w_q)/w_q and h_q/w_q), kv(r) the rows of K^-1.
+//
+// Fluid collision (Eqs. equilc1, equilc2, coeffforce1), folded per cell: f~_q -
+// w_q = (1 - 1/tau)(f_q - w_q) + w_q b_q with
+//   b_q = K + c.W + (c.V')(c.X),   P = rho (1 - 1/(2 tau)),
+//   W = 3 (rho/tau V' + P F_e),  Y = 3 (rho/(2 tau) V' + P F_e),  X = 3/eps Y,
+//   K = (rho - 1)/tau - V'.Y / eps
+// (surface tension: + A eps ((c.F)^2/|F| - |F|), + A eps |F| at rest). Opposite
+// directions are formed from the sum s and the difference d of their old
+// values as E + O and E - O, E = (1 - 1/tau)/2 s + w (K + (c.V')(c.X)), O = (1 -
+// 1/tau)/2 d + w c.W: for a pair of diagonals of both lattices two packed
+// additions give the dot products, one fma and two packed fmas E and O, two
+// packed additions the new values: 7 instructions where the unfolded form took
+// ~26. Where the density is away from 1 (E much larger than O: a wood sample
+// under pressure) the rounding of E drops out of the momentum: after 60 steps
+// at 256x192x64 FP32 u is 4.1e-6 from the 64-bit result, 1.0e-5 before. Without
+// the solute the flow is driven by a force at density 1 (O the larger part),
+// and the new values are (1 - 1/tau)(f_q - w_q) + w b_q, which keeps the two
+// roundings of opposite directions independent. The weights 1/36
+// (diagonal), 2/36 (axis) and 12/36 (rest) are folded into the coefficients.
+// Every operation is an explicit fma, product or sum, so all kernels that
+// inline this round alike.
+//
+// 16-bit storage keeps the order of operations of FluidCollide (its results
+// are compared bit by bit), both lattices in packed instructions.
 // VOUT: the cell's bare V and V' are returned in vout[0..2], vout[3..5]
 // (for the further solute species of the same thread).
-template <class S, int KMODE, bool SOLUTE, bool VOUT = false, class FV, class HV, class KV>
+template <class S, int KMODE, bool SOLUTE, bool TENS, bool VOUT = false, class FV, class HV, class KV>
 __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a, unsigned n,
                                              const CellGeo &g, FV fv, HV hv, KV kv,
-                                             typename S::Real drho, typename S::Real rho,
+                                             const Lat<typename S::Real, SOLUTE> (&sd)[Q],
+                                             typename S::Real drho,
                                              const typename S::Real (&V)[3], typename S::Real ie,
                                              typename S::Real eps, typename S::Real sC,
                                              typename S::Real gx, typename S::Real gy,
@@ -563,360 +793,201 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
                                              typename S::Real *vout = nullptr) {
   using Real = typename S::Real;
   using T = typename S::T;
+  using L = Lat<Real, SOLUTE>;
+  using D = Lat<Real, true>;
   const unsigned N = a.N;
-  T *__restrict__ fo = static_cast<T *>(a.f_out) + n;
+  const Real rho = Real(1) + drho;
   const Real C = sC * ie;
   const Real tau = tau_of(a, C);
-  const Real nu = (tau - Real(0.5)) * Real(1.0 / 3.0);
-
+  const Real nu = a.visc_law == 0 ? a.nu0 : (tau - Real(0.5)) * Real(1.0 / 3.0);
   FluidCollide<Real> fc;
-  fc.F[0] = fc.F[1] = fc.F[2] = Real(0);
-  if (a.A != Real(0)) colour_gradient(a.rhohat, n, g, a.f_wall, a.wall_rho, fc.F);
-  velocity_solve_kv<KMODE>(kv, eps, nu, V, a.G, a.forch, fc.Vp, fc.Fe);
-  fc.drho = drho;
-  fc.rho = rho;
-  fc.ie = ie;
-  fc.uu = fc.Vp[0] * fc.Vp[0] + fc.Vp[1] * fc.Vp[1] + fc.Vp[2] * fc.Vp[2];
-  fc.uF = fc.Vp[0] * fc.Fe[0] + fc.Vp[1] * fc.Fe[1] + fc.Vp[2] * fc.Fe[2];
-  fc.itau = rcp(tau);
-  fc.omt = Real(1) - fc.itau;
-  fc.pre = rho * (Real(1) - Real(0.5) * fc.itau);
-  fc.st = false;
-  fc.Fn = fc.stc = fc.iFn = Real(0);
-  if (a.A != Real(0)) {
-    fc.Fn = sqrt(fc.F[0] * fc.F[0] + fc.F[1] * fc.F[1] + fc.F[2] * fc.F[2]);
-    fc.st = fc.Fn > st_threshold<Real>();
-    fc.stc = fc.st ? a.A * eps * tau : Real(0);
-    fc.iFn = fc.st ? Real(1) / fc.Fn : Real(0);
+  Real(&Vp)[3] = fc.Vp, (&Fe)[3] = fc.Fe, (&F)[3] = fc.F;
+  velocity_solve_kv<KMODE, S::kShift>(kv, eps, nu, V, a.G, a.forch, Vp, Fe);
+  Real Fn = Real(0);
+  bool st = false;
+  F[0] = F[1] = F[2] = Real(0);
+  if constexpr (TENS) {
+    colour_gradient(a.rhohat, n, g, a.f_wall, a.wall_rho, F);
+    Fn = sqrt(F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
+    st = Fn > st_threshold<Real>();
   }
-  if constexpr (S::kShift && SOLUTE) {
-    // paired layout: both lattices per unit weight in one loop, one 32-bit
-    // pair store per direction. The references are drho and sC rounded to
-    // FP16; the remainders are formed against the rounded values.
-    // f: (f~_q - w_q)/w_q = omt e_q + b_q, stored scale ((f~_q - w_q)/w_q - Rf).
-    // h: h~_q/w_q = (1 - 1/tau_D) h_q/w_q + h^eq_q/(w_q tau_D) with
-    // h^eq_q/w_q = sC (1 + 3 c_q.v), stored scale (h~_q/w_q - Rh); the rest
-    // direction takes sC - sum_{q>0} h^eq_q, divided by its weight with a
-    // correctly rounded division, so the weights' rounding adds no solute.
-    // Opposite directions are formed together: they share c.V', c.F_e and
-    // c.v, and their h^eq sum to 2 w sC.
-    const __half2 r2 = __floats2half2_rn(drho, sC);
-    const float2 R = __half22float2(r2);
-    using T2 = typename S::T2;
-    T2 *__restrict__ po = static_cast<T2 *>(a.f_out) + n;
+  const Real itd = a.inv_tau_D, vs[3] = {Vp[0] + gx, Vp[1] + gy, Vp[2] + gz};
+  T *__restrict__ fo = static_cast<T *>(a.f_out) + n;
+  if constexpr (S::kShift) {
+    fc.drho = drho;
+    fc.rho = rho;
+    fc.ie = ie;
+    fc.uu = Vp[0] * Vp[0] + Vp[1] * Vp[1] + Vp[2] * Vp[2];
+    fc.uF = Vp[0] * Fe[0] + Vp[1] * Fe[1] + Vp[2] * Fe[2];
+    fc.itau = rcp(tau);
+    fc.omt = Real(1) - fc.itau;
+    fc.pre = rho * (Real(1) - Real(0.5) * fc.itau);
+    fc.st = st;
+    fc.Fn = Fn;
+    fc.stc = st ? a.A * eps * tau : Real(0);
+    fc.iFn = st ? Real(1) / Fn : Real(0);
     const Real sc = Real(S::kScale);
-    fc.fold(sc, R.x);
-    const Real so = sc * fc.omt;
-    const Real vs0 = fc.Vp[0] + gx, vs1 = fc.Vp[1] + gy, vs2 = fc.Vp[2] + gz;
-    const Real itd = a.inv_tau_D;
-    const Real sod = sc * (Real(1) - itd), h0 = sc * (itd * sC - R.y),
-               h3 = Real(3) * sc * itd * sC;
-    Real hsum = Real(0);
+    if constexpr (SOLUTE) {
+      // paired layout: the references are drho and sC rounded to FP16, the
+      // remainders are formed against the rounded values.
+      // f: (f~_q - w_q)/w_q = omt e_q + b_q, stored scale ((f~_q - w_q)/w_q - Rf).
+      // h: h~_q/w_q = (1 - 1/tau_D) h_q/w_q + h^eq_q/(w_q tau_D) with
+      // h^eq_q/w_q = sC (1 + 3 c_q.v), stored scale (h~_q/w_q - Rh); the rest
+      // direction takes sC - sum_{q>0} h^eq_q, divided by its weight, so the
+      // weights' rounding adds no solute.
+      using T2 = typename S::T2;
+      const __half2 r2 = __floats2half2_rn(drho, sC);
+      const float2 R = __half22float2(r2);
+      T2 *__restrict__ po = static_cast<T2 *>(a.f_out) + n;
+      fc.fold(sc, R.x);
+      const Real so = sc * fc.omt, sod = sc * (Real(1) - itd), h0 = sc * (itd * sC - R.y),
+                 h3 = Real(3) * sc * itd * sC;
+      const L om = L::mk(so, sod), up = L::mk(Real(1), h3), down = L::mk(Real(-1), -h3);
+      const L uv[3] = {L::mk(Vp[0], vs[0]), L::mk(Vp[1], vs[1]), L::mk(Vp[2], vs[2])};
+      Real hsum = Real(0);
+      Unroll<0, 9>::run([&](auto kc) {
+        constexpr int q = pair_first(decltype(kc)::value), o = opp(q);
+        const auto qq = std::integral_constant<int, q>{};
+        const auto oo = std::integral_constant<int, o>{};
+        const L c = along<q>(uv, L{});
+        hsum = fma(Real(2) * wq<Real>(q), sC, hsum);
+        Real ev, od;
+        fc.template even_odd<q>(c.lo(), ev, od);
+        const L e = L::mk(ev, h0), odd = L::mk(od, c.hi());
+        const L vq = L::fma(om, L::mk(fv(qq), hv(qq)), L::fma(up, odd, e));
+        const L vo = L::fma(om, L::mk(fv(oo), hv(oo)), L::fma(down, odd, e));
+        S::st2(po + int(q * N), vq.lo(), vq.hi());
+        S::st2(po + int(o * N), vo.lo(), vo.hi());
+      });
+      const Real he0 = div_third(sC - hsum);
+      const auto q0 = std::integral_constant<int, 0>{};
+      S::st2(po, fma(so, fv(q0), fc.template br<0>()), fma(sod, hv(q0), sc * (itd * he0 - R.y)));
+      reinterpret_cast<__half2 *>(a.rf_out)[n] = r2;
+    } else {
+      // per unit weight, (f~_q - w_q)/w_q = omt e_q + b_q; stored as the
+      // remainder scale ((f~_q - w_q)/w_q - drho)
+      fc.fold(sc, drho);
+      const Real so = sc * fc.omt;
+      Unroll<0, Q>::run([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        S::template st_raw<q>(fo + int(q * N), fma(so, fv(qc), fc.template br<q>()));
+      });
+      a.rf_out[n] = float(drho);
+    }
+  } else {
+    constexpr Real w = wq<Real>(1);
+    const Real itau = a.visc_law == 0 ? a.itau : rcp1(tau), omt = Real(1) - itau;
+    const Real it = w * itau, r3 = Real(3) * (it * rho), r15 = Real(0.5) * r3;
+    const Real p3 = Real(3) * w * (rho * fma(Real(-0.5), itau, Real(1)));
+    const Real ie3 = Real(3) * ie;
+    Real K, Wv[3], X[3], VY = Real(0);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const Real t = mul_rn(p3, Fe[i]), Y = fma(r15, Vp[i], t);
+      Wv[i] = fma(r3, Vp[i], t);
+      X[i] = mul_rn(ie3, Y);
+      VY = fma(Vp[i], Y, VY);
+    }
+    K = fma(it, drho, -mul_rn(ie, VY));
+    Real K0 = K, S2 = Real(0);
+    if (TENS && st) {
+      const Real ae = w * a.A * eps, ks = ae * Fn;
+      K0 = K + ks;
+      K -= ks;
+      S2 = ae / Fn;
+    }
+    SoluteRows<Real> so{};
+    T *__restrict__ ho = nullptr;
+    if constexpr (SOLUTE) {
+      so.fold(sC, itd, vs[0], vs[1], vs[2]);
+      ho = static_cast<T *>(a.h_out) + n;
+    }
+    const Real omd = Real(1) - itd;
+    const L om = L::mk(omt, omd), half = L::mk(Real(0.5) * omt, Real(0.5) * omd);
+    const L W2[3] = {L::mk(Wv[0], so.H[0]), L::mk(Wv[1], so.H[1]), L::mk(Wv[2], so.H[2])};
+    const D VX[3] = {D::mk(Vp[0], X[0]), D::mk(Vp[1], X[1]), D::mk(Vp[2], X[2])};
+    auto store = [&](auto qc, L v) {
+      constexpr int q = decltype(qc)::value;
+      S::template st_f<q>(fo + int(q * N), v.lo());
+      if constexpr (SOLUTE) S::template st_h<q>(ho + int(q * N), v.hi());
+    };
     Unroll<0, 9>::run([&](auto kc) {
-      constexpr int q = pair_first(decltype(kc)::value), o = opp(q);
+      constexpr int k = decltype(kc)::value, q = pair_first(k), o = opp(q);
+      L od = along<q>(W2, L{});
+      const D vx = along<q>(VX, D{});
+      Real ev = fma(vx.lo(), vx.hi(), K);
+      if constexpr (TENS) {
+        const Real cs = Real(cx(q)) * F[0] + Real(cy(q)) * F[1] + Real(cz(q)) * F[2];
+        ev = fma(S2 * cs, cs, ev);
+      }
+      L e = L::mk(ev, so.e);
+      if constexpr (inv_wq(q) == 18) {  // weight 2/36
+        od = L::add(od, od);
+        e = L::add(e, e);
+      }
       const auto qq = std::integral_constant<int, q>{};
       const auto oo = std::integral_constant<int, o>{};
-      const Real cv = Real(cx(q)) * vs0 + Real(cy(q)) * vs1 + Real(cz(q)) * vs2;
-      hsum = fma(Real(2) * wq<Real>(q), sC, hsum);
-      Real bq, bo;
-      fc.template br_pair<q>(bq, bo);
-      S::st2(po + int(q * N), fma(so, fv(qq), bq), fma(sod, hv(qq), fma(h3, cv, h0)));
-      S::st2(po + int(o * N), fma(so, fv(oo), bo), fma(sod, hv(oo), fma(-h3, cv, h0)));
+      if constexpr (SOLUTE) {
+        e = L::fma(half, sd[k], e);
+        od = L::fma(half, sd[9 + k], od);
+        store(qq, L::add(e, od));
+        store(oo, L::sub(e, od));
+      } else {
+        store(qq, L::fma(om, L::mk(fv(qq), Real(0)), L::add(e, od)));
+        store(oo, L::fma(om, L::mk(fv(oo), Real(0)), L::sub(e, od)));
+      }
     });
-    const Real he0 = (sC - hsum) / wq<Real>(0);
-    const auto q0 = std::integral_constant<int, 0>{};
-    S::st2(po, fma(so, fv(q0), fc.template br<0>()), fma(sod, hv(q0), sc * (itd * he0 - R.y)));
-    reinterpret_cast<__half2 *>(a.rf_out)[n] = r2;
-  } else if constexpr (S::kShift) {
-    // per unit weight, (f~_q - w_q)/w_q = omt e_q + b_q; stored as the
-    // remainder scale ((f~_q - w_q)/w_q - drho)
-    fc.fold(Real(S::kScale), drho);
-    const Real so = Real(S::kScale) * fc.omt;
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      S::template st_raw<q>(fo + int(q * N), fma(so, fv(qc), fc.template br<q>()));
-    });
-  } else {
-    fc.fold(Real(1), Real(0));
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      S::template st_f<q>(fo + int(q * N), fc.template post<q>(fv(qc)));
-    });
+    store(std::integral_constant<int, 0>{},
+          L::fma(om, sd[18], L::mk(mul_rn(Real(12), K0), so.rest)));
   }
-  if constexpr (S::kShift && !SOLUTE) a.rf_out[n] = float(drho);
-
-  if constexpr (SOLUTE && !S::kShift) {
-    T *__restrict__ ho = static_cast<T *>(a.h_out) + n;
-    const Real vs0 = fc.Vp[0] + gx, vs1 = fc.Vp[1] + gy, vs2 = fc.Vp[2] + gz;
-    const Real itd = a.inv_tau_D;
-    // h^eq of the moving directions; the rest component takes the remainder
-    // so that sum_q h^eq_q = sum_q h_q holds to rounding (the weights rounded
-    // to the collision type sum to 1 + 1.5e-8 in FP32, which would otherwise
-    // create solute at every collision)
-    Real hsum = Real(0);
-    Unroll<1, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      const Real cv = Real(cx(q)) * vs0 + Real(cy(q)) * vs1 + Real(cz(q)) * vs2;
-      const Real heq = wq<Real>(q) * sC * (Real(1) + Real(3) * cv);
-      hsum += heq;
-      const Real h = hv(qc);
-      S::template st_h<q>(ho + int(q * N), h + (heq - h) * itd);
-    });
-    {
-      const Real h = hv(std::integral_constant<int, 0>{});
-      S::template st_h<0>(ho, h + ((sC - hsum) - h) * itd);
-    }
-  }
-  if (a.fields) write_fields(a.fields, N, n, rho, fc.Vp, C, nu);
+  if (a.fields) write_fields(a.fields, N, n, rho, Vp, C, nu);
   if constexpr (VOUT) {
-    vout[0] = V[0];
-    vout[1] = V[1];
-    vout[2] = V[2];
-    vout[3] = fc.Vp[0];
-    vout[4] = fc.Vp[1];
-    vout[5] = fc.Vp[2];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      vout[i] = V[i];
+      vout[3 + i] = Vp[i];
+    }
   }
 }
 
-// The rows of a cell's K^-1 for the velocity solve. With a full tensor, with
-// the Forchheimer drag, in the kernel that also advances further solute
-// species, and with 16-bit paired storage, they are loaded with the cell's
-// other static fields, before the moments, so their latency hides behind the
-// gather (loaded inside the solve they were a second wait per cell: 256^3
-// FP32 0.955 -> 0.862 ms, FP16 0.738 -> 0.675 ms, 128^3 Forchheimer 0.136 ->
-// 0.122 ms, three species 0.230 -> 0.221 ms, 128^3 FP16 0.0985 -> 0.0914 ms);
-// the three rows of a plain diagonal tensor with FP32/FP64 storage stay in the
-// solve, where the register budget prefers them (128^3 FP32 0.1126 ms,
-// 0.1165 ms early).
-template <class Real, int KMODE, bool SPEC = false, bool PAIRED = false>
+// The rows of a cell's K^-1, loaded with its other static fields before the
+// moments, so that their latency hides behind the gather (inside the velocity
+// solve they are a second wait per cell: 256^3 FP32 with a full tensor 0.955 ->
+// 0.862 ms, and since the collision needs fewer registers also the diagonal
+// tensor, 128^3 FP32 0.1091 -> 0.1084 ms).
+template <class Real, int KMODE>
 struct KinvRows {
-  static constexpr bool kEarly =
-      KMODE == KM_SPD || KMODE == KM_FORCH || ((SPEC || PAIRED) && KMODE == KM_DIAG);
-  Real v[kEarly ? 6 : 1];
+  static constexpr int kRows = KMODE == KM_NONE ? 0 : (KMODE == KM_SPD ? 6 : 3);
+  Real v[kRows ? kRows : 1];
   __device__ __forceinline__ void load(const Real *kinv, unsigned N, unsigned n) {
-    if constexpr (kEarly)
-      for (int r = 0; r < 6; ++r) v[r] = __ldg(kinv + size_t(r) * N + n);
-  }
-  __device__ __forceinline__ Real row(const Real *kinv, unsigned N, unsigned n, int r) const {
-    if constexpr (kEarly)
-      return v[r];
-    else
-      return __ldg(kinv + size_t(r) * N + n);
+    for (int r = 0; r < kRows; ++r) v[r] = __ldg(kinv + size_t(r) * N + n);
   }
 };
 
-// update_cell for 16-bit storage with solute (the paired layout): one 32-bit
-// load brings f_q and h_q of a source cell, one more its reference pair, and
-// both lattices are gathered per unit weight, d[q] = (f_q - w_q)/w_q and
-// hh[q] = h_q/w_q (remainder + the source's reference).
-template <class S, int KMODE, int FEAT>
-__device__ __forceinline__ void update_cell_paired(const StepArgs<float> &a, unsigned x, unsigned y,
-                                                   unsigned z, unsigned n, uint32_t link,
-                                                   float &fin_acc, float &fout_acc, float &drho,
-                                                   float &sC, bool &open_face,
-                                                   float *vout = nullptr) {
-  using Real = float;
-  using T2 = typename S::T2;
-  const unsigned N = a.N;
-  const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
-  const T2 *__restrict__ pb = static_cast<const T2 *>(a.f_in) + n;
-  const float *__restrict__ rb = a.rf_in + n;  // a __half2 per cell
-  Real d[Q], hh[Q];
-  const unsigned s_open = a.s_inlet | a.s_outlet;
-  open_face = (g.onface & s_open) != 0;
-  bool f_simple = link == 0 && !(g.onface & a.f_wall);
-  if constexpr ((FEAT & FEAT_OPEN) != 0) f_simple = f_simple && !(g.onface & (a.f_press | a.f_vel));
-  const bool both = f_simple && link == 0 && !(g.onface & (a.s_wall | s_open));
-  if (both) {
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      const float2 p = S::ld2(pb + (int(q * N) + src_delta<q>(g)));
-      const float2 r = ld_ref2(rb + src_delta<q>(g));
-      d[q] = p.x + r.x;
-      hh[q] = p.y + r.y;
-    });
-  } else if (((FEAT & FEAT_OPEN) != 0) && (g.onface & (a.f_press | a.f_vel))) {
-    const Pops<Real> o = gather_open_faces<S>(a, g, n, link);
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      d[q] = o.v[q] * Real(inv_wq(q));
-    });
-  } else {
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      const bool bb = fluid_class<q>(g, link, a.f_wall) == PULL_BOUNCE;
-      d[q] = S::ld2(pb + (bb ? int(opp(q) * N) : int(q * N) + src_delta<q>(g))).x +
-             ld_ref2(rb + (bb ? 0 : src_delta<q>(g))).x;
-    });
-  }
-  const Real eps = __ldg(a.eps + n);
-  const Real gx = __ldg(a.geps + n), gy = __ldg(a.geps + N + n),
-             gz = __ldg(a.geps + 2 * size_t(N) + n);
-  KinvRows<Real, KMODE, (FEAT & FEAT_SPEC) != 0, true> kr;
-  kr.load(a.kinv, N, n);
-  Real V[3];
-  fluid_moments<true>([&](auto qc) { return d[decltype(qc)::value]; }, drho, V);
-  const Real rho = Real(1) + drho;
-  const Real ie = rcp(eps);
-  if (!both) {
-    // the solute classes, per unit weight; the fluxes carry the weights
-    const Real vi0 = V[0] + gx, vi1 = V[1] + gy, vi2 = V[2] + gz;
-    const Real own = ld_ref2(rb).y;
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      const int cls = solute_class<q>(g, link, a.s_wall, a.s_inlet, a.s_outlet);
-      Real v;
-      if (cls == PULL_CELL) {
-        v = S::ld2(pb + (int(q * N) + src_delta<q>(g))).y + ld_ref2(rb + src_delta<q>(g)).y;
-      } else if (cls == PULL_BOUNCE) {
-        v = S::ld2(pb + int(opp(q) * N)).y + own;
-      } else if (cls == PULL_INLET) {
-        // entering through an inlet face: h^eq at C_in with the cell's bare
-        // streamed velocity plus D grad(eps)/eps
-        const Real cv = Real(cx(q)) * vi0 + Real(cy(q)) * vi1 + Real(cz(q)) * vi2;
-        v = eps * a.C_in * (Real(1) + Real(3) * cv);
-        fin_acc += wq<Real>(q) * (v - (S::ld2(pb + int(opp(q) * N)).y + own));
-      } else {
-        // outlet: the cell's own post-collision value (zero gradient)
-        v = S::ld2(pb + int(q * N)).y + own;
-        fout_acc += wq<Real>(q) * ((S::ld2(pb + int(opp(q) * N)).y + own) - v);
-      }
-      hh[q] = v;
-    });
-  }
-  Unroll<0, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    sC = fma(wq<Real>(q), hh[q], sC);
-  });
-  collide_tail<S, KMODE, true, (FEAT & FEAT_SPEC) != 0>(
-      a, n, g, [&](auto qc) { return d[decltype(qc)::value]; },
-      [&](auto qc) { return hh[decltype(qc)::value]; },
-      [&](int r) { return kr.row(a.kinv, N, n, r); }, drho, rho, V, ie, eps, sC, gx, gy, gz,
-      vout);
+// The directions whose pull leaves through one of the given faces.
+__host__ __device__ constexpr uint32_t dirs_through(unsigned faces) {
+  uint32_t m = 0;
+  for (int q = 1; q < Q; ++q)
+    if (faces_crossed(q) & faces) m |= 1u << q;
+  return m;
+}
+// The directions that bounce back in a cell, as a mask: sources that are
+// solid (link) or behind a wall face.
+__device__ __forceinline__ uint32_t bounce_mask(uint32_t link, unsigned walls_on) {
+  uint32_t m = link & 0x7ffffu;
+#pragma unroll
+  for (int f = 0; f < 6; ++f)
+    if ((walls_on >> f) & 1u) m |= dirs_through(1u << f);
+  return m;
 }
 
-// The per-cell update of one step from global memory: stream f (and h),
-// moments, viscosity, colour gradient, V' and the Darcy force, fluid and
-// solute collision, store; accumulates the cell's flux and totals.
-template <class S, int KMODE, bool SOLUTE, int FEAT = 0>
-__device__ __forceinline__ void update_cell_sep(const StepArgs<typename S::Real> &a, unsigned x,
-                                            unsigned y, unsigned z, unsigned n, uint32_t link,
-                                            typename S::Real &fin_acc,
-                                            typename S::Real &fout_acc, typename S::Real &drho,
-                                            typename S::Real &sC, bool &open_face,
-                                            typename S::Real *vout = nullptr) {
-  using Real = typename S::Real;
-  using T = typename S::T;
-  const unsigned N = a.N;
-  const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
-  const T *__restrict__ fb = static_cast<const T *>(a.f_in) + n;
-  Real d[Q];
-  // FEAT_OPEN: the lattice has pressure or velocity faces. A separate
-  // instantiation keeps the code of the lattices without them as it is (any
-  // extra branch in this gather changes the register allocation of the
-  // plain path at its 80-register cap and costs it ~15 %).
-  // 16-bit storage: d[q] = (f_q - w_q)/w_q = g_q + the source cell's reference
-  auto gather_cells = [&]() {
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      if constexpr (S::kShift)
-        d[q] = S::template ld_e<q>(fb + (int(q * N) + src_delta<q>(g))) +
-               __ldg(a.rf_in + (long long)n + src_delta<q>(g));
-      else
-        d[q] = S::template ld_f<q>(fb + (int(q * N) + src_delta<q>(g)));
-    });
-  };
-  auto gather_bounce = [&]() {
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      const bool bb = fluid_class<q>(g, link, a.f_wall) == PULL_BOUNCE;
-      if constexpr (S::kShift)
-        d[q] = S::template ld_e<q>(fb + (bb ? int(opp(q) * N) : int(q * N) + src_delta<q>(g))) +
-               __ldg(a.rf_in + (long long)n + (bb ? 0 : src_delta<q>(g)));
-      else
-        d[q] = S::template ld_f<q>(fb + (bb ? int(opp(q) * N) : int(q * N) + src_delta<q>(g)));
-    });
-  };
-  if constexpr (!(FEAT & FEAT_OPEN)) {
-    // every source is a cell, or bounce-back
-    if (link == 0 && !(g.onface & a.f_wall))
-      gather_cells();
-    else
-      gather_bounce();
-  } else {
-    if (link == 0 && !(g.onface & (a.f_wall | a.f_press | a.f_vel))) {
-      gather_cells();
-    } else if (g.onface & (a.f_press | a.f_vel)) {
-      const Pops<Real> o = gather_open_faces<S>(a, g, n, link);
-      Unroll<0, Q>::run([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        d[q] = S::kShift ? o.v[q] * Real(inv_wq(q)) : o.v[q];
-      });
-    } else {
-      gather_bounce();
-    }
-  }
-  // every load of the interior path is issued before any arithmetic, so a
-  // warp keeps its 38 population rows and static fields in flight together
-  const Real eps = __ldg(a.eps + n);
-  KinvRows<Real, KMODE, (FEAT & FEAT_SPEC) != 0> kr;
-  kr.load(a.kinv, N, n);
-  Real hh[SOLUTE ? Q : 1];
-  Real gx = Real(0), gy = Real(0), gz = Real(0);
-  const T *__restrict__ hb = static_cast<const T *>(a.h_in) + n;
-  const unsigned s_open = a.s_inlet | a.s_outlet;
-  const bool h_simple = SOLUTE && link == 0 && !(g.onface & (a.s_wall | s_open));
-  if (SOLUTE) {
-    gx = __ldg(a.geps + n);
-    gy = __ldg(a.geps + N + n);
-    gz = __ldg(a.geps + 2 * size_t(N) + n);
-    open_face = (g.onface & s_open) != 0;
-    if (h_simple) {
-      Unroll<0, Q>::run([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        hh[SOLUTE ? q : 0] = S::template ld_h<q>(hb + (int(q * N) + src_delta<q>(g)));
-      });
-    }
-  }
-  Real V[3];
-  fluid_moments<S::kShift>([&](auto qc) { return d[decltype(qc)::value]; }, drho, V);
-  const Real rho = Real(1) + drho;
-  const Real ie = rcp(eps);
-
-  if constexpr (SOLUTE) {
-    if (!h_simple) {
-      const Real vi0 = V[0] + gx, vi1 = V[1] + gy, vi2 = V[2] + gz;
-      Unroll<0, Q>::run([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        const int cls = solute_class<q>(g, link, a.s_wall, a.s_inlet, a.s_outlet);
-        Real v;
-        if (cls == PULL_CELL) {
-          v = S::template ld_h<q>(hb + (int(q * N) + src_delta<q>(g)));
-        } else if (cls == PULL_BOUNCE) {
-          v = S::template ld_h<opp(q)>(hb + int(opp(q) * N));
-        } else if (cls == PULL_INLET) {
-          // entering through an inlet face: h^eq at C_in with the cell's
-          // bare streamed velocity plus D grad(eps)/eps
-          const Real cv = Real(cx(q)) * vi0 + Real(cy(q)) * vi1 + Real(cz(q)) * vi2;
-          v = wq<Real>(q) * eps * a.C_in * (Real(1) + Real(3) * cv);
-          fin_acc += v - S::template ld_h<opp(q)>(hb + int(opp(q) * N));
-        } else {
-          // outlet: the cell's own post-collision value (zero gradient)
-          v = S::template ld_h<q>(hb + int(q * N));
-          fout_acc += S::template ld_h<opp(q)>(hb + int(opp(q) * N)) - v;
-        }
-        hh[SOLUTE ? q : 0] = v;
-      });
-    }
-    Unroll<0, Q>::run([&](auto qc) { sC += hh[SOLUTE ? decltype(qc)::value : 0]; });
-  }
-  collide_tail<S, KMODE, SOLUTE, (FEAT & FEAT_SPEC) != 0>(
-      a, n, g, [&](auto qc) { return d[decltype(qc)::value]; },
-      [&](auto qc) { return hh[SOLUTE ? decltype(qc)::value : 0]; },
-      [&](int r) { return kr.row(a.kinv, N, n, r); }, drho, rho, V, ie, eps, sC, gx, gy, gz,
-      vout);
-}
-
+// One step of a cell from global memory: stream f (and h), moments,
+// viscosity, colour gradient, V' and the Darcy force, fluid and solute
+// collision, store; accumulates the cell's flux and totals. 16-bit storage
+// with solute (the paired layout): one 32-bit load brings f_q and h_q of a
+// source cell, one more its reference pair, and both lattices are gathered
+// per unit weight, d[q] = (f_q - w_q)/w_q and hh[q] = h_q/w_q (remainder + the
+// source's reference).
 template <class S, int KMODE, bool SOLUTE, int FEAT = 0>
 __device__ __forceinline__ void update_cell(const StepArgs<typename S::Real> &a, unsigned x,
                                             unsigned y, unsigned z, unsigned n, uint32_t link,
@@ -924,12 +995,153 @@ __device__ __forceinline__ void update_cell(const StepArgs<typename S::Real> &a,
                                             typename S::Real &fout_acc, typename S::Real &drho,
                                             typename S::Real &sC, bool &open_face,
                                             typename S::Real *vout = nullptr) {
-  if constexpr (S::kShift && SOLUTE)
-    update_cell_paired<S, KMODE, FEAT>(a, x, y, z, n, link, fin_acc, fout_acc, drho, sC, open_face,
-                                       vout);
-  else
-    update_cell_sep<S, KMODE, SOLUTE, FEAT>(a, x, y, z, n, link, fin_acc, fout_acc, drho, sC,
-                                            open_face, vout);
+  using Real = typename S::Real;
+  using T = typename S::T;
+  constexpr bool kPair = S::kShift && SOLUTE;
+  const unsigned N = a.N;
+  const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
+  Real d[Q], hh[SOLUTE ? Q : 1];
+  // element of row `row` of a population buffer at n + off
+  auto at = [&](auto e, const void *base, int row, int off) {
+    using E = decltype(e);
+    return static_cast<const E *>(base) + n + (row * int(N) + off);
+  };
+  auto both = [&](auto qc, int row, int off) {
+    [[maybe_unused]] constexpr int q = decltype(qc)::value;
+    if constexpr (kPair) {
+      const float2 p = S::ld2(at(typename S::T2{}, a.f_in, row, off));
+      const float2 r = ld_ref2(a.rf_in + n + off);
+      const auto v = Lat<Real, true>::add(Lat<Real, true>::mk(p.x, p.y), Lat<Real, true>::mk(r.x, r.y));
+      d[q] = v.lo();
+      hh[SOLUTE ? q : 0] = v.hi();
+    }
+  };
+  auto ld_f = [&](auto qc, int row, int off) -> Real {  // the row of q or of opp(q): same weight
+    [[maybe_unused]] constexpr int q = decltype(qc)::value;
+    if constexpr (kPair)
+      return S::ld2(at(typename S::T2{}, a.f_in, row, off)).x + ld_ref2(a.rf_in + n + off).x;
+    else if constexpr (S::kShift)
+      return S::template ld_e<q>(at(T{}, a.f_in, row, off)) + __ldg(a.rf_in + n + off);
+    else
+      return S::template ld_f<q>(at(T{}, a.f_in, row, off));
+  };
+  auto ld_h = [&](auto qc, int row, int off) -> Real {
+    [[maybe_unused]] constexpr int q = decltype(qc)::value;
+    if constexpr (kPair)
+      return S::ld2(at(typename S::T2{}, a.f_in, row, off)).y + ld_ref2(a.rf_in + n + off).y;
+    else
+      return S::template ld_h<q>(at(T{}, a.h_in, row, off));
+  };
+  Real eps, gx = Real(0), gy = Real(0), gz = Real(0);
+  KinvRows<Real, KMODE> kr;
+  auto statics = [&]() {
+    eps = __ldg(a.eps + n);
+    if constexpr (SOLUTE) {
+      gx = __ldg(a.geps + n);
+      gy = __ldg(a.geps + N + n);
+      gz = __ldg(a.geps + 2 * size_t(N) + n);
+    }
+    kr.load(a.kinv, N, n);
+  };
+  const unsigned s_open = a.s_inlet | a.s_outlet;
+  open_face = SOLUTE && (g.onface & s_open) != 0;
+  const unsigned open = ((FEAT & FEAT_OPEN) ? a.f_press | a.f_vel : 0u) | (SOLUTE ? s_open : 0u);
+  const unsigned walls = a.f_wall | (SOLUTE ? a.s_wall : 0u);
+  if (!(g.onface & open)) {
+    // Every lane first loads from the cells at n - c_q, whatever is there (the
+    // wrapped source is always a cell of the lattice): a warp keeps its 38
+    // population rows in flight together, and the link word travels with
+    // them. The directions that bounce back are loaded again afterwards. (When
+    // the link word decided the addresses, a warp of a medium with 10 % solid
+    // cells waited for it, then for a gather of its plain lanes, then for one
+    // of its lanes beside solid cells.)
+    Unroll<0, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      if constexpr (kPair)
+        both(qc, q, src_delta<q>(g));
+      else
+        d[q] = ld_f(qc, q, src_delta<q>(g));
+    });
+    if constexpr (SOLUTE && !kPair)
+      Unroll<0, Q>::run([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        hh[q] = ld_h(qc, q, src_delta<q>(g));
+      });
+    statics();
+    if (link != 0 || (g.onface & walls)) {
+      const uint32_t mf = bounce_mask(link, g.onface & a.f_wall);
+      const uint32_t mh = SOLUTE ? bounce_mask(link, g.onface & a.s_wall) : mf;
+      Unroll<1, Q>::run([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        if (kPair && ((mf & mh) >> q & 1u)) {
+          both(qc, opp(q), 0);
+        } else {
+          if ((mf >> q) & 1u) d[q] = ld_f(qc, opp(q), 0);
+          if (SOLUTE && ((mh >> q) & 1u)) hh[SOLUTE ? q : 0] = ld_h(qc, opp(q), 0);
+        }
+      });
+    }
+  } else {
+    // on inlet, outlet, pressure or velocity faces
+    if (((FEAT & FEAT_OPEN) != 0) && (g.onface & (a.f_press | a.f_vel))) {
+      const Pops<Real> o = gather_open_faces<S>(a, g, n, link);
+      Unroll<0, Q>::run([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        d[q] = S::kShift ? o.v[q] * Real(inv_wq(q)) : o.v[q];
+      });
+    } else {
+      const uint32_t mf = bounce_mask(link, g.onface & a.f_wall);
+      Unroll<0, Q>::run([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        const bool b = (mf >> q) & 1u;
+        d[q] = ld_f(qc, b ? opp(q) : q, b ? 0 : src_delta<q>(g));
+      });
+    }
+    if constexpr (SOLUTE) {
+      // the solute classes; 16-bit paired values are per unit weight, their
+      // fluxes carry the weights
+      Real V[3], r_, s_;
+      Lat<Real, false> sd_[Q];
+      moments<S, false>([&](auto qc) { return d[decltype(qc)::value]; },
+                        [&](auto) { return Real(0); }, r_, s_, V, sd_);
+      const Real vi0 = V[0] + __ldg(a.geps + n), vi1 = V[1] + __ldg(a.geps + N + n),
+                 vi2 = V[2] + __ldg(a.geps + 2 * size_t(N) + n);
+      Unroll<0, Q>::run([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        constexpr Real wu = kPair ? Real(1) : wq<Real>(q), wf = kPair ? wq<Real>(q) : Real(1);
+        const int cls = solute_class<q>(g, link, a.s_wall, a.s_inlet, a.s_outlet);
+        Real v;
+        if (cls == PULL_CELL) {
+          v = ld_h(qc, q, src_delta<q>(g));
+        } else if (cls == PULL_BOUNCE) {
+          v = ld_h(qc, opp(q), 0);
+        } else if (cls == PULL_INLET) {
+          // entering through an inlet face: h^eq at C_in with the cell's bare
+          // streamed velocity plus D grad(eps)/eps
+          const Real cv = Real(cx(q)) * vi0 + Real(cy(q)) * vi1 + Real(cz(q)) * vi2;
+          v = wu * __ldg(a.eps + n) * a.C_in * (Real(1) + Real(3) * cv);
+          const Real f = wf * (v - ld_h(qc, opp(q), 0));
+          if (!(link >> 31)) fin_acc += f;
+        } else {
+          // outlet: the cell's own post-collision value (zero gradient)
+          v = ld_h(qc, q, 0);
+          const Real f = wf * (ld_h(qc, opp(q), 0) - v);
+          if (!(link >> 31)) fout_acc += f;
+        }
+        hh[q] = v;
+      });
+    }
+  }
+  if (g.onface & open) statics();
+  if (link >> 31) return;  // impermeable: never updated
+  Real V[3];
+  auto fv = [&](auto qc) { return d[decltype(qc)::value]; };
+  auto hv = [&](auto qc) { return hh[SOLUTE ? decltype(qc)::value : 0]; };
+  Lat<Real, SOLUTE> sd[Q];
+  moments<S, SOLUTE>(fv, hv, drho, sC, V, sd);
+  const Real ie = rcp_as<S>(eps);
+  collide_tail<S, KMODE, SOLUTE, (FEAT & FEAT_TENS) != 0, (FEAT & FEAT_SPEC) != 0>(
+      a, n, g, fv, hv, [&](int r) { return kr.v[r]; }, sd, drho, V, ie, eps, sC, gx, gy, gz, vout);
 }
 
 // Solute species sp >= 1 of one cell, after the fluid and species 0 of the
@@ -992,57 +1204,120 @@ __device__ __forceinline__ void species_update(const StepArgs<typename S::Real> 
       hh[q] = v;
     });
   }
-  Unroll<0, Q>::run([&](auto qc) { sC += hh[decltype(qc)::value]; });
-  const Real vs0 = vel[3] + gx, vs1 = vel[4] + gy, vs2 = vel[5] + gz;
-  Real hsum = Real(0);
-  Unroll<1, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const Real cv = Real(cx(q)) * vs0 + Real(cy(q)) * vs1 + Real(cz(q)) * vs2;
-    const Real heq = wq<Real>(q) * sC * (Real(1) + Real(3) * cv);
-    hsum += heq;
-    const Real h = hh[q];
-    const Real shift = S::kShift ? wq<Real>(q) * sC : Real(0);
-    S::template st_h<q>(ho + int(q * N), h + (heq - h) * itd - shift);
-  });
-  {
+  if constexpr (S::kShift) {
+    // weighted rows against an FP32 reference: the remainder h~_q - w_q sC
+    Unroll<0, Q>::run([&](auto qc) { sC += hh[decltype(qc)::value]; });
+    const Real vs0 = vel[3] + gx, vs1 = vel[4] + gy, vs2 = vel[5] + gz;
+    Real hsum = Real(0);
+    Unroll<1, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const Real cv = Real(cx(q)) * vs0 + Real(cy(q)) * vs1 + Real(cz(q)) * vs2;
+      const Real heq = wq<Real>(q) * sC * (Real(1) + Real(3) * cv);
+      hsum += heq;
+      const Real h = hh[q];
+      S::template st_h<q>(ho + int(q * N), h + (heq - h) * itd - wq<Real>(q) * sC);
+    });
     const Real h = hh[0];
-    const Real shift = S::kShift ? wq<Real>(0) * sC : Real(0);
-    S::template st_h<0>(ho, h + ((sC - hsum) - h) * itd - shift);
+    S::template st_h<0>(ho, h + ((sC - hsum) - h) * itd - wq<Real>(0) * sC);
+    a.rh_out[size_t(sp) * N + n] = float(sC);
+  } else {
+    // the same operations as species 0's (moments, collide_tail), so that
+    // equal species stay bit-identical
+    Real diag = Real(0), axis = Real(0), dif[9];
+    Unroll<0, 9>::run([&](auto kc) {
+      constexpr int k = decltype(kc)::value, q = pair_first(k), o = opp(q);
+      const Real p = add_rn(hh[q], hh[o]);
+      dif[k] = sub_rn(hh[q], hh[o]);
+      hh[q] = p;  // the pair's sum
+      if (inv_wq(q) == 18)
+        axis = q == 5 ? p : add_rn(axis, p);
+      else
+        diag = q == 1 ? p : add_rn(diag, p);
+    });
+    sC = add_rn(add_rn(diag, axis), hh[0]);
+    SoluteRows<Real> so;
+    so.fold(sC, itd, vel[3] + gx, vel[4] + gy, vel[5] + gz);
+    const Real om = Real(1) - itd, half = Real(0.5) * om;
+    Unroll<0, 9>::run([&](auto kc) {
+      constexpr int k = decltype(kc)::value, q = pair_first(k), o = opp(q);
+      Real od = along<q>(so.H, Lat1<Real>{}), e = so.e;
+      if (inv_wq(q) == 18) {
+        od = add_rn(od, od);
+        e = add_rn(e, e);
+      }
+      e = fma(half, hh[q], e);
+      od = fma(half, dif[k], od);
+      S::template st_h<q>(ho + int(q * N), add_rn(e, od));
+      S::template st_h<o>(ho + int(o * N), sub_rn(e, od));
+    });
+    S::template st_h<0>(ho, fma(om, hh[0], so.rest));
   }
-  if constexpr (S::kShift) a.rh_out[size_t(sp) * N + n] = float(sC);
   if (a.fields) a.fields[(5 + size_t(sp)) * N + n] = float(sC * rcp(eps));
 }
 
-// One time step for every non-solid cell (see update_cell).
-// Launch: block (BX, BY) of STEP_BLOCK threads with BX a multiple of 32,
-// grid (ceil(nx/BX), ceil(ny/BY), nz); a warp covers 32 consecutive x of one
-// row. Six resident 128-thread blocks per SM (at most 85 registers a
+// The cell of thread `tid` of block (bx, by, bz) of a per-cell launch with
+// rows of `row` threads, and its warp's number in the launch.
+// Two mappings. Rows: block (row, STEP_BLOCK/row), grid (ceil(nx/row),
+// ceil(ny/(STEP_BLOCK/row)), nz), a warp covers 32 consecutive x of one row
+// (nothing to divide). Linear (a.linear): the threads of the launch take the
+// cells in the order of n. Where the rows do not fill whole warps the row
+// mapping leaves lanes idle (half of them at nx = 16, a warp in four at nx =
+// 96), and its rows start inside a 128-byte line; cell_shape picks.
+struct CellIndex {
+  unsigned x, y, z, n, warp;
+  bool in;
+};
+template <class Real>
+__device__ __forceinline__ CellIndex cell_index(const StepArgs<Real> &a, unsigned bx, unsigned by,
+                                                unsigned bz, unsigned gx, unsigned gy, unsigned row,
+                                                unsigned tx, unsigned ty,
+                                                unsigned threads = STEP_BLOCK) {
+  CellIndex c;
+  if (a.linear) {
+    const unsigned tid = ty * row + tx;
+    c.n = bx * threads + tid;
+    c.in = c.n < a.N;
+    const unsigned yz = a.by_nx.div(c.n);
+    c.x = c.n - yz * unsigned(a.nx);
+    c.z = a.by_ny.div(yz);
+    c.y = yz - c.z * unsigned(a.ny);
+    c.warp = c.n >> 5;
+  } else {
+    c.x = bx * row + tx;
+    c.y = by * (STEP_BLOCK / row) + ty;
+    c.z = bz;
+    c.in = c.x < unsigned(a.nx) && c.y < unsigned(a.ny);
+    c.n = c.x + unsigned(a.nx) * (c.y + unsigned(a.ny) * c.z);
+    c.warp = ((bz * gy + by) * gx + bx) * (STEP_BLOCK / 32) + ((ty * row + tx) >> 5);
+  }
+  return c;
+}
+
+// One time step for every non-solid cell (see update_cell; launch shapes at
+// cell_index). Six resident 128-thread blocks per SM (at most 85 registers a
 // thread): measured on GB300 at 128^3 this is 1.1x faster than the
 // unconstrained build (112 registers), since the kernel is bound by loads in
 // flight, and a little faster than 256-thread blocks at the same occupancy.
+// FP64 populations take twice the registers, and the FP64 pipe is busy with a
+// few warps: three blocks (168 registers) instead of six with spills.
+template <class Real>
+constexpr int step_blocks() {
+  return sizeof(Real) == 8 ? 3 : 6;
+}
 template <class S, int KMODE, bool SOLUTE, int FEAT>
-__global__ void __launch_bounds__(STEP_BLOCK, 6) step_kernel(const StepArgs<typename S::Real> a) {
+__global__ void __launch_bounds__(STEP_BLOCK, step_blocks<typename S::Real>()) step_kernel(const StepArgs<typename S::Real> a) {
   using Real = typename S::Real;
-  const unsigned x = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned y = blockIdx.y * blockDim.y + threadIdx.y;
-  const unsigned z = blockIdx.z;
-  const unsigned nx = a.nx, ny = a.ny;
-  const unsigned warp_gid =
-      ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (STEP_BLOCK / 32) +
-      ((threadIdx.y * blockDim.x + threadIdx.x) >> 5);
-  bool live = x < nx && y < ny;
-  const unsigned n = x + nx * (y + ny * z);
-  uint32_t link = 0;
-  if (live && a.link) {
-    link = __ldg(a.link + n);
-    live = !(link >> 31);
-  }
+  const CellIndex c = cell_index(a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y,
+                                 blockDim.x, threadIdx.x, threadIdx.y, blockDim.x);
+  const unsigned x = c.x, y = c.y, z = c.z, n = c.n, warp_gid = c.warp;
+  const uint32_t link = (c.in && a.link) ? __ldg(a.link + n) : 0u;
   Real fin_acc = Real(0), fout_acc = Real(0), drho = Real(0), sC = Real(0);
   bool open_face = false;
   Real vel[6];
-  if (live)
+  if (c.in)  // returns early in solid cells
     update_cell<S, KMODE, SOLUTE, FEAT>(a, x, y, z, n, link, fin_acc, fout_acc, drho, sC,
                                         open_face, (FEAT & FEAT_SPEC) ? vel : nullptr);
+  [[maybe_unused]] const bool live = c.in && !(link >> 31);
   warp_reductions(a, warp_gid, open_face, fin_acc, fout_acc, drho, sC);
   if constexpr ((FEAT & FEAT_SPEC) != 0) {
     // further species, each with its per-warp flux slots and finite check
@@ -1059,10 +1334,7 @@ __global__ void __launch_bounds__(STEP_BLOCK, 6) step_kernel(const StepArgs<type
           slot[1] += double(so);
         }
       }
-      if (a.reduce) {
-        const Real c = warp_sum(sC_s);
-        if (lane == 0 && !isfinite(c)) atomicOr(&a.state->status, 1u);
-      }
+      if (a.reduce) finite_check(a.state, sC_s, Real(0));
     }
   }
 }

@@ -120,7 +120,8 @@ __global__ void __launch_bounds__(STEP_BLOCK, 4)
     bool open_face = false;
     if (live) {
       const CellGeo g = cell_geo_xyz(x, y, z, nx, ny, nz);
-      const bool simple = link == 0 && !(g.onface & a.f_wall) &&
+      // (surface tension takes the per-cell path: one inlined collision fewer)
+      const bool simple = a.A == Real(0) && link == 0 && !(g.onface & a.f_wall) &&
                           (!SOLUTE || !(g.onface & (a.s_wall | a.s_inlet | a.s_outlet)));
       if (simple) {
         const Real *const src = sv + size_t(s) * L::kRows * bx + tid;
@@ -132,16 +133,20 @@ __global__ void __launch_bounds__(STEP_BLOCK, 4)
           gx = src[L::kGeps * bx];
           gy = src[(L::kGeps + 1) * bx];
           gz = src[(L::kGeps + 2) * bx];
-          Unroll<0, Q>::run([&](auto qc) { sC += src[(L::kH + decltype(qc)::value) * bx]; });
         }
         Real V[3];
-        fluid_moments([&](auto qc) { return d[decltype(qc)::value]; }, drho, V);
-        const Real rho = Real(1) + drho;
-        const Real ie = rcp(eps);
-        collide_tail<S, KMODE, SOLUTE>(
-            a, n, g, [&](auto qc) { return d[decltype(qc)::value]; },
-            [&](auto qc) { return src[(L::kH + decltype(qc)::value) * bx]; },
-            [&](int k) { return src[(L::kKin + k) * bx]; }, drho, rho, V, ie, eps, sC, gx, gy, gz);
+        auto fv = [&](auto qc) { return d[decltype(qc)::value]; };
+        auto hv = [&](auto qc) {
+          return SOLUTE ? src[(L::kH + decltype(qc)::value) * bx] : Real(0);
+        };
+        Lat<Real, SOLUTE> sd[Q];
+        moments<S, SOLUTE>(fv, hv, drho, sC, V, sd);
+        const Real ie = rcp1(eps);
+        auto kv = [&](int k) { return src[(L::kKin + k) * bx]; };
+        collide_tail<S, KMODE, SOLUTE, false>(a, n, g, fv, hv, kv, sd, drho, V, ie, eps, sC, gx, gy, gz);
+      } else if (a.A != Real(0)) {
+        update_cell<S, KMODE, SOLUTE, FEAT_TENS>(a, x, y, z, n, link, fin_acc, fout_acc, drho, sC,
+                                                 open_face);
       } else {
         update_cell<S, KMODE, SOLUTE>(a, x, y, z, n, link, fin_acc, fout_acc, drho, sC, open_face);
       }

@@ -255,9 +255,12 @@ __global__ void __launch_bounds__(32 * (NW + 1), MINB)
     const unsigned closed = a.f_wall | a.s_wall | a.s_inlet | a.s_outlet;
     const unsigned yzface = (y == 0 ? 4u : 0u) | (y == ny - 1 ? 8u : 0u) | (z == 0 ? 16u : 0u) |
                             (z == nz - 1 ? 32u : 0u);
-    const bool interior = !a.link && !(closed & 3u) && !(yzface & closed);
+    const bool interior = a.A == Real(0) && !a.link && !(closed & 3u) && !(yzface & closed);
     if (live && !interior) {
-      update_cell<S, KMODE, SOLUTE>(a, x, y, z, n, link, fa, fo_, drho, sC, open_face);
+      if (a.A != Real(0))
+        update_cell<S, KMODE, SOLUTE, FEAT_TENS>(a, x, y, z, n, link, fa, fo_, drho, sC, open_face);
+      else
+        update_cell<S, KMODE, SOLUTE>(a, x, y, z, n, link, fa, fo_, drho, sC, open_face);
     } else if (live) {
       const unsigned xm = (x == 0) ? nx - 1 : x - 1, xp = (x == nx - 1) ? 0 : x + 1;
       // arriving populations from the staged rows (re-read in the collision pass)
@@ -272,22 +275,21 @@ __global__ void __launch_bounds__(32 * (NW + 1), MINB)
         return S::template cv_h<q>(lds_row<T>(shp + q * nx + xs));
       };
       Real V[3];
-      fluid_moments(fval, drho, V);
-      const Real rho = Real(1) + drho;
+      Lat<Real, SOLUTE> sd[Q];
+      moments<S, SOLUTE>(fval, hval, drho, sC, V, sd);
       const Real eps = Real(sst[x]);
-      const Real ie = rcp(eps);
+      const Real ie = rcp1(eps);
       Real gx = Real(0), gy = Real(0), gz = Real(0);
       if (SOLUTE) {
         gx = Real(sst[(1 + L::kinv_rows) * nx + x]);
         gy = Real(sst[(2 + L::kinv_rows) * nx + x]);
         gz = Real(sst[(3 + L::kinv_rows) * nx + x]);
-        Unroll<0, Q>::run([&](auto qc) { sC += hval(qc); });
       }
       // the collision pass re-reads the staged rows; K^-1 from shared memory
-      collide_tail<S, KMODE, SOLUTE>(
-          a, n, cell_geo_xyz(x, y, z, nx, ny, nz), fval, hval,
-          [&](int k2) { return Real(sst[(1 + k2) * nx + x]); }, drho, rho, V, ie, eps, sC, gx, gy,
-          gz);
+      const CellGeo g = cell_geo_xyz(x, y, z, nx, ny, nz);
+      auto kv = [&](int k2) { return Real(sst[(1 + k2) * nx + x]); };
+      collide_tail<S, KMODE, SOLUTE, false>(a, n, g, fval, hval, kv, sd, drho, V, ie, eps, sC, gx, gy,
+                                            gz);
     }
     // the stage may be refilled once every compute warp has read it
     __syncwarp();
@@ -297,10 +299,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), MINB)
       flux_in += warp_sum(fa);
       flux_out += warp_sum(fo_);
     }
-    if (a.reduce) {
-      const Real m = warp_sum(drho), c = warp_sum(sC);
-      if (lane == 0 && !(isfinite(m) && isfinite(c))) atomicOr(&a.state->status, 1u);
-    }
+    if (a.reduce) finite_check(a.state, drho, sC);
   }
   if (a.flux && lane == 0 && (flux_in != Real(0) || flux_out != Real(0))) {
     a.flux_slots[2 * size_t(warp_gid)] += double(flux_in);
