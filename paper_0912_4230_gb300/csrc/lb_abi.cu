@@ -92,16 +92,13 @@ struct lb_ctx {
   double *flux_slots = nullptr;  // per-warp cumulative inlet / outlet flux
   DevState *state = nullptr;
   // free surface
-  uint8_t *type[2] = {nullptr, nullptr};
-  void *mass[2] = {nullptr, nullptr};
-  void *lam = nullptr, *rho_post = nullptr, *share = nullptr, *mom = nullptr;
-  uint8_t *flag_a = nullptr, *flag_b = nullptr;
-  unsigned *any = nullptr;
-  // free surface: active-tile lists (step parity), their lengths, tile stamps
+  uint8_t *type = nullptr, *flag = nullptr;
+  void *mass = nullptr, *lam = nullptr, *rho_post = nullptr, *mom = nullptr;
+  uint32_t *flagged = nullptr, *near = nullptr;  // cells that convert, and with their neighbours
+  // free surface: active-tile lists (parity of the epoch), tile stamps, counters
   uint32_t *tiles[2] = {nullptr, nullptr};
-  unsigned *n_tiles = nullptr;
   unsigned *stamp = nullptr;
-  unsigned *stamp_ctr = nullptr;  // steps taken since lb_init (device)
+  FsCount *fs_cnt = nullptr;
   unsigned ntx = 0, nty = 0, ntz = 0, fs_grid = 0;
   // table of lb_step_batch calls led by this context
   void *batch_tab = nullptr;
@@ -264,8 +261,7 @@ struct Layout {
   size_t f, h, rf, rh;   // per population buffer (two of each; 0 = not allocated)
   size_t spec;           // several species: per-species constants
   size_t eps, link, fields, partials, state, geps, rhohat, face;
-  size_t fs_type, fs_mass, fs_lam, fs_rho, fs_share, fs_mom, fs_flag, fs_any, fs_tiles, fs_ntiles,
-      fs_stamp, fs_stamp_ctr;
+  size_t fs_type, fs_mass, fs_lam, fs_rho, fs_mom, fs_flag, fs_list, fs_tiles, fs_stamp, fs_cnt;
   size_t kinv, flux_slots;
   size_t create_stage;   // inputs of lb_create, released before it returns
   size_t init_stage;     // inputs of lb_init, kept for later staging
@@ -309,14 +305,12 @@ Layout layout_of(const lb_domain &dom, const lb_params &prm, const StorageOps &o
     L.fs_mass = N * rb;
     L.fs_lam = N * rb;
     L.fs_rho = N * rb;
-    L.fs_share = N * rb;
     L.fs_mom = 4 * N * rb;
-    L.fs_flag = N;
-    L.fs_any = sizeof(unsigned);
+    L.fs_flag = (N + 3) / 4 * 4;  // updated by whole words
+    L.fs_list = N * sizeof(uint32_t);
     L.fs_tiles = ntiles * sizeof(uint32_t);
-    L.fs_ntiles = 2 * sizeof(unsigned);
     L.fs_stamp = ntiles * sizeof(unsigned);
-    L.fs_stamp_ctr = sizeof(unsigned);
+    L.fs_cnt = sizeof(FsCount);
   }
   L.kinv = size_t(k_rows) * N * rb;
   L.flux_slots = size_t(slot_warps(dom)) * 2 * S * sizeof(double);
@@ -438,35 +432,32 @@ bool pipe_shape(const lb_ctx *c, unsigned bx, lb_ctx::PipeShape *ps) {
   return ps->grid * (bx / 32) <= c->nwarps;  // within the flux slots (always, by slot_warps)
 }
 
-// Free-surface arguments of the step that brings the state to step index t
-// (t = 0: the arguments that seed the first step's tiles).
+// Free-surface arguments (the same for every step of a parity; the step's
+// index and lists live on the device).
 template <class Real>
-FsArgs<Real> fs_args(lb_ctx *c, const StepArgs<Real> &a, long long t) {
+FsArgs<Real> fs_args(lb_ctx *c, const StepArgs<Real> &a) {
   FsArgs<Real> fa;
   fa.a = a;
-  fa.a.fields = c->fields;  // rho and V' of every live cell feed the re-typing
   fa.a.link = c->link;
-  fa.type_old = c->type[c->cur];
-  fa.type_new = c->type[1 - c->cur];
-  fa.m_old = static_cast<Real *>(c->mass[c->cur]);
-  fa.m_new = static_cast<Real *>(c->mass[1 - c->cur]);
+  fa.fields = c->fields;
+  fa.type = c->type;
+  fa.m = static_cast<Real *>(c->mass);
   fa.lam = static_cast<Real *>(c->lam);
   fa.rhohat_w = static_cast<Real *>(c->rhohat);
-  fa.flag_a = c->flag_a;
-  fa.flag_b = c->flag_b;
+  fa.flag = c->flag;
+  fa.flagged = c->flagged;
+  fa.near = c->near;
   fa.rho_post = static_cast<Real *>(c->rho_post);
-  fa.share = static_cast<Real *>(c->share);
   fa.mom = static_cast<Real *>(c->mom);
-  fa.any = c->any;
-  fa.tiles = c->tiles[t & 1];
-  fa.n_tiles = c->n_tiles + (t & 1);
-  fa.next_tiles = c->tiles[(t + 1) & 1];
-  fa.next_n_tiles = c->n_tiles + ((t + 1) & 1);
+  fa.cnt = c->fs_cnt;
+  fa.tiles[0] = c->tiles[0];
+  fa.tiles[1] = c->tiles[1];
   fa.stamp = c->stamp;
-  fa.stamp_ctr = c->stamp_ctr;
   fa.ntx = c->ntx;
   fa.nty = c->nty;
   fa.ntz = c->ntz;
+  fa.by_ntx = FastDiv::of(c->ntx);
+  fa.by_nty = FastDiv::of(c->nty);
   return fa;
 }
 
@@ -497,9 +488,8 @@ int enqueue_step(lb_ctx *c, cudaStream_t s, bool last) {
     a.reduce = (c->prm.check_every > 0 && a.t % c->prm.check_every == 0) ? 1 : 0;
     a.fields = last ? c->fields : nullptr;
     if (c->fs) {
-      a.fields = c->fields;
-      const FsArgs<Real> fa = fs_args(c, a, a.t);
-      CK(c, c->ops->fs_step(&fa, c->fs_grid, (fs_tile_count(c) + BLOCK - 1) / BLOCK, s));
+      const FsArgs<Real> fa = fs_args(c, a);
+      CK(c, c->ops->fs_step(&fa, c->fs_grid, s));
       return int(LB_OK);
     }
     if (c->prm.A != 0.0) CK(c, c->ops->rhohat(args, c->rhohat, c->nblk, s));
@@ -623,10 +613,10 @@ int lb_bytes_required(const lb_domain *dom, const lb_params *prm, int32_t k_rows
   if (prm->species < 0 || prm->species > LB_MAX_SPECIES)
     return fail(nullptr, LB_EINVAL, "species outside [0, LB_MAX_SPECIES]");
   const Layout L = layout_of(*dom, *prm, *ops, k_rows, f_scale != 0);
-  const size_t twice[] = {L.f, L.h, L.rf, L.rh, L.fs_type, L.fs_mass, L.fs_flag, L.fs_tiles};
+  const size_t twice[] = {L.f, L.h, L.rf, L.rh, L.fs_list, L.fs_tiles};
   const size_t once[] = {L.spec, L.eps, L.link, L.fields, L.partials, L.state, L.geps,
-                         L.rhohat, L.face, L.fs_lam, L.fs_rho, L.fs_share, L.fs_mom, L.fs_any,
-                         L.fs_ntiles, L.fs_stamp, L.fs_stamp_ctr, L.kinv, L.flux_slots,
+                         L.rhohat, L.face, L.fs_type, L.fs_mass, L.fs_lam, L.fs_rho, L.fs_mom,
+                         L.fs_flag, L.fs_stamp, L.fs_cnt, L.kinv, L.flux_slots,
                          L.batch_share};
   size_t total = 0;
   for (size_t b : twice) total += 2 * granule(b);
@@ -782,29 +772,24 @@ int lb_create(const lb_domain *dom, const float *porosity, const float *K6, cons
       return bail(fail(c, LB_ECUDA, std::string("face values: ") + cudaGetErrorString(e)));
   }
   if (c->fs) {
-    for (int b = 0; b < 2; ++b) {
-      c->type[b] = static_cast<uint8_t *>(dev_alloc(c, L.fs_type));
-      c->mass[b] = dev_alloc(c, L.fs_mass);
-      if (!c->type[b] || !c->mass[b]) return bail(fail(c, LB_ENOMEM, "free surface"));
-    }
+    c->type = static_cast<uint8_t *>(dev_alloc(c, L.fs_type));
+    c->mass = dev_alloc(c, L.fs_mass);
     c->lam = dev_alloc(c, L.fs_lam);
     c->rho_post = dev_alloc(c, L.fs_rho);
-    c->share = dev_alloc(c, L.fs_share);
     c->mom = dev_alloc(c, L.fs_mom);
-    c->flag_a = static_cast<uint8_t *>(dev_alloc(c, L.fs_flag));
-    c->flag_b = static_cast<uint8_t *>(dev_alloc(c, L.fs_flag));
-    c->any = static_cast<unsigned *>(dev_alloc(c, L.fs_any));
+    c->flag = static_cast<uint8_t *>(dev_alloc(c, L.fs_flag));
+    c->flagged = static_cast<uint32_t *>(dev_alloc(c, L.fs_list));
+    c->near = static_cast<uint32_t *>(dev_alloc(c, L.fs_list));
     c->ntx = (unsigned(dom->nx) + FS_TX - 1) / FS_TX;
     c->nty = (unsigned(dom->ny) + FS_TY - 1) / FS_TY;
     c->ntz = (unsigned(dom->nz) + FS_TZ - 1) / FS_TZ;
     const size_t ntiles = size_t(c->ntx) * c->nty * c->ntz;
     c->tiles[0] = static_cast<uint32_t *>(dev_alloc(c, L.fs_tiles));
     c->tiles[1] = static_cast<uint32_t *>(dev_alloc(c, L.fs_tiles));
-    c->n_tiles = static_cast<unsigned *>(dev_alloc(c, L.fs_ntiles));
     c->stamp = static_cast<unsigned *>(dev_alloc(c, L.fs_stamp));
-    c->stamp_ctr = static_cast<unsigned *>(dev_alloc(c, L.fs_stamp_ctr));
-    if (!c->lam || !c->rho_post || !c->share || !c->mom || !c->flag_a || !c->flag_b || !c->any || !c->tiles[0] ||
-        !c->tiles[1] || !c->n_tiles || !c->stamp || !c->stamp_ctr)
+    c->fs_cnt = static_cast<FsCount *>(dev_alloc(c, L.fs_cnt));
+    if (!c->type || !c->mass || !c->lam || !c->rho_post || !c->mom || !c->flag || !c->flagged ||
+        !c->near || !c->tiles[0] || !c->tiles[1] || !c->stamp || !c->fs_cnt)
       return bail(fail(c, LB_ENOMEM, "free surface"));
     // persistent grid of the tile passes: enough resident blocks to cover
     // the list of a typical step in one round
@@ -977,19 +962,15 @@ int lb_init(lb_ctx *c, const float *rho0, const float *u0, const float *C0,
                         size_t(c->nwarps) * 2 * size_t(std::max(c->S, 1)) * sizeof(double),
                         c->stream));
   if (c->fs) {
-    CK(c, fs_init(c->N, c->link, d_type, d_rho, lambda0 ? d_lam : nullptr, c->type[0], c->type[1],
-                  c->mass[0], c->lam, c->ops->fp64, c->stream));
-    CK(c, rhohat_init(c->N, c->link, d_rho, c->mass[0], c->prm.wall_rho, c->rhohat, c->ops->fp64,
+    CK(c, fs_init(c->N, c->link, d_type, d_rho, lambda0 ? d_lam : nullptr, c->type, c->mass, c->lam,
+                  c->ops->fp64, c->stream));
+    CK(c, rhohat_init(c->N, c->link, d_rho, c->mass, c->prm.wall_rho, c->rhohat, c->ops->fp64,
                       c->stream));
-    // cells outside the active tiles are never written by a step: both mass
-    // buffers and both flag arrays start equal (no flag), no tile is stamped
-    const size_t rb = c->ops->fp64 ? 8 : 4;
-    CK(c, cudaMemcpyAsync(c->mass[1], c->mass[0], N * rb, cudaMemcpyDeviceToDevice, c->stream));
-    CK(c, cudaMemsetAsync(c->flag_a, 0, N, c->stream));
-    CK(c, cudaMemsetAsync(c->flag_b, 0, N, c->stream));
-    CK(c, cudaMemsetAsync(c->stamp, 0, size_t(fs_tile_count(c)) * sizeof(unsigned), c->stream));
-    CK(c, cudaMemsetAsync(c->stamp_ctr, 0, sizeof(unsigned), c->stream));
-    CK(c, cudaMemsetAsync(c->n_tiles, 0, 2 * sizeof(unsigned), c->stream));
+    // no flags, no tile listed, step 0
+    const Layout L = layout_of(c->dom, c->prm, *c->ops, 0, false);
+    CK(c, cudaMemsetAsync(c->flag, 0, L.fs_flag, c->stream));
+    CK(c, cudaMemsetAsync(c->stamp, 0, L.fs_stamp, c->stream));
+    CK(c, cudaMemsetAsync(c->fs_cnt, 0, sizeof(FsCount), c->stream));
   } else if (c->prm.A != 0.0) {
     CK(c, rhohat_init(c->N, c->link, d_rho, nullptr, c->prm.wall_rho, c->rhohat, c->ops->fp64,
                       c->stream));
@@ -1004,13 +985,12 @@ int lb_init(lb_ctx *c, const float *rho0, const float *u0, const float *C0,
     in.u0 = d_u;
     in.C0 = C0 ? d_C : nullptr;
     in.f_scale = f_scale ? d_fs : nullptr;
-    in.type = c->fs ? c->type[0] : nullptr;
+    in.type = c->fs ? c->type : nullptr;
     CK(c, c->ops->init(c->kmode, c->solute, args, &in, c->nblk, c->stream));
     if (c->S > 1) CK(c, c->ops->species_init(args, d_u, d_C, c->nblk, c->stream));
     if (c->fs) {  // the first step's active tiles
-      const FsArgs<Real> fa = fs_args(c, a, 0);
-      CK(c, c->ops->fs_seed(&fa, fs_tile_count(c), (fs_tile_count(c) + BLOCK - 1) / BLOCK,
-                            c->stream));
+      const FsArgs<Real> fa = fs_args(c, a);
+      CK(c, c->ops->fs_seed(&fa, fs_tile_count(c), c->stream));
     }
     return int(LB_OK);
   });
@@ -1324,7 +1304,7 @@ int lb_reduce(lb_ctx *c, double *mass, double *solute, double *flux_in, double *
   if (!out) return fail(c, LB_ENOMEM, "staging");
   double tot[4] = {0.0, 0.0, 0.0, 0.0};
   if (c->fs)
-    CK(c, fs_totals(c->N, c->link, c->mass[c->cur], c->partials, c->ops->fp64, c->stream));
+    CK(c, fs_totals(c->N, c->link, c->mass, c->partials, c->ops->fp64, c->stream));
   else
     CK(c, c->ops->totals(f_view(c), c->solute ? h_view(c, 0) : PopView{},
                          c->has_solid ? c->link : nullptr, c->N, c->partials, c->nblk, c->stream));
@@ -1430,11 +1410,11 @@ int lb_free_surface_state(lb_ctx *c, uint8_t *type, double *mass) {
   if (!c) return LB_EINVAL;
   if (!c->fs) return fail(c, LB_EINVAL, "no free surface in this context");
   const size_t N = c->N;
-  if (type) CK(c, cudaMemcpyAsync(type, c->type[c->cur], N, cudaMemcpyDefault, c->stream));
+  if (type) CK(c, cudaMemcpyAsync(type, c->type, N, cudaMemcpyDefault, c->stream));
   if (mass) {
     double *st = static_cast<double *>(stage(c, N * sizeof(double)));
     if (!st) return fail(c, LB_ENOMEM, "staging");
-    CK(c, to_double(c->N, c->mass[c->cur], st, c->ops->fp64, c->stream));
+    CK(c, to_double(c->N, c->mass, st, c->ops->fp64, c->stream));
     CK(c, cudaMemcpyAsync(mass, st, N * sizeof(double), cudaMemcpyDefault, c->stream));
   }
   CK(c, cudaStreamSynchronize(c->stream));

@@ -295,39 +295,51 @@ struct StepArgs {
 
 // Free-surface state of one step (Section 3): cell types, liquid mass m,
 // liquid fraction lambda and the re-typing scratch.
-// Conversion flags: an interface cell that fills or empties, and (re-typing
-// pass onwards) an empty cell that has become an interface cell.
-enum : uint8_t { FS_NONE = 0, FS_FILL = 1, FS_EMPTYING = 2, FS_NEWCELL = 3 };
+// Conversion flags of a cell, bits of one byte: an interface cell that fills
+// or empties (by its liquid fraction), an emptying cell that stays interface
+// because a neighbour fills, an empty cell that has become an interface cell,
+// and a cell listed as near a conversion.
+enum : uint8_t { FS_NONE = 0, FS_FILL = 1, FS_EMPTYING = 2, FS_NEWCELL = 4, FS_CANCELLED = 8,
+                 FS_CLAIMED = 16 };
+
+// Counters of the free surface, on the device, so that a step's launches are
+// the same every time: steps taken since lb_init (read by a step's first pass,
+// advanced by its second) and the step in progress, the cells flagged in this
+// step, the cells near a conversion (this and the previous step, by parity),
+// the tiles of the current and the next list (by parity of the epoch).
+struct FsCount {
+  unsigned step, now, n_flag, n_near[2], n_tiles[2];
+};
 
 template <class Real>
 struct FsArgs {
-  StepArgs<Real> a;      // fields must be set: rho and V' of every live cell
-  uint8_t *type_old;     // read by the step; the last pass settles it to the new type
-  uint8_t *type_new;
-  Real *m_old;           // read by the step; the last pass settles it to the new mass
-  Real *m_new;
-  Real *lam;             // lambda(t) in, lambda(t+1) out
+  StepArgs<Real> a;      // fields set when the step exports them
+  float *fields;         // the exported fields (an emptied cell's are zeroed at once)
+  uint8_t *type;
+  Real *m;
+  Real *lam;             // of interface cells; a cell that has just filled or
+                         // emptied holds the excess mass of each receiver
   Real *rhohat_w;        // colour-gradient field written by the mass exchange
-  uint8_t *flag_a, *flag_b;
+  uint8_t *flag;         // (N rounded up to whole words)
+  uint32_t *flagged;     // cells that fill or empty in this step
+  uint32_t *near;        // converted cells and their neighbours
   Real *rho_post;        // post-collision density of each live cell (new interface cells:
                          // of their initial populations)
-  Real *share;           // excess mass handed to each interface neighbour
   Real *mom;             // rho, V'_x, V'_y, V'_z (4 x N) of each live cell that pulls
                          // from an empty cell, written by the step pass
-  unsigned *any;         // nonzero when some cell fills or empties this step
-  // Active tiles of FS_TX x FS_TY x FS_TZ cells: the tiles within one tile
-  // (26-neighbourhood, wrapped) of a tile holding a liquid or interface cell.
-  // The step runs over this step's list; its last pass stamps the tiles of
-  // the next step and lists each tile the first time it stamps it.
-  const uint32_t *tiles;
-  const unsigned *n_tiles;
-  uint32_t *next_tiles;
-  unsigned *next_n_tiles;
-  unsigned *stamp;       // per tile: the step whose list holds it
-  unsigned *stamp_ctr;   // steps taken; the next step's stamp is *stamp_ctr + 1 (the
-                         // first pass of a step advances it, so a step is launch-invariant)
+  FsCount *cnt;
+  // Active tiles of FS_TX x FS_TY x FS_TZ cells: the tiles holding a cell
+  // within one link of a liquid or interface cell (wrapped), by parity of the
+  // epoch, and per tile 1 + the latest epoch whose list holds it.
+  uint32_t *tiles[2];
+  unsigned *stamp;
   unsigned ntx, nty, ntz;
+  FastDiv by_ntx, by_nty;
 };
+// steps that one tile list serves before it is built afresh
+constexpr unsigned FS_EPOCH = 16;
+// the launches over the converting cells: a thread per cell
+constexpr unsigned FS_LIST_BLOCK = 64, FS_LIST_GRID = 128;
 constexpr unsigned FS_TX = 32, FS_TY = 1, FS_TZ = 2;
 // the tile passes run one block of FS_BLOCK threads per tile (one thread a
 // cell), with as many blocks per SM as its 2048 threads and 32 blocks allow

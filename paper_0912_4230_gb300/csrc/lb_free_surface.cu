@@ -11,8 +11,8 @@ namespace {
 // when not given), empty m = 0; solid cells are typed empty and never updated
 template <class Real>
 __global__ void fs_init_kernel(unsigned N, const uint32_t *link, const uint8_t *type_in,
-                               const float *rho0, const float *lambda0, uint8_t *type0,
-                               uint8_t *type1, Real *mass, Real *lam) {
+                               const float *rho0, const float *lambda0, uint8_t *type,
+                               Real *mass, Real *lam) {
   const unsigned n = blockIdx.x * BLOCK + threadIdx.x;
   if (n >= N) return;
   uint8_t t = type_in[n];
@@ -26,8 +26,7 @@ __global__ void fs_init_kernel(unsigned N, const uint32_t *link, const uint8_t *
   } else {
     t = CELL_EMPTY;
   }
-  type0[n] = t;
-  type1[n] = t;
+  type[n] = t;
   lam[n] = l;
   mass[n] = (link[n] >> 31) ? Real(0) : l * Real(rho0[n]);
 }
@@ -60,15 +59,15 @@ unsigned blocks_for(unsigned N) { return (N + BLOCK - 1) / BLOCK; }
 }  // namespace
 
 cudaError_t fs_init(unsigned N, const uint32_t *link, const uint8_t *type_in, const float *rho0,
-                    const float *lambda0, uint8_t *type0, uint8_t *type1, void *mass, void *lam,
-                    bool fp64, cudaStream_t s) {
+                    const float *lambda0, uint8_t *type, void *mass, void *lam, bool fp64,
+                    cudaStream_t s) {
   if (fp64)
-    fs_init_kernel<double><<<blocks_for(N), BLOCK, 0, s>>>(N, link, type_in, rho0, lambda0, type0,
-                                                           type1, static_cast<double *>(mass),
+    fs_init_kernel<double><<<blocks_for(N), BLOCK, 0, s>>>(N, link, type_in, rho0, lambda0, type,
+                                                           static_cast<double *>(mass),
                                                            static_cast<double *>(lam));
   else
-    fs_init_kernel<float><<<blocks_for(N), BLOCK, 0, s>>>(N, link, type_in, rho0, lambda0, type0,
-                                                          type1, static_cast<float *>(mass),
+    fs_init_kernel<float><<<blocks_for(N), BLOCK, 0, s>>>(N, link, type_in, rho0, lambda0, type,
+                                                          static_cast<float *>(mass),
                                                           static_cast<float *>(lam));
   return cudaGetLastError();
 }

@@ -1,30 +1,25 @@
 // Free-surface kernels (Section 3 of the paper): liquid-mass exchange,
 // stream/collide of liquid and interface cells with the reconstruction of
 // populations coming from empty cells, and the re-typing of cells whose
-// liquid fraction leaves [0, 1]. One step is five passes over the active
-// tiles (tiles within one tile of a liquid or interface cell; every cell
-// outside them is empty with nothing to do): the mass exchange, the
-// stream/collide with the conversion flags, the re-typing, the new interface
-// cells and excess mass, and the finish (shares received, liquid fraction,
-// the next step's tile list). Each pass needs its neighbours' results of the
-// one before; the conversion passes do nothing unless some cell flagged a
-// conversion in this step.
+// liquid fraction leaves [0, 1].
+//
+// One step is two passes over the active tiles (tiles holding a cell within
+// one link of a liquid or interface cell; every cell outside them is empty
+// with nothing to do) and three launches over the few cells that convert:
+//   fs_mass      liquid-mass exchange, colour-gradient field
+//   fs_step      stream/collide; lists the interface cells that fill or empty
+//   fs_convert   re-types the listed cells and their neighbours
+//   fs_newcell   populations of new interface cells, excess mass
+//   fs_finish    receives the excess mass; liquid fraction, tiles of new cells
+// Each needs its neighbours' results of the one before. A drop of radius 24
+// converts ~100 of its 70 000 cells a step: as passes over all active tiles the
+// conversions took 36 us of a 192x192x128 step (of 55 us), as launches over
+// lists about 10 us (of 39).
 #pragma once
 
 #include "lb_kernels.cuh"
 
 namespace lbgb {
-
-// the neighbour x + c_q, or -1 when the step leaves through a wall face or
-// lands on a solid cell (bit opp(q) of the link word is the solidity of
-// x - c_opp(q) = x + c_q)
-template <int q>
-__device__ __forceinline__ long long fs_neighbor(const CellGeo &g, unsigned n, uint32_t link,
-                                                 unsigned f_wall) {
-  if (faces_ahead(q) & g.onface & f_wall) return -1;
-  if ((link >> opp(q)) & 1u) return -1;
-  return (long long)n + ahead_delta<q>(g);
-}
 
 static_assert(FS_BLOCK % 32 == 0 && FS_BLOCK >= 27,
               "whole warps per tile, and a thread for each of the 27 tiles around it");
@@ -55,14 +50,27 @@ __device__ __forceinline__ unsigned fs_tile_mask(unsigned lx, unsigned ly, unsig
   return m;
 }
 
-// Stamps, for the next step, the tiles of the block-wide OR of the cells'
-// masks around tile (bx, by, bz) (wrapped; every thread of the block calls
-// it); the stamp that first marks a tile for the next step also appends it to
-// the next step's list, so every tile is listed once (in no particular order:
-// a cell's update depends only on the previous step's values).
+// The tile list that step c runs over. A list serves FS_EPOCH steps: tiles of
+// new interface cells are appended as they appear, and its last step stamps the
+// next list from the cells that are live then (a tile that has emptied stays
+// listed until then; its cells do nothing).
+__device__ __forceinline__ unsigned fs_epoch(unsigned c) { return c / FS_EPOCH; }
+__device__ __forceinline__ bool fs_rebuilds(unsigned c) { return c % FS_EPOCH == FS_EPOCH - 1; }
+
+// Adds tile t to the list of epoch e unless it is there (stamp e + 1).
+template <class Real>
+__device__ __forceinline__ void fs_add_tile(const FsArgs<Real> &s, unsigned t, unsigned e) {
+  if (atomicExch(s.stamp + t, e + 1u) != e + 1u)
+    s.tiles[e & 1u][atomicAdd(&s.cnt->n_tiles[e & 1u], 1u)] = t;
+}
+
+// Adds the tiles of the block-wide OR of the cells' masks around tile (bx, by,
+// bz) (wrapped; every thread of the block calls it) to the list of epoch e, in
+// no particular order: a cell's update depends only on the previous step's
+// values.
 template <class Real>
 __device__ __forceinline__ void fs_stamp_tiles(const FsArgs<Real> &s, unsigned bx, unsigned by,
-                                               unsigned bz, unsigned mask) {
+                                               unsigned bz, unsigned mask, unsigned e) {
   __shared__ unsigned block_mask;
   if (threadIdx.x == 0) block_mask = 0u;
   __syncthreads();
@@ -74,30 +82,32 @@ __device__ __forceinline__ void fs_stamp_tiles(const FsArgs<Real> &s, unsigned b
     const unsigned mx = (bx + s.ntx + k % 3 - 1) % s.ntx;
     const unsigned my = (by + s.nty + (k / 3) % 3 - 1) % s.nty;
     const unsigned mz = (bz + s.ntz + k / 9 - 1) % s.ntz;
-    const unsigned t = mx + s.ntx * (my + s.nty * mz), v = *s.stamp_ctr + 1u;
-    if (atomicExch(s.stamp + t, v) != v) s.next_tiles[atomicAdd(s.next_n_tiles, 1u)] = t;
+    fs_add_tile(s, mx + s.ntx * (my + s.nty * mz), e);
   }
   __syncthreads();  // block_mask is reset for the next tile only after every read
 }
 
-// Cells of this step's active tiles: block b takes list entries b, b +
+// Cells of step c's active tiles: block b takes list entries b, b +
 // gridDim.x, ...; thread k is cell (k % FS_TX, (k / FS_TX) % FS_TY, k /
 // (FS_TX FS_TY)) of the tile. cell(n, lx, ly, lz) runs for cells inside the
-// lattice; with MARK it returns the cell's tile mask (fs_tile_mask) and the
-// tiles of the block's masks are stamped for the next step (the trip count
-// is uniform in the block, so every thread reaches the barriers).
+// lattice; with MARK it returns the cell's tile mask (fs_tile_mask), and when
+// step c rebuilds the list the tiles of the block's masks are added to the next
+// one (the trip count is uniform in the block, so every thread reaches the
+// barriers).
 template <bool MARK, class Real, class F>
-__device__ __forceinline__ void fs_tile_loop(const FsArgs<Real> &s, F &&cell) {
-  const unsigned cnt = *s.n_tiles;
+__device__ __forceinline__ void fs_tile_loop(const FsArgs<Real> &s, unsigned c, F &&cell) {
+  const unsigned e = fs_epoch(c), cnt = s.cnt->n_tiles[e & 1u];
+  const uint32_t *list = s.tiles[e & 1u];
   const unsigned tx = threadIdx.x % FS_TX, ty = (threadIdx.x / FS_TX) % FS_TY,
                  tz = threadIdx.x / (FS_TX * FS_TY);
   for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const unsigned tile = s.tiles[i];
-    const unsigned bx = tile % s.ntx, r = tile / s.ntx, by = r % s.nty, bz = r / s.nty;
+    const unsigned tile = list[i];
+    const unsigned r = s.by_ntx.div(tile), bx = tile - r * s.ntx, bz = s.by_nty.div(r),
+                   by = r - bz * s.nty;
     const unsigned x = bx * FS_TX + tx, y = by * FS_TY + ty, z = bz * FS_TZ + tz;
     unsigned mask = 0u;
-    if (x < s.a.nx && y < s.a.ny && z < s.a.nz) mask = cell(x + s.a.nx * (y + s.a.ny * z), tx, ty, tz);
-    if (MARK) fs_stamp_tiles(s, bx, by, bz, mask);
+    if (x < s.a.nx && y < s.a.ny && z < s.a.nz) mask = cell(x, y, z, tx, ty, tz);
+    if (MARK && fs_rebuilds(c)) fs_stamp_tiles(s, bx, by, bz, mask, e + 1u);
   }
 }
 
@@ -114,10 +124,10 @@ __global__ void __launch_bounds__(FS_BLOCK) fs_seed_kernel(const FsArgs<Real> s)
   if (x < s.a.nx && y < s.a.ny && z < s.a.nz) {
     const unsigned n = x + s.a.nx * (y + s.a.ny * z);
     const uint32_t link = s.a.link ? s.a.link[n] : 0u;
-    const bool live = !(link >> 31) && s.type_old[n] != CELL_EMPTY;
+    const bool live = !(link >> 31) && s.type[n] != CELL_EMPTY;
     mask = fs_tile_mask(tx, ty, tz, live, live);
   }
-  fs_stamp_tiles(s, bx, by, bz, mask);
+  fs_stamp_tiles(s, bx, by, bz, mask, 0u);
 }
 
 // Flowchart step g, Eqs. eq:massmacro, eq:massevol, eq:deltamass:
@@ -125,51 +135,83 @@ __global__ void __launch_bounds__(FS_BLOCK) fs_seed_kernel(const FsArgs<Real> s)
 // either cell is liquid, (lambda(x) + lambda(x + c_q))/2 between two
 // interface cells, and no exchange with empty or solid cells. The colour
 // gradient field is the new liquid mass (0 in empty, wall_rho in solid cells).
+// The types of all neighbours are loaded together, then the populations of
+// nine directions at a time, whatever the types (every address is a cell): one
+// wait each instead of one per direction.
 template <class S>
-__global__ void __launch_bounds__(FS_BLOCK) fs_mass_kernel(const FsArgs<typename S::Real> s) {
+__global__ void __launch_bounds__(FS_BLOCK, sizeof(typename S::Real) == 4 ? 12 : 6)
+    fs_mass_kernel(const FsArgs<typename S::Real> s) {
   using Real = typename S::Real;
   using T = typename S::T;
   const StepArgs<Real> &a = s.a;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *s.any = 0u;
-    *s.next_n_tiles = 0u;
-    *s.stamp_ctr += 1u;  // read only by the later passes of this step
+  const unsigned c = s.cnt->step;
+  {
+    // the flags of the cells that the previous step converted; this step's
+    // lists start empty (the counts alternate: the previous ones are read here)
+    const unsigned last = (c & 1u) ^ 1u, k = s.cnt->n_near[last];
+    for (unsigned i = blockIdx.x * FS_BLOCK + threadIdx.x; i < k; i += gridDim.x * FS_BLOCK)
+      s.flag[s.near[i]] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      s.cnt->now = c;
+      s.cnt->n_flag = 0u;
+      s.cnt->n_near[c & 1u] = 0u;
+      if (c % FS_EPOCH == 0) s.cnt->n_tiles[(fs_epoch(c) + 1u) & 1u] = 0u;
+    }
   }
-  fs_tile_loop<false>(s, [&](unsigned n, unsigned, unsigned, unsigned) -> unsigned {
-  const uint32_t link = a.link ? __ldg(a.link + n) : 0u;
-  if (link >> 31) {
-    s.m_new[n] = Real(0);
-    s.rhohat_w[n] = a.wall_rho;
+  fs_tile_loop<false>(s, c, [&](unsigned x, unsigned y, unsigned z, unsigned, unsigned,
+                                unsigned) -> unsigned {
+    const unsigned n = x + a.nx * (y + a.ny * z), N = a.N;
+    const uint32_t link = a.link ? __ldg(a.link + n) : 0u;
+    const uint8_t t = s.type[n];
+    const Real lx = s.lam[n];
+    Real m = s.m[n];
+    if (link >> 31) {
+      s.rhohat_w[n] = a.wall_rho;
+      return 0u;
+    }
+    if (t == CELL_EMPTY) {
+      s.rhohat_w[n] = Real(0);
+      return 0u;
+    }
+    const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
+    const T *fin = static_cast<const T *>(a.f_in);
+    // directions that exchange, and those to an interface cell
+    uint32_t live = 0, face = 0;
+    Unroll<1, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const uint8_t ty = s.type[(long long)n + ahead_delta<q>(g)];
+      if (ty != CELL_EMPTY) live |= 1u << q;
+      if (ty == CELL_INTERFACE) face |= 1u << q;
+    });
+    Unroll<1, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      if ((faces_ahead(q) & g.onface & a.f_wall) || ((link >> opp(q)) & 1u)) live &= ~(1u << q);
+    });
+    if (t != CELL_INTERFACE) face = 0;
+    auto part = [&](auto first) {
+      constexpr int q0 = decltype(first)::value;
+      Real in[9], out[9];
+      Unroll<0, 9>::run([&](auto kc) {
+        constexpr int k = decltype(kc)::value, q = q0 + k;
+        in[k] = S::template ld_f<opp(q)>(fin + size_t(opp(q)) * N + (long long)n + ahead_delta<q>(g));
+        out[k] = S::template ld_f<q>(fin + size_t(q) * N + n);
+      });
+      Unroll<0, 9>::run([&](auto kc) {
+        constexpr int k = decltype(kc)::value, q = q0 + k;
+        if (!((live >> q) & 1u)) return;
+        // the equilibrium weights of q and opp(q) are equal, so deviations subtract
+        const Real diff = in[k] - out[k];
+        const Real w = ((face >> q) & 1u)
+                           ? Real(0.5) * (lx + s.lam[(long long)n + ahead_delta<q>(g)])
+                           : Real(1);
+        m += w * diff;
+      });
+    };
+    part(std::integral_constant<int, 1>{});
+    part(std::integral_constant<int, 10>{});
+    s.m[n] = m;
+    s.rhohat_w[n] = m;
     return 0u;
-  }
-  const uint8_t t = s.type_old[n];
-  if (t == CELL_EMPTY) {
-    s.m_new[n] = s.m_old[n];
-    s.rhohat_w[n] = Real(0);
-    return 0u;
-  }
-  const CellGeo g = cell_geo(n, a.nx, a.ny, a.nz);
-  const T *fin = static_cast<const T *>(a.f_in);
-  const unsigned N = a.N;
-  const Real lx = s.lam[n];
-  Real m = s.m_old[n];
-  Unroll<1, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const long long y = fs_neighbor<q>(g, n, link, a.f_wall);
-    if (y < 0) return;
-    const uint8_t ty = s.type_old[y];
-    if (ty == CELL_EMPTY) return;
-    // the equilibrium weights of q and opp(q) are equal, so deviations subtract
-    const Real diff = S::template ld_f<opp(q)>(fin + size_t(opp(q)) * N + y) -
-                      S::template ld_f<q>(fin + size_t(q) * N + n);
-    const Real w = (t == CELL_INTERFACE && ty == CELL_INTERFACE)
-                       ? Real(0.5) * (lx + s.lam[y])
-                       : Real(1);
-    m += w * diff;
-  });
-  s.m_new[n] = m;
-  s.rhohat_w[n] = m;
-  return 0u;
   });
 }
 
@@ -178,7 +220,10 @@ __global__ void __launch_bounds__(FS_BLOCK) fs_mass_kernel(const FsArgs<typename
 // equilempty: f_q = f^eq_q + f^eq_opp(q) - f~_opp(q)(x) at gas density 1 and
 // the cell's own V' (recovered from its post-collision populations; exact
 // without Darcy drag); moments, colour gradient, BGK collision with forcing
-// and surface tension; then lambda = m / rho and the fill/empty flags.
+// and surface tension; then lambda = m / rho, and the cells that fill or empty
+// are flagged and listed. Populations, colour-gradient field and types of the
+// neighbours are loaded together; the populations whose source turns out
+// empty are replaced.
 template <class S>
 __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
     fs_step_kernel(const FsArgs<typename S::Real> s) {
@@ -187,31 +232,40 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
   static_assert(std::is_same<T, Real>::value, "free surface: storage in the collision type");
   const StepArgs<Real> &a = s.a;
   const unsigned N = a.N;
-  fs_tile_loop<false>(s, [&](unsigned n, unsigned, unsigned, unsigned) -> unsigned {
+  const unsigned c = s.cnt->now;
+  if (blockIdx.x == 0 && threadIdx.x == 0) s.cnt->step = c + 1u;  // read by the next step's first pass
+  fs_tile_loop<true>(s, c, [&](unsigned x, unsigned y, unsigned z, unsigned lx, unsigned ly,
+                               unsigned lz) -> unsigned {
+  const unsigned n = x + a.nx * (y + a.ny * z);
   const uint32_t link = a.link ? __ldg(a.link + n) : 0u;
-  const uint8_t t = s.type_old[n];
-  s.flag_b[n] = FS_NONE;  // the re-typing pass rewrites it when some cell flags
-  if ((link >> 31) || t == CELL_EMPTY) {
-    s.flag_a[n] = FS_NONE;
-    return 0u;
-  }
-  const CellGeo g = cell_geo(n, a.nx, a.ny, a.nz);
+  const uint8_t t = s.type[n];
+  if ((link >> 31) || t == CELL_EMPTY) return 0u;
+  const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
   const T *__restrict__ fin = static_cast<const T *>(a.f_in);
   T *__restrict__ fout = static_cast<T *>(a.f_out);
   const Real eps = __ldg(a.eps + n);
-
+  const uint32_t bounce = bounce_mask(link, g.onface & a.f_wall);
+  Real d[Q];
+  Unroll<0, Q>::run([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const bool b = (bounce >> q) & 1u;
+    d[q] = S::template ld_f<q>(fin + size_t(b ? opp(q) : q) * N + (long long)n +
+                               (b ? 0 : src_delta<q>(g)));
+  });
   // sources that are empty cells
-  unsigned from_gas = 0;
+  uint32_t from_gas = 0;
   Unroll<1, Q>::run([&](auto qc) {
     constexpr int q = decltype(qc)::value;
-    if (fluid_class<q>(g, link, a.f_wall) == PULL_CELL &&
-        s.type_old[(long long)n + src_delta<q>(g)] == CELL_EMPTY)
-      from_gas |= 1u << q;
+    if (s.type[(long long)n + src_delta<q>(g)] == CELL_EMPTY) from_gas |= 1u << q;
   });
+  from_gas &= ~bounce;
+  FluidCollide<Real> fc;
+  fc.F[0] = fc.F[1] = fc.F[2] = Real(0);
+  if (a.A != Real(0)) colour_gradient(a.rhohat, n, g, a.f_wall, a.wall_rho, fc.F);
+  const Real mass = s.m[n];
   // f^eq_q - w_q at gas density 1 and the cell's own V' (time t), formed per
   // direction from u, 1/eps and u.u (a 19-value array held the kernel at 128
   // registers)
-  Real gu0 = Real(0), gu1 = Real(0), gu2 = Real(0), gie = Real(0), guu = Real(0);
   if (from_gas) {
     Real r = Real(0), j0 = Real(0), j1 = Real(0), j2 = Real(0);
     Unroll<0, Q>::run([&](auto qc) {
@@ -223,33 +277,23 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
       if (cz(q)) j2 += Real(cz(q)) * v;
     });
     const Real ir = Real(1) / (Real(1) + r);
-    const Real u0 = j0 * ir - Real(0.5) * eps * a.G[0];
-    const Real u1 = j1 * ir - Real(0.5) * eps * a.G[1];
-    const Real u2 = j2 * ir - Real(0.5) * eps * a.G[2];
-    gu0 = u0;
-    gu1 = u1;
-    gu2 = u2;
-    gie = Real(1) / eps;
-    guu = u0 * u0 + u1 * u1 + u2 * u2;
+    const Real gu0 = j0 * ir - Real(0.5) * eps * a.G[0];
+    const Real gu1 = j1 * ir - Real(0.5) * eps * a.G[1];
+    const Real gu2 = j2 * ir - Real(0.5) * eps * a.G[2];
+    const Real gie = Real(1) / eps;
+    const Real guu = gu0 * gu0 + gu1 * gu1 + gu2 * gu2;
+    auto ge = [&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const Real cu = Real(cx(q)) * gu0 + Real(cy(q)) * gu1 + Real(cz(q)) * gu2;
+      return wq<Real>(q) * (Real(3) * cu + Real(4.5) * gie * cu * cu - Real(1.5) * gie * guu);
+    };
+    Unroll<1, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      if ((from_gas >> q) & 1u)
+        d[q] = ge(qc) + ge(std::integral_constant<int, opp(q)>{}) -
+               S::template ld_f<opp(q)>(fin + size_t(opp(q)) * N + n);
+    });
   }
-  auto ge = [&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const Real cu = Real(cx(q)) * gu0 + Real(cy(q)) * gu1 + Real(cz(q)) * gu2;
-    return wq<Real>(q) * (Real(3) * cu + Real(4.5) * gie * cu * cu - Real(1.5) * gie * guu);
-  };
-  Real d[Q];
-  Unroll<0, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const int cls = fluid_class<q>(g, link, a.f_wall);
-    if (cls == PULL_BOUNCE) {
-      d[q] = S::template ld_f<opp(q)>(fin + size_t(opp(q)) * N + n);
-    } else if ((from_gas >> q) & 1u) {
-      d[q] = ge(qc) + ge(std::integral_constant<int, opp(q)>{}) -
-             S::template ld_f<opp(q)>(fin + size_t(opp(q)) * N + n);
-    } else {
-      d[q] = S::template ld_f<q>(fin + size_t(q) * N + (long long)n + src_delta<q>(g));
-    }
-  });
   Real drho = Real(0), j0 = Real(0), j1 = Real(0), j2 = Real(0);
   Unroll<0, Q>::run([&](auto qc) {
     constexpr int q = decltype(qc)::value;
@@ -263,9 +307,6 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
   const Real V[3] = {j0 * irho, j1 * irho, j2 * irho};
   const Real tau = a.tau;
   const Real nu = (tau - Real(0.5)) * Real(1.0 / 3.0);
-  FluidCollide<Real> fc;
-  fc.F[0] = fc.F[1] = fc.F[2] = Real(0);
-  if (a.A != Real(0)) colour_gradient(a.rhohat, n, g, a.f_wall, a.wall_rho, fc.F);
   velocity_solve<KM_NONE>(a.kinv, N, n, eps, nu, V, a.G, fc.Vp, fc.Fe);
   fc.drho = drho;
   fc.rho = rho;
@@ -289,8 +330,9 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
     S::template st_f<q>(fout + size_t(q) * N + n, v);
     rp += v;  // the stored value: FP32 / FP64 storage holds the collision type
   });
-  s.rho_post[n] = Real(1) + rp;
-  write_fields(a.fields, N, n, rho, fc.Vp, Real(0), nu);
+  const Real rho_post = Real(1) + rp;
+  s.rho_post[n] = rho_post;
+  if (a.fields) write_fields(a.fields, N, n, rho, fc.Vp, Real(0), nu);
   // the moments a new interface cell averages: it was empty, so each of its
   // live neighbours pulled from it in this pass
   if (from_gas) {
@@ -300,112 +342,154 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
     s.mom[3 * size_t(N) + n] = fc.Vp[2];
   }
   // flowchart step j, candidates: lambda > 1 + 1e-3 fills, lambda < -1e-3 empties
-  uint8_t flag = FS_NONE;
   if (t == CELL_INTERFACE) {
-    const Real lam = s.m_new[n] / rho;
-    if (lam > Real(1.001))
-      flag = FS_FILL;
-    else if (lam < Real(-0.001))
-      flag = FS_EMPTYING;
+    const Real lam = mass / rho;
+    s.lam[n] = mass / rho_post;
+    const uint8_t flag = lam > Real(1.001) ? FS_FILL : (lam < Real(-0.001) ? FS_EMPTYING : FS_NONE);
+    if (flag) {
+      s.flag[n] = flag;
+      s.flagged[atomicAdd(&s.cnt->n_flag, 1u)] = n;
+    }
   }
-  s.flag_a[n] = flag;
-  if (flag) atomicOr(s.any, 1u);
-  return 0u;
+  // the tiles the next list needs: every cell within one link of this one
+  return fs_rebuilds(c) ? fs_tile_mask(lx, ly, lz, true, true) : 0u;
   });
 }
 
-// Whether an emptying cell y is next to a filling one (then it stays an
-// interface cell), from the step's flags.
+// Sets bits of a cell's flag byte; returns the byte before.
 template <class Real>
-__device__ __forceinline__ bool fs_near_fill(const FsArgs<Real> &s, long long y) {
-  const StepArgs<Real> &a = s.a;
-  const uint32_t link = a.link ? a.link[y] : 0u;
-  const CellGeo g = cell_geo(unsigned(y), a.nx, a.ny, a.nz);
-  bool near = false;
+__device__ __forceinline__ unsigned fs_flag_or(const FsArgs<Real> &s, unsigned n, unsigned bits) {
+  const unsigned sh = 8u * (n & 3u);
+  return (atomicOr(reinterpret_cast<unsigned *>(s.flag) + (n >> 2), bits << sh) >> sh) & 0xffu;
+}
+// Component `axis` of c_q for the direction q = lane (0 beyond Q), from the
+// table packed in two bits each.
+__device__ __forceinline__ int fs_lane_c(unsigned lane, int axis) {
+  constexpr auto pack = [](int ax) constexpr {
+    unsigned long long p = 0;
+    for (int q = 0; q < Q; ++q)
+      p |= (unsigned long long)((ax == 0 ? cx(q) : ax == 1 ? cy(q) : cz(q)) + 1) << (2 * q);
+    return p;
+  };
+  constexpr unsigned long long px = pack(0), py = pack(1), pz = pack(2);
+  const unsigned long long p = axis == 0 ? px : axis == 1 ? py : pz;
+  return lane < Q ? int((p >> (2 * lane)) & 3u) - 1 : 0;
+}
+// a cell's settled flag: filled, emptied, or neither
+__device__ __forceinline__ bool fs_settled(unsigned b) {
+  return (b & FS_FILL) || ((b & FS_EMPTYING) && !(b & FS_CANCELLED));
+}
+
+// A mask over the directions q of test(y) for the neighbour y = n + c_q, without
+// those behind a wall face or solid. All neighbours are read before any is
+// used, whatever they are (the wrapped neighbour is always a cell).
+template <class F>
+__device__ __forceinline__ uint32_t fs_neighbors_that(unsigned n, const CellGeo &g, uint32_t link,
+                                                      unsigned f_wall, F &&test) {
+  uint32_t m = 0;
   Unroll<1, Q>::run([&](auto qc) {
     constexpr int q = decltype(qc)::value;
-    const long long y2 = fs_neighbor<q>(g, unsigned(y), link, a.f_wall);
-    if (y2 >= 0 && s.flag_a[y2] == FS_FILL) near = true;
+    if (test(unsigned((long long)n + ahead_delta<q>(g)))) m |= 1u << q;
   });
-  return near;
+  Unroll<1, Q>::run([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    if ((faces_ahead(q) & g.onface & f_wall) || ((link >> opp(q)) & 1u)) m &= ~(1u << q);
+  });
+  return m;
 }
 
-// New cell types, with the cancellation of an emptying cell next to a filling
-// one folded in (it reads the step's flags two links away): filled -> liquid,
-// emptied -> empty, empty next to a filled cell -> interface (flagged
-// FS_NEWCELL), liquid next to an emptied cell -> interface. flag_b gets each
-// cell's settled flag.
+// New cell types, by the cells the step flagged, a warp per flagged cell and a
+// lane per direction (few cells, each a chain of dependent loads and atomics:
+// as a thread per cell the 18 neighbours' chains ran one after another, 25 us
+// a step): an emptying cell next to a filling one is cancelled; filled ->
+// liquid, emptied -> empty, empty next to a filled cell -> interface (flagged
+// FS_NEWCELL), liquid next to an emptied cell -> interface. Every settled cell
+// lists itself and its neighbours. The types are changed in place: only
+// flagged cells become liquid or empty, an emptied one is never next to a
+// filled one, and the other changes depend on none of them, so no thread
+// misreads a type that another has changed.
 template <class Real>
-__global__ void __launch_bounds__(FS_BLOCK) fs_retype_kernel(const FsArgs<Real> s) {
+__global__ void __launch_bounds__(FS_LIST_BLOCK) fs_convert_kernel(const FsArgs<Real> s) {
   const StepArgs<Real> &a = s.a;
-  fs_tile_loop<false>(s, [&](unsigned n, unsigned, unsigned, unsigned) -> unsigned {
-  uint8_t t = s.type_old[n];
-  const uint32_t link = a.link ? a.link[n] : 0u;
-  if (*s.any != 0u && !(link >> 31)) {
-    uint8_t f = s.flag_a[n];
-    if (f == FS_EMPTYING && fs_near_fill(s, n)) f = FS_NONE;
-    if (f == FS_FILL) {
-      t = CELL_LIQUID;
-    } else if (f == FS_EMPTYING) {
-      t = CELL_EMPTY;
-    } else if (t == CELL_EMPTY || t == CELL_LIQUID) {
-      const CellGeo g = cell_geo(n, a.nx, a.ny, a.nz);
-      const bool empty = t == CELL_EMPTY;
-      bool hit = false;
-      Unroll<1, Q>::run([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        const long long y = fs_neighbor<q>(g, n, link, a.f_wall);
-        if (y < 0) return;
-        const uint8_t fy = s.flag_a[y];
-        if (empty ? fy == FS_FILL : (fy == FS_EMPTYING && !fs_near_fill(s, y))) hit = true;
-      });
-      if (hit) {
-        t = CELL_INTERFACE;
-        if (empty) f = FS_NEWCELL;
-      }
+  const unsigned c = s.cnt->now, k = s.cnt->n_flag, lane = threadIdx.x & 31u;
+  const int dx = fs_lane_c(lane, 0), dy = fs_lane_c(lane, 1), dz = fs_lane_c(lane, 2);
+  for (unsigned i = (blockIdx.x * FS_LIST_BLOCK + threadIdx.x) >> 5; i < k;
+       i += gridDim.x * FS_LIST_BLOCK >> 5) {
+    const unsigned n = s.flagged[i];
+    const bool fill = s.flag[n] & FS_FILL;
+    // this lane's neighbour n + c_lane (lane 0: the cell itself)
+    const unsigned yz = a.by_nx.div(n), x = n - yz * a.nx, z = a.by_ny.div(yz), y = yz - z * a.ny;
+    const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
+    const unsigned ahead = (dx > 0 ? 2u : 0u) | (dx < 0 ? 1u : 0u) | (dy > 0 ? 8u : 0u) |
+                           (dy < 0 ? 4u : 0u) | (dz > 0 ? 32u : 0u) | (dz < 0 ? 16u : 0u);
+    const unsigned b = n + unsigned((dx > 0 ? g.dxp : (dx < 0 ? g.dxm : 0)) +
+                                    (dy > 0 ? g.dyp : (dy < 0 ? g.dym : 0)) +
+                                    (dz > 0 ? g.dzp : (dz < 0 ? g.dzm : 0)));
+    bool there = lane < Q && !(ahead & g.onface & a.f_wall);
+    const unsigned fb = there ? s.flag[b] : 0u;
+    const uint8_t tb = there ? s.type[b] : uint8_t(CELL_INTERFACE);
+    if (there && a.link && (a.link[b] >> 31)) there = false;
+    if (!fill && __any_sync(0xffffffffu, there && lane > 0 && (fb & FS_FILL))) {
+      if (lane == 0) fs_flag_or(s, n, FS_CANCELLED);
+      continue;
     }
-    s.flag_b[n] = f;
+    bool fresh = false;
+    if (lane == 0) {
+      s.type[n] = fill ? CELL_LIQUID : CELL_EMPTY;
+    } else if (there) {
+      fresh = fill && tb == CELL_EMPTY;
+      if (fresh || (!fill && tb == CELL_LIQUID)) s.type[b] = CELL_INTERFACE;
+    }
+    const bool first =
+        there && !(fs_flag_or(s, b, FS_CLAIMED | (fresh ? unsigned(FS_NEWCELL) : 0u)) & FS_CLAIMED);
+    const unsigned won = __ballot_sync(0xffffffffu, first);
+    unsigned at = 0;
+    if (lane == 0 && won) at = atomicAdd(&s.cnt->n_near[c & 1u], unsigned(__popc(won)));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (first) s.near[at + __popc(won & ((1u << lane) - 1u))] = b;
   }
-  s.type_new[n] = t;
-  return 0u;
-  });
 }
 
 // New interface cells take f = f^eq(mean rho, mean V') of their liquid and
 // interface neighbours that are not new themselves (hydrodynamic
 // equilibrium, no mass); filled and emptied cells hand their excess mass (m -
 // rho, or m) in equal shares to the neighbours that are interface cells after
-// the re-typing (they keep it when there are none).
+// the re-typing (they keep it when there are none). The share waits in the
+// converted cell's liquid fraction, which only interface cells use.
 template <class S>
-__global__ void __launch_bounds__(FS_BLOCK) fs_newcell_kernel(const FsArgs<typename S::Real> s) {
+__global__ void __launch_bounds__(FS_LIST_BLOCK) fs_newcell_kernel(const FsArgs<typename S::Real> s) {
   using Real = typename S::Real;
   using T = typename S::T;
   const StepArgs<Real> &a = s.a;
   const unsigned N = a.N;
-  if (*s.any == 0u) return;
-  fs_tile_loop<false>(s, [&](unsigned n, unsigned, unsigned, unsigned) -> unsigned {
-  const uint8_t f = s.flag_b[n];
-  if (f == FS_NONE) return 0u;
+  const unsigned c = s.cnt->now, k = s.cnt->n_near[c & 1u];
+  for (unsigned i = blockIdx.x * FS_LIST_BLOCK + threadIdx.x; i < k; i += gridDim.x * FS_LIST_BLOCK) {
+  const unsigned n = s.near[i];
+  const unsigned f = s.flag[n];
+  if (!(f & FS_NEWCELL) && !fs_settled(f)) continue;
   const uint32_t link = a.link ? a.link[n] : 0u;
-  const CellGeo g = cell_geo(n, a.nx, a.ny, a.nz);
-  if (f == FS_NEWCELL) {
+  const unsigned yz = a.by_nx.div(n), x = n - yz * a.nx, z = a.by_ny.div(yz), y = yz - z * a.ny;
+  const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
+  if (f & FS_NEWCELL) {
     // density and V' of each neighbour as its collision in this step left
     // them (its post-collision populations carry the same moments: the
     // collision conserves mass, and without Darcy drag their momentum is
     // rho (V' + eps G / 2)); the loads of all neighbours are in flight together
+    const uint32_t old = fs_neighbors_that(n, g, link, a.f_wall, [&](unsigned y) {
+      return s.type[y] != CELL_EMPTY && !(s.flag[y] & FS_NEWCELL);
+    });
     Real rs = Real(0), u0 = Real(0), u1 = Real(0), u2 = Real(0);
-    int cnt = 0;
+    const int cnt = __popc(old);
     Unroll<1, Q>::run([&](auto qc) {
       constexpr int q = decltype(qc)::value;
-      const long long y = fs_neighbor<q>(g, n, link, a.f_wall);
-      if (y < 0) return;
-      const uint8_t ty = s.type_new[y];
-      if ((ty != CELL_LIQUID && ty != CELL_INTERFACE) || s.flag_b[y] == FS_NEWCELL) return;
-      rs += s.mom[y];
-      u0 += s.mom[size_t(N) + y];
-      u1 += s.mom[2 * size_t(N) + y];
-      u2 += s.mom[3 * size_t(N) + y];
-      ++cnt;
+      const unsigned y = unsigned((long long)n + ahead_delta<q>(g));
+      const Real m0 = s.mom[y], m1 = s.mom[size_t(N) + y], m2 = s.mom[2 * size_t(N) + y],
+                 m3 = s.mom[3 * size_t(N) + y];
+      const bool in = (old >> q) & 1u;
+      rs = in ? rs + m0 : rs;
+      u0 = in ? u0 + m1 : u0;
+      u1 = in ? u1 + m2 : u1;
+      u2 = in ? u2 + m3 : u2;
     });
     const Real ic = Real(1) / Real(cnt > 0 ? cnt : 1);
     const Real r = cnt > 0 ? rs * ic : Real(1);
@@ -424,67 +508,72 @@ __global__ void __launch_bounds__(FS_BLOCK) fs_newcell_kernel(const FsArgs<typen
       rp += dev;
     });
     s.rho_post[n] = Real(1) + rp;  // the density of the stored populations, for lambda
-    write_fields(a.fields, N, n, r, u, Real(0), (a.tau - Real(0.5)) / Real(3));
-    return 0u;
+    if (a.fields) write_fields(a.fields, N, n, r, u, Real(0), (a.tau - Real(0.5)) / Real(3));
+    continue;
   }
-  int cnt = 0;
-  Unroll<1, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const long long y = fs_neighbor<q>(g, n, link, a.f_wall);
-    if (y >= 0 && s.type_new[y] == CELL_INTERFACE) ++cnt;
-  });
+  const int cnt = __popc(fs_neighbors_that(
+      n, g, link, a.f_wall, [&](unsigned y) { return s.type[y] == CELL_INTERFACE; }));
   // a filled cell keeps m = rho: its post-collision density in the collision
   // type (the exported field is float)
   Real share = Real(0);
   if (cnt > 0) {
-    const Real m = s.m_new[n];
-    const Real excess = (f == FS_FILL) ? m - s.rho_post[n] : m;
+    const Real m = s.m[n];
+    const Real excess = (f & FS_FILL) ? m - s.rho_post[n] : m;
     share = excess / Real(cnt);
-    s.m_new[n] = m - excess;
+    s.m[n] = m - excess;
   }
-  s.share[n] = share;
-  return 0u;
-  });
+  s.lam[n] = share;
+  if (!(f & FS_FILL)) zero_fields(s.fields, N, n);  // emptied
+  }
 }
 
-// Excess mass arrives at interface cells; types settle; lambda = m / rho;
-// the next step's tiles are stamped and listed.
+// Excess mass arrives at the interface cells near a conversion; their lambda =
+// m / rho; the tiles around new interface cells join the list (the next one
+// when this step builds it).
 template <class S>
-__global__ void __launch_bounds__(FS_BLOCK) fs_finish_kernel(const FsArgs<typename S::Real> s) {
+__global__ void __launch_bounds__(FS_LIST_BLOCK) fs_finish_kernel(const FsArgs<typename S::Real> s) {
   using Real = typename S::Real;
   const StepArgs<Real> &a = s.a;
-  const unsigned N = a.N;
-  fs_tile_loop<true>(s, [&](unsigned n, unsigned lx, unsigned ly, unsigned lz) -> unsigned {
-  const uint32_t link = a.link ? a.link[n] : 0u;
-  if (link >> 31) {
-    s.lam[n] = Real(0);
-    return 0u;
-  }
-  const uint8_t tn = s.type_new[n];
-  Real m = s.m_new[n];
-  if (*s.any != 0u) {
-    if (tn == CELL_INTERFACE) {
-      const CellGeo g = cell_geo(n, a.nx, a.ny, a.nz);
-      Unroll<1, Q>::run([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        const long long y = fs_neighbor<q>(g, n, link, a.f_wall);
-        if (y < 0) return;
-        const uint8_t fy = s.flag_b[y];
-        if (fy == FS_FILL || fy == FS_EMPTYING) m += s.share[y];
+  const unsigned c = s.cnt->now, k = s.cnt->n_near[c & 1u];
+  const unsigned e = fs_epoch(c) + (fs_rebuilds(c) ? 1u : 0u);
+  for (unsigned i = blockIdx.x * FS_LIST_BLOCK + threadIdx.x; i < k; i += gridDim.x * FS_LIST_BLOCK) {
+    const unsigned n = s.near[i];
+    const uint8_t t = s.type[n];
+    const unsigned own = s.flag[n];
+    const uint32_t link = a.link ? a.link[n] : 0u;
+    const unsigned yz = a.by_nx.div(n), x = n - yz * a.nx, z = a.by_ny.div(yz), y = yz - z * a.ny;
+    const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
+    Real m = s.m[n];
+    const Real rho_post = s.rho_post[n];
+    const uint32_t from = fs_neighbors_that(n, g, link, a.f_wall,
+                                            [&](unsigned y) { return fs_settled(s.flag[y]); });
+    if (t != CELL_INTERFACE) continue;
+    Unroll<1, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      if ((from >> q) & 1u) m += s.lam[(long long)n + ahead_delta<q>(g)];
+    });
+    s.m[n] = m;
+    s.lam[n] = m / rho_post;
+    if (own & FS_NEWCELL) {
+      const unsigned bx = x / FS_TX, by = y / FS_TY, bz = z / FS_TZ;
+      // most of the tiles are listed: look at all of them together first, the
+      // atomics of the others run one after another
+      const unsigned mask = fs_tile_mask(x % FS_TX, y % FS_TY, z % FS_TZ, true, true);
+      unsigned missing = 0;
+      auto tile = [&](int j) {
+        const int mx = int(bx) + j % 3 - 1, my = int(by) + (j / 3) % 3 - 1, mz = int(bz) + j / 9 - 1;
+        const int X = int(s.ntx), Y = int(s.nty), Z = int(s.ntz);
+        return unsigned((mx < 0 ? mx + X : (mx >= X ? mx - X : mx)) +
+                        X * ((my < 0 ? my + Y : (my >= Y ? my - Y : my)) +
+                             Y * (mz < 0 ? mz + Z : (mz >= Z ? mz - Z : mz))));
+      };
+      Unroll<0, 27>::run([&](auto jc) {
+        constexpr int j = decltype(jc)::value;
+        if (s.stamp[tile(j)] != e + 1u) missing |= 1u << j;
       });
-      s.m_new[n] = m;
+      for (missing &= mask; missing; missing &= missing - 1u) fs_add_tile(s, tile(__ffs(missing) - 1), e);
     }
-    if (tn == CELL_EMPTY && s.flag_b[n] == FS_EMPTYING) zero_fields(a.fields, N, n);
   }
-  s.lam[n] = tn == CELL_LIQUID ? Real(1) : (tn == CELL_EMPTY ? Real(0) : m / s.rho_post[n]);
-  // both buffers of the type and the mass agree after the step, so a cell
-  // whose tile leaves the list keeps the same values under either parity
-  s.type_old[n] = tn;
-  s.m_old[n] = m;
-  // the next step needs every cell within one link of a liquid or interface
-  // cell, and each cell flagged in this step (its flags are cleared then)
-  return fs_tile_mask(lx, ly, lz, s.flag_b[n] != FS_NONE, tn != CELL_EMPTY);
-  });
 }
 
 }  // namespace lbgb

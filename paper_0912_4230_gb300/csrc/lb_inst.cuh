@@ -108,22 +108,18 @@ struct Instance {
                                                           partials);
     return cudaGetLastError();
   }
-  static cudaError_t fs_step(const void *args, unsigned grid, unsigned tile_blocks,
-                             cudaStream_t s) {
+  static cudaError_t fs_step(const void *args, unsigned grid, cudaStream_t s) {
     const FsArgs<Real> &f = *static_cast<const FsArgs<Real> *>(args);
     fs_mass_kernel<S><<<grid, FS_BLOCK, 0, s>>>(f);
     fs_step_kernel<S><<<grid, FS_BLOCK, 0, s>>>(f);
-    fs_retype_kernel<Real><<<grid, FS_BLOCK, 0, s>>>(f);
-    fs_newcell_kernel<S><<<grid, FS_BLOCK, 0, s>>>(f);
-    fs_finish_kernel<S><<<grid, FS_BLOCK, 0, s>>>(f);
-    (void)tile_blocks;
+    fs_convert_kernel<Real><<<FS_LIST_GRID, FS_LIST_BLOCK, 0, s>>>(f);
+    fs_newcell_kernel<S><<<FS_LIST_GRID, FS_LIST_BLOCK, 0, s>>>(f);
+    fs_finish_kernel<S><<<FS_LIST_GRID, FS_LIST_BLOCK, 0, s>>>(f);
     return cudaGetLastError();
   }
-  static cudaError_t fs_seed(const void *args, unsigned tiles, unsigned tile_blocks,
-                             cudaStream_t s) {
+  static cudaError_t fs_seed(const void *args, unsigned tiles, cudaStream_t s) {
     const FsArgs<Real> &f = *static_cast<const FsArgs<Real> *>(args);
     fs_seed_kernel<Real><<<tiles, FS_BLOCK, 0, s>>>(f);
-    (void)tile_blocks;
     return cudaGetLastError();
   }
   // The row-pipelined kernel is built for the coupled lattice (solute on),

@@ -54,13 +54,12 @@ struct StorageOps {
                           cudaStream_t s);
   cudaError_t (*totals)(PopView f, PopView h, const uint32_t *link, unsigned N, double *partials,
                         unsigned nblk, cudaStream_t s);
-  // one free-surface step, FsArgs<Real>*: five passes over the active tiles
-  // (grid blocks each; the last one also lists the next step's tiles);
-  // fs_seed stamps and lists the first step's tiles after initialisation (one
-  // block per tile; tile_blocks is unused). NULL when the storage format has
-  // no free-surface build
-  cudaError_t (*fs_step)(const void *fs_args, unsigned grid, unsigned tile_blocks, cudaStream_t s);
-  cudaError_t (*fs_seed)(const void *fs_args, unsigned tiles, unsigned tile_blocks, cudaStream_t s);
+  // one free-surface step, FsArgs<Real>*: two passes over the active tiles
+  // (grid blocks each) and three launches over the converting cells; fs_seed
+  // lists the first step's tiles after initialisation (one block per tile).
+  // NULL when the storage format has no free-surface build
+  cudaError_t (*fs_step)(const void *fs_args, unsigned grid, cudaStream_t s);
+  cudaError_t (*fs_seed)(const void *fs_args, unsigned tiles, cudaStream_t s);
   // row-pipelined step kernel (NULL when not built for this storage):
   // tma_config fills the dynamic shared memory, threads per block and
   // resident blocks per SM for a row of nx cells (returns false if it does
@@ -111,8 +110,8 @@ cudaError_t finish_sum(const double *partials, unsigned nblk, int k, double *out
 cudaError_t neighbors(const void *args, bool fp64, int lattice, int32_t *src, unsigned nblk,
                       cudaStream_t s);
 cudaError_t fs_init(unsigned N, const uint32_t *link, const uint8_t *type_in, const float *rho0,
-                    const float *lambda0, uint8_t *type0, uint8_t *type1, void *mass, void *lam,
-                    bool fp64, cudaStream_t s);
+                    const float *lambda0, uint8_t *type, void *mass, void *lam, bool fp64,
+                    cudaStream_t s);
 cudaError_t fs_totals(unsigned N, const uint32_t *link, const void *mass, double *partials,
                       bool fp64, cudaStream_t s);
 cudaError_t to_double(unsigned N, const void *src, double *dst, bool fp64, cudaStream_t s);
