@@ -182,6 +182,12 @@ void free_all(lb_ctx *c) {
   c->allocs.clear();
 }
 
+// Scratch of the flux slots' sum: the totals' partials, already summed by then
+// (NULL where they are too few).
+double *sum_scratch(const lb_ctx *c) {
+  return size_t(c->nblk) * 4 >= 2 * FINISH_BLOCKS ? c->partials : nullptr;
+}
+
 void *stage(lb_ctx *c, size_t bytes) {
   if (c->stage_bytes >= bytes) return c->stage;
   dev_free(c, c->stage);
@@ -1308,8 +1314,8 @@ int lb_reduce(lb_ctx *c, double *mass, double *solute, double *flux_in, double *
   else
     CK(c, c->ops->totals(f_view(c), c->solute ? h_view(c, 0) : PopView{},
                          c->has_solid ? c->link : nullptr, c->N, c->partials, c->nblk, c->stream));
-  CK(c, finish_sum(c->partials, c->fs ? c->nblk : totals_blocks(c->nblk), 2, out, c->stream));
-  CK(c, finish_sum(c->flux_slots, c->nwarps, 2, out + 2, c->stream));
+  CK(c, finish_sum(c->partials, totals_blocks(c->nblk), nullptr, out, c->stream));
+  CK(c, finish_sum(c->flux_slots, c->nwarps, sum_scratch(c), out + 2, c->stream));
   CK(c, cudaMemcpyAsync(tot, out, sizeof tot, cudaMemcpyDeviceToHost, c->stream));
   DevState st;
   CK(c, cudaMemcpyAsync(&st, c->state, sizeof st, cudaMemcpyDeviceToHost, c->stream));
@@ -1336,8 +1342,8 @@ int lb_species_state(lb_ctx *c, int32_t sp, float *C, double *totals, double *h)
     if (!out) return fail(c, LB_ENOMEM, "staging");
     CK(c, c->ops->totals(f_view(c), hv, c->has_solid ? c->link : nullptr, c->N, c->partials,
                          c->nblk, c->stream));
-    CK(c, finish_sum(c->partials, totals_blocks(c->nblk), 2, out, c->stream));
-    CK(c, finish_sum(c->flux_slots + size_t(sp) * c->nwarps * 2, c->nwarps, 2, out + 2,
+    CK(c, finish_sum(c->partials, totals_blocks(c->nblk), nullptr, out, c->stream));
+    CK(c, finish_sum(c->flux_slots + size_t(sp) * c->nwarps * 2, c->nwarps, sum_scratch(c), out + 2,
                      c->stream));
     double tot[4];
     CK(c, cudaMemcpyAsync(tot, out, sizeof tot, cudaMemcpyDeviceToHost, c->stream));

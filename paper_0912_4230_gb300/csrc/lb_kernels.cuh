@@ -1362,7 +1362,9 @@ __global__ void __launch_bounds__(BLOCK) rhohat_kernel(const StepArgs<typename S
 }
 
 // ------------------------------------------------------------------------
-// Initialisation (flowchart step c): f = f^eq, h = h^eq.
+// Initialisation (flowchart step c): f = f^eq, h = h^eq. The first step
+// writes the other buffer of every updated cell; only the cells that no step
+// writes (solid, empty) are set in both.
 // ------------------------------------------------------------------------
 template <class Real>
 struct InitArgs {
@@ -1379,7 +1381,7 @@ __global__ void __launch_bounds__(BLOCK) init_kernel(const StepArgs<typename S::
   const unsigned N = a.N;
   if (n >= N) return;
   T *fout = static_cast<T *>(a.f_out);
-  T *fout2 = static_cast<T *>(const_cast<void *>(a.f_in));  // both buffers get the same state
+  T *fout2 = static_cast<T *>(const_cast<void *>(a.f_in));
   const bool solid = a.link && (__ldg(a.link + n) >> 31);
   const bool empty = in.type && in.type[n] == CELL_EMPTY;
   if constexpr (S::kShift && SOLUTE) {
@@ -1473,17 +1475,14 @@ __global__ void __launch_bounds__(BLOCK) init_kernel(const StepArgs<typename S::
     const __half2 r2 = __floats2half2_rn(dsum, hsum);
     const float2 R = __half22float2(r2);
     using T2 = typename S::T2;
-    T2 *p1 = static_cast<T2 *>(a.f_out) + n;
     T2 *p0 = static_cast<T2 *>(const_cast<void *>(a.f_in)) + n;
     const Real sc = Real(S::kScale);
     Unroll<0, Q>::run([&](auto qc) {
       constexpr int q = decltype(qc)::value;
       const Real gf = sc * (devs[q] * Real(inv_wq(q)) - R.x);
       const Real gh = sc * (hs[q] * Real(inv_wq(q)) - R.y);
-      S::st2(p1 + size_t(q) * N, gf, gh);
       S::st2(p0 + size_t(q) * N, gf, gh);
     });
-    reinterpret_cast<__half2 *>(a.rf_out)[n] = r2;
     reinterpret_cast<__half2 *>(const_cast<float *>(a.rf_in))[n] = r2;
     if (a.fields) write_fields(a.fields, N, n, rho, u, C, (tau - Real(0.5)) / Real(3));
     return;
@@ -1491,13 +1490,9 @@ __global__ void __launch_bounds__(BLOCK) init_kernel(const StepArgs<typename S::
   Unroll<0, Q>::run([&](auto qc) {
     constexpr int q = decltype(qc)::value;
     const Real v = devs[q] - (S::kShift ? wq<Real>(q) * dsum : Real(0));
-    S::template st_f<q>(fout + size_t(q) * N + n, v);
     S::template st_f<q>(fout2 + size_t(q) * N + n, v);
   });
-  if constexpr (S::kShift) {
-    a.rf_out[n] = float(dsum);
-    const_cast<float *>(a.rf_in)[n] = float(dsum);
-  }
+  if constexpr (S::kShift) const_cast<float *>(a.rf_in)[n] = float(dsum);
   if (SOLUTE) {
     const Real vs0 = u[0] + a.geps[n], vs1 = u[1] + a.geps[N + n], vs2 = u[2] + a.geps[2 * size_t(N) + n];
     Real hs[Q];
@@ -1511,13 +1506,9 @@ __global__ void __launch_bounds__(BLOCK) init_kernel(const StepArgs<typename S::
     Unroll<0, Q>::run([&](auto qc) {
       constexpr int q = decltype(qc)::value;
       const Real h = hs[q] - (S::kShift ? wq<Real>(q) * hsum : Real(0));
-      S::template st_h<q>(static_cast<T *>(a.h_out) + size_t(q) * N + n, h);
       S::template st_h<q>(const_cast<T *>(static_cast<const T *>(a.h_in)) + size_t(q) * N + n, h);
     });
-    if constexpr (S::kShift) {
-      a.rh_out[n] = float(hsum);
-      const_cast<float *>(a.rh_in)[n] = float(hsum);
-    }
+    if constexpr (S::kShift) const_cast<float *>(a.rh_in)[n] = float(hsum);
   }
   if (a.fields) write_fields(a.fields, N, n, rho, u, C, (tau - Real(0.5)) / Real(3));
 }
@@ -1587,6 +1578,22 @@ __global__ void __launch_bounds__(BLOCK) totals_kernel(const PopView f, const Po
   double m = 0.0, s = 0.0;
   for (unsigned n = blockIdx.x * BLOCK + threadIdx.x; n < N; n += gridDim.x * BLOCK) {
     if (link && (link[n] >> 31)) continue;
+    if constexpr (S::kShift)
+      if (f.ref_pair && h.p == f.p) {
+        // the paired layout: f and species 0 in one load (half of each 4-byte
+        // pair was loaded twice, 139 us at 160^3 FP16)
+        using T2 = typename S::T2;
+        Real a = Real(0), b = Real(0);
+        Unroll<0, Q>::run([&](auto qc) {
+          constexpr int q = decltype(qc)::value;
+          const T2 p = static_cast<const T2 *>(f.p)[size_t(q) * N + n];
+          a += S::template cv_f<q>(p.x);
+          b += S::template cv_h<q>(p.y);
+        });
+        m += 1.0 + pop_ref(f, n) + double(a);
+        s += pop_ref(h, n) + double(b);
+        continue;
+      }
     Real a = Real(0);
     Unroll<0, Q>::run([&](auto qc) {
       constexpr int q = decltype(qc)::value;
@@ -1623,9 +1630,9 @@ __global__ void __launch_bounds__(BLOCK) totals_kernel(const PopView f, const Po
   }
 }
 
-// Fixed-order sum of nblk x K partials by one block of FINISH_THREADS
-// threads (thread t sums partials t, t + FINISH_THREADS, ..., then a fixed
-// tree), so the result does not depend on timing.
+// Fixed-order sum of nblk x K partials by blocks of FINISH_THREADS threads
+// into a set of K sums per block (thread t of the launch sums partials t, t +
+// threads, ..., then a fixed tree), so the result does not depend on timing.
 constexpr int FINISH_THREADS = 1024;
 template <int K>
 __global__ void __launch_bounds__(FINISH_THREADS) finish_sum_kernel(const double *partials,
@@ -1633,7 +1640,8 @@ __global__ void __launch_bounds__(FINISH_THREADS) finish_sum_kernel(const double
   __shared__ double sh[FINISH_THREADS][K];
   double acc[K];
   for (int k = 0; k < K; ++k) acc[k] = 0.0;
-  for (unsigned b = threadIdx.x; b < nblk; b += FINISH_THREADS)
+  for (unsigned b = blockIdx.x * FINISH_THREADS + threadIdx.x; b < nblk;
+       b += gridDim.x * FINISH_THREADS)
     for (int k = 0; k < K; ++k) acc[k] += partials[size_t(b) * K + k];
   for (int k = 0; k < K; ++k) sh[threadIdx.x][k] = acc[k];
   __syncthreads();
@@ -1642,7 +1650,7 @@ __global__ void __launch_bounds__(FINISH_THREADS) finish_sum_kernel(const double
       for (int k = 0; k < K; ++k) sh[threadIdx.x][k] += sh[threadIdx.x + s][k];
     __syncthreads();
   }
-  if (threadIdx.x < K) out[threadIdx.x] = sh[0][threadIdx.x];
+  if (threadIdx.x < K) out[blockIdx.x * K + threadIdx.x] = sh[0][threadIdx.x];
 }
 
 template <class Real>

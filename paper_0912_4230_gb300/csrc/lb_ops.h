@@ -106,7 +106,11 @@ struct SetupArgs {
 };
 cudaError_t setup_scan(const SetupArgs &a, bool fp64, cudaStream_t s);
 cudaError_t setup_fields(const SetupArgs &a, bool fp64, cudaStream_t s);
-cudaError_t finish_sum(const double *partials, unsigned nblk, int k, double *out, cudaStream_t s);
+// the sum of nblk pairs of doubles into out, in a fixed order; scratch (may be
+// NULL) holds 2 FINISH_BLOCKS doubles
+constexpr unsigned FINISH_BLOCKS = 64;
+cudaError_t finish_sum(const double *partials, unsigned nblk, double *scratch, double *out,
+                       cudaStream_t s);
 cudaError_t neighbors(const void *args, bool fp64, int lattice, int32_t *src, unsigned nblk,
                       cudaStream_t s);
 cudaError_t fs_init(unsigned N, const uint32_t *link, const uint8_t *type_in, const float *rho0,

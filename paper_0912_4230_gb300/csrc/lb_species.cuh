@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(BLOCK) species_init_kernel(const StepArgs<type
   for (int sp = 1; sp < a.species; ++sp) {
     const size_t off = size_t(sp - a.paired) * Q * N;
     T *h0 = const_cast<T *>(static_cast<const T *>(a.h_in)) + off + n;
-    T *h1 = static_cast<T *>(a.h_out) + off + n;
+    T *h1 = static_cast<T *>(a.h_out) + off + n;  // (solid cells only)
     const Real C = solid ? Real(0) : Real(C0[size_t(sp) * N + n]);
     const Real ratio = a.spec[16 + sp];
     const Real vs0 = Real(u0[3 * size_t(n)]) + ratio * a.geps[n];
@@ -41,11 +41,11 @@ __global__ void __launch_bounds__(BLOCK) species_init_kernel(const StepArgs<type
       constexpr int q = decltype(qc)::value;
       const Real h = hs[q] - (S::kShift ? wq<Real>(q) * hsum : Real(0));
       S::template st_h<q>(h0 + size_t(q) * N, h);
-      S::template st_h<q>(h1 + size_t(q) * N, h);
+      if (solid) S::template st_h<q>(h1 + size_t(q) * N, h);
     });
     if constexpr (S::kShift) {
       const_cast<float *>(a.rh_in)[size_t(sp) * N + n] = float(hsum);
-      a.rh_out[size_t(sp) * N + n] = float(hsum);
+      if (solid) a.rh_out[size_t(sp) * N + n] = float(hsum);
     }
     if (a.fields) a.fields[(5 + size_t(sp)) * N + n] = solid ? 0.0f : float(C);
   }
