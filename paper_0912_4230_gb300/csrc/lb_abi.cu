@@ -100,9 +100,6 @@ struct lb_ctx {
   unsigned *stamp = nullptr;
   FsCount *fs_cnt = nullptr;
   unsigned ntx = 0, nty = 0, ntz = 0, fs_grid = 0;
-  // table of lb_step_batch calls led by this context
-  void *batch_tab = nullptr;
-  size_t batch_tab_bytes = 0;
   // reusable staging for lb_init and the FP64 population exchange
   void *stage = nullptr;
   size_t stage_bytes = 0;
@@ -271,7 +268,7 @@ struct Layout {
   size_t kinv, flux_slots;
   size_t create_stage;   // inputs of lb_create, released before it returns
   size_t init_stage;     // inputs of lb_init, kept for later staging
-  size_t batch_share;    // this lattice's part of a batch work list (lb_step_batch)
+  size_t batch_share;    // allowance for lb_step_batch (8 bytes per block of a launch by rows)
 };
 
 Layout layout_of(const lb_domain &dom, const lb_params &prm, const StorageOps &ops, int k_rows,
@@ -323,7 +320,7 @@ Layout layout_of(const lb_domain &dom, const lb_params &prm, const StorageOps &o
   L.create_stage = N * 4 + (k_rows ? 6 * N * 4 : 0) + N + 64 + 256;
   L.init_stage = N * 4 * (4 + S) + (f_scale ? size_t(Q) * N * 4 : 0) + N * 4 + N + 256;
   dim3 g, b;
-  row_shape(dom, &g, &b);  // at least as many blocks as any other shape by default
+  row_shape(dom, &g, &b);
   L.batch_share = size_t(g.x) * g.y * g.z * sizeof(uint64_t);
   return L;
 }
@@ -1048,12 +1045,6 @@ int lb_set_graphs(lb_ctx *c, int32_t enable) {
 
 namespace {
 
-// A lattice's blocks of STEP_BLOCK threads in a batch work list.
-dim3 batch_grid(const lb_ctx *c) {
-  if (!c->linear) return c->sgrid;
-  return dim3((c->N + STEP_BLOCK - 1) / STEP_BLOCK, 1, 1);
-}
-
 template <class Real>
 int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   lb_ctx *c0 = ctxs[0];
@@ -1074,35 +1065,7 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
     shared.clear();
   }
   const int ns = int(shared.size());
-  std::vector<unsigned> begin(size_t(ns) + 1);
-  unsigned total = 0;
-  for (int j = 0; j < ns; ++j) {
-    const dim3 g = batch_grid(ctxs[shared[j]]);
-    begin[j] = total;
-    total += g.x * g.y * g.z;
-  }
-  begin[ns] = total;
   cudaStream_t s = c0->stream;
-  const uint64_t *d_work = nullptr;
-  if (ns > 0) {
-    std::vector<uint64_t> work(total);
-    for (int j = 0; j < ns; ++j) {
-      const dim3 g = batch_grid(ctxs[shared[j]]);
-      unsigned b = begin[j];
-      for (unsigned bz = 0; bz < g.z; ++bz)
-        for (unsigned by = 0; by < g.y; ++by)
-          for (unsigned bx = 0; bx < g.x; ++bx) work[b++] = batch_item(unsigned(j), bx, by, bz);
-    }
-    const size_t wbytes = work.size() * sizeof(uint64_t);
-    if (c0->batch_tab_bytes < wbytes) {
-      dev_free(c0, c0->batch_tab);
-      c0->batch_tab = dev_alloc(c0, wbytes);
-      c0->batch_tab_bytes = c0->batch_tab ? wbytes : 0;
-      if (!c0->batch_tab) return fail(c0, LB_ENOMEM, "batch work list");
-    }
-    d_work = static_cast<const uint64_t *>(c0->batch_tab);
-    CK(c0, cudaMemcpyAsync(c0->batch_tab, work.data(), wbytes, cudaMemcpyHostToDevice, s));
-  }
   // one table per launch of at most BATCH_MAX lattices, filled on the host
   // for every step (the launch copies it into its parameter space)
   std::unique_ptr<BatchTable<Real>> tab(new BatchTable<Real>());
@@ -1121,18 +1084,17 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
     }
     for (int g0 = 0; g0 < ns; g0 += BATCH_MAX) {
       const int g1 = std::min(ns, g0 + BATCH_MAX);
-      std::memset(tab.get(), 0, sizeof(BatchTable<Real>));
+      unsigned blocks = 0;
       for (int j = g0; j < g1; ++j) {
         lb_ctx *c = ctxs[shared[j]];
-        BatchEntry<Real> &e = tab->e[j - g0];
-        step_args(c, e.a);
-        e.gx = batch_grid(c).x;
-        e.gy = batch_grid(c).y;
-        e.bx = c->linear ? unsigned(STEP_BLOCK) : c->sblock.x;
+        step_args(c, tab->a[j - g0]);
+        tab->a[j - g0].linear = 1;
+        tab->begin[j - g0] = blocks;
+        blocks += (c->N + STEP_BLOCK - 1) / STEP_BLOCK;
       }
-      const unsigned blocks = begin[g1] - begin[g0];
-      CK(c0, c0->ops->batch_step(c0->kmode, c0->solute, tab.get(), d_work, unsigned(g0),
-                                 begin[g0], begin[g1], std::min(blocks, wave), st));
+      tab->n = g1 - g0;
+      tab->begin[tab->n] = blocks;
+      CK(c0, c0->ops->batch_step(c0->kmode, c0->solute, tab.get(), std::min(blocks, wave), st));
     }
     return int(LB_OK);
   };
@@ -1142,11 +1104,10 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
       ctxs[i]->cur = 1 - ctxs[i]->cur;
     }
   };
-  // the graph of a step pair is valid for this set of lattices in this order,
-  // these parities and this work list
+  // the graph of a step pair is valid for this set of lattices in this order
+  // and these parities
   bool safe = true;
   std::vector<uint64_t> key;
-  key.push_back(uint64_t(reinterpret_cast<uintptr_t>(d_work)));
   for (int i = 0; i < n; ++i) {
     safe = safe && graph_safe(ctxs[i]);
     key.push_back(ctxs[i]->serial * 2 + uint64_t(ctxs[i]->cur));

@@ -217,13 +217,12 @@ struct Instance {
     });
     return cudaGetLastError();
   }
-  static cudaError_t batch_step(int kmode, bool solute, const void *tab, const uint64_t *work,
-                                unsigned d_begin, unsigned vb_begin, unsigned vb_end,
-                                unsigned grid, cudaStream_t s) {
+  static cudaError_t batch_step(int kmode, bool solute, const void *tab, unsigned grid,
+                                cudaStream_t s) {
     const BatchTable<Real> &t = *static_cast<const BatchTable<Real> *>(tab);
     dispatch_mode(kmode, solute, [&](auto km, auto sol) {
       batched_step_kernel<S, decltype(km)::value, decltype(sol)::value>
-          <<<grid, STEP_BLOCK, 0, s>>>(t, work, d_begin, vb_begin, vb_end);
+          <<<grid, STEP_BLOCK, 0, s>>>(t);
     });
     return cudaGetLastError();
   }

@@ -76,9 +76,8 @@ struct StorageOps {
   cudaError_t (*pipe_step)(int kmode, bool solute, const void *args, unsigned grid, unsigned bx,
                            size_t smem, unsigned gxr, unsigned items, cudaStream_t s);
   // one batched step: tab is a host BatchTable<Real> (passed by value in the
-  // launch), work the device work list (batch_item descriptors)
-  cudaError_t (*batch_step)(int kmode, bool solute, const void *tab, const uint64_t *work,
-                            unsigned d_begin, unsigned vb_begin, unsigned vb_end, unsigned grid,
+  // launch)
+  cudaError_t (*batch_step)(int kmode, bool solute, const void *tab, unsigned grid,
                             cudaStream_t s);
 };
 
