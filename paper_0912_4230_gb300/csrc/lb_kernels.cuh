@@ -554,81 +554,6 @@ __device__ __forceinline__ void warp_reductions(const StepArgs<Real> &a, unsigne
   if (a.reduce) finite_check(a.state, drho, sC);
 }
 
-// Stream of a cell on a pressure or velocity face of the fluid lattice into
-// d[] (f_q - w_q). The face rules need the cell's own post-collision density
-// and velocity, from its 19 populations of the input buffer: a population
-// entering through a pressure face is -f~_qbar + 2 w_q rho_b (1 + 4.5
-// (c_q.u)^2/eps - 1.5 u.u/eps) with rho_b = 3 eps P_face; through a velocity
-// face f~_qbar + 6 w_q rho (c_q . u_face). Kept out of line: face cells are
-// few, and the hot path keeps its registers.
-template <class Real>
-struct Pops {
-  Real v[Q];
-};
-
-template <class S>
-__device__ __noinline__ Pops<typename S::Real> gather_open_faces(
-    const StepArgs<typename S::Real> &a, const CellGeo &g, unsigned n, uint32_t link) {
-  using Real = typename S::Real;
-  Pops<Real> d;
-  using T = typename S::T;
-  const unsigned N = a.N;
-  const T *__restrict__ fb = static_cast<const T *>(a.f_in) + n;
-  Real own[Q];
-  Real r = Real(0), j0 = Real(0), j1 = Real(0), j2 = Real(0);
-  // 16-bit storage: f_q - w_q = w_q (remainder + reference), from the pairs
-  // of the paired layout or the plain rows
-  auto ld_src = [&](auto qc, int off, int roff) -> Real {
-    constexpr int q = decltype(qc)::value;
-    if constexpr (S::kShift) {
-      if (a.paired)
-        return wq<Real>(q) * (S::ld2(static_cast<const typename S::T2 *>(a.f_in) + n + off).x +
-                              ld_ref2(a.rf_in + (long long)n + roff).x);
-      return S::template ld_f<q>(fb + off) + wq<Real>(q) * __ldg(a.rf_in + (long long)n + roff);
-    } else {
-      return S::template ld_f<q>(fb + off);
-    }
-  };
-  Unroll<0, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const Real v = ld_src(qc, int(q * N), 0);
-    own[q] = v;
-    r += v;
-    if (cx(q)) j0 += Real(cx(q)) * v;
-    if (cy(q)) j1 += Real(cy(q)) * v;
-    if (cz(q)) j2 += Real(cz(q)) * v;
-  });
-  const Real rho = Real(1) + r, irho = rcp(rho);
-  const Real u0 = j0 * irho, u1 = j1 * irho, u2 = j2 * irho;
-  const Real ie = rcp(__ldg(a.eps + n)), eps = __ldg(a.eps + n);
-  const Real uu = u0 * u0 + u1 * u1 + u2 * u2;
-  Unroll<0, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const int cls = fluid_class_open<q>(g, link, a.f_wall, a.f_vel, a.f_press);
-    Real v;
-    if (cls == PULL_BOUNCE) {
-      v = own[opp(q)];
-    } else if (cls == PULL_PRESSURE) {
-      // rho_b - 1 from 3P = hi + lo with one rounding of eps hi - 1
-      const int fi = crossed_face<q>(g, a.f_press);
-      const Real rbm1 = fma(eps, __ldg(a.face + fi), Real(-1)) + eps * __ldg(a.face + 24 + fi);
-      const Real rb = Real(1) + rbm1;
-      const Real cu = Real(cx(q)) * u0 + Real(cy(q)) * u1 + Real(cz(q)) * u2;
-      const Real e = wq<Real>(q) * (rbm1 + rb * (Real(4.5) * ie * cu * cu - Real(1.5) * ie * uu));
-      v = Real(2) * e - own[opp(q)];
-    } else if (cls == PULL_VELOCITY) {
-      const Real *uf = a.face + 6 + 3 * crossed_face<q>(g, a.f_vel);
-      const Real cub = Real(cx(q)) * __ldg(uf) + Real(cy(q)) * __ldg(uf + 1) +
-                       Real(cz(q)) * __ldg(uf + 2);
-      v = own[opp(q)] + Real(6) * wq<Real>(q) * rho * cub;
-    } else {
-      v = ld_src(qc, int(q * N) + src_delta<q>(g), src_delta<q>(g));
-    }
-    d.v[q] = v;
-  });
-  return d;
-}
-
 // Reciprocals up to the velocity: with 16-bit storage the correctly rounded
 // one. In a tight medium the drag balances the body force, F_e is the small
 // difference of the two, and its FP32 rounding is as large as the last bit of
@@ -981,6 +906,71 @@ __device__ __forceinline__ uint32_t bounce_mask(uint32_t link, unsigned walls_on
   return m;
 }
 
+// The rules of pressure and velocity faces for the directions of fprs and
+// fvel, whose d[q] holds the cell's own f~_qbar: a population entering through a
+// pressure face is -f~_qbar + 2 w_q rho_b (1 + 4.5 (c_q.u)^2/eps - 1.5 u.u/eps)
+// with rho_b = 3 eps P_face and u the velocity of the cell's own post-collision
+// populations; through a velocity face f~_qbar + 6 w_q rho (c_q . u_face), rho
+// their density. 16-bit storage: d per unit weight. Out of line: face cells
+// are few, and the hot path keeps its registers.
+template <class Real>
+struct Pops {
+  Real v[Q];
+};
+
+template <class S>
+__device__ __noinline__ Pops<typename S::Real> open_face_rules(
+    const StepArgs<typename S::Real> &a, const CellGeo &g, unsigned n, typename S::Real eps,
+    uint32_t fvel, uint32_t fprs, Pops<typename S::Real> d) {
+  using Real = typename S::Real;
+  using T = typename S::T;
+  const unsigned N = a.N;
+  Real r = Real(0), j0 = Real(0), j1 = Real(0), j2 = Real(0);
+  Unroll<0, Q>::run([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    Real v;  // the own f~_q - w_q
+    if constexpr (S::kShift) {
+      if (a.paired)
+        v = wq<Real>(q) * (S::ld2(static_cast<const typename S::T2 *>(a.f_in) + size_t(q) * N + n).x +
+                           ld_ref2(a.rf_in + n).x);
+      else
+        v = S::template ld_f<q>(static_cast<const T *>(a.f_in) + size_t(q) * N + n) +
+            wq<Real>(q) * __ldg(a.rf_in + n);
+    } else {
+      v = S::template ld_f<q>(static_cast<const T *>(a.f_in) + size_t(q) * N + n);
+    }
+    r += v;
+    if (cx(q)) j0 += Real(cx(q)) * v;
+    if (cy(q)) j1 += Real(cy(q)) * v;
+    if (cz(q)) j2 += Real(cz(q)) * v;
+  });
+  const Real rho = Real(1) + r, irho = rcp(rho);
+  const Real u0 = j0 * irho, u1 = j1 * irho, u2 = j2 * irho;
+  const Real ie = rcp(eps);
+  const Real uu = u0 * u0 + u1 * u1 + u2 * u2;
+  Unroll<0, Q>::run([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const Real own = S::kShift ? d.v[q] * wq<Real>(q) : d.v[q];
+    Real v = own;
+    if ((fprs >> q) & 1u) {
+      // rho_b - 1 from 3P = hi + lo with one rounding of eps hi - 1
+      const int fi = crossed_face<q>(g, a.f_press);
+      const Real rbm1 = fma(eps, __ldg(a.face + fi), Real(-1)) + eps * __ldg(a.face + 24 + fi);
+      const Real rb = Real(1) + rbm1;
+      const Real cu = Real(cx(q)) * u0 + Real(cy(q)) * u1 + Real(cz(q)) * u2;
+      const Real e = wq<Real>(q) * (rbm1 + rb * (Real(4.5) * ie * cu * cu - Real(1.5) * ie * uu));
+      v = Real(2) * e - own;
+    } else if ((fvel >> q) & 1u) {
+      const Real *uf = a.face + 6 + 3 * crossed_face<q>(g, a.f_vel);
+      const Real cub = Real(cx(q)) * __ldg(uf) + Real(cy(q)) * __ldg(uf + 1) +
+                       Real(cz(q)) * __ldg(uf + 2);
+      v = own + Real(6) * wq<Real>(q) * rho * cub;
+    }
+    d.v[q] = S::kShift ? v * Real(inv_wq(q)) : v;
+  });
+  return d;
+}
+
 // One step of a cell from global memory: stream f (and h), moments,
 // viscosity, colour gradient, V' and the Darcy force, fluid and solute
 // collision, store; accumulates the cell's flux and totals. 16-bit storage
@@ -1082,57 +1072,72 @@ __device__ __forceinline__ void update_cell(const StepArgs<typename S::Real> &a,
       });
     }
   } else {
-    // on inlet, outlet, pressure or velocity faces
-    if (((FEAT & FEAT_OPEN) != 0) && (g.onface & (a.f_press | a.f_vel))) {
-      const Pops<Real> o = gather_open_faces<S>(a, g, n, link);
+    // On inlet, outlet, pressure or velocity faces: the class of every
+    // direction as masks (walls take precedence, then velocity, then pressure;
+    // for the solute inlets, then outlets), so that all loads go out together
+    // without a branch per direction. In a small lattice these few warps are
+    // the longest chain of a step.
+    statics();
+    const uint32_t solid = link & 0x7ffffu;
+    const uint32_t fw = bounce_mask(0u, g.onface & a.f_wall);
+    uint32_t fvel = 0, fprs = 0;
+    if constexpr ((FEAT & FEAT_OPEN) != 0) {
+      fvel = bounce_mask(0u, g.onface & a.f_vel) & ~fw;
+      fprs = bounce_mask(0u, g.onface & a.f_press) & ~(fw | fvel);
+    }
+    // the own population of the opposite direction: bounce-back, and what the
+    // pressure and velocity rules start from
+    const uint32_t fown = fw | fvel | fprs | solid;
+    const uint32_t hw = SOLUTE ? bounce_mask(0u, g.onface & a.s_wall) : 0u;
+    const uint32_t hin = SOLUTE ? bounce_mask(0u, g.onface & a.s_inlet) & ~hw : 0u;
+    const uint32_t hout = SOLUTE ? bounce_mask(0u, g.onface & a.s_outlet) & ~(hw | hin) : 0u;
+    const uint32_t hown = hw | hin | (solid & ~hout);
+    Unroll<0, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const bool b = (fown >> q) & 1u;
+      d[q] = ld_f(qc, b ? opp(q) : q, b ? 0 : src_delta<q>(g));
+    });
+    if constexpr (SOLUTE)
       Unroll<0, Q>::run([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        d[q] = S::kShift ? o.v[q] * Real(inv_wq(q)) : o.v[q];
+        const bool b = (hown >> q) & 1u;
+        hh[q] = ld_h(qc, b ? opp(q) : q, (b || ((hout >> q) & 1u)) ? 0 : src_delta<q>(g));
       });
-    } else {
-      const uint32_t mf = bounce_mask(link, g.onface & a.f_wall);
-      Unroll<0, Q>::run([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        const bool b = (mf >> q) & 1u;
-        d[q] = ld_f(qc, b ? opp(q) : q, b ? 0 : src_delta<q>(g));
-      });
+    if constexpr ((FEAT & FEAT_OPEN) != 0) {
+      if (g.onface & (a.f_press | a.f_vel)) {
+        Pops<Real> o;
+        Unroll<0, Q>::run([&](auto qc) { o.v[decltype(qc)::value] = d[decltype(qc)::value]; });
+        o = open_face_rules<S>(a, g, n, eps, fvel, fprs, o);
+        Unroll<0, Q>::run([&](auto qc) { d[decltype(qc)::value] = o.v[decltype(qc)::value]; });
+      }
     }
     if constexpr (SOLUTE) {
-      // the solute classes; 16-bit paired values are per unit weight, their
-      // fluxes carry the weights
+      // 16-bit paired values are per unit weight, their fluxes carry the weights
       Real V[3], r_, s_;
       Lat<Real, false> sd_[Q];
       moments<S, false>([&](auto qc) { return d[decltype(qc)::value]; },
                         [&](auto) { return Real(0); }, r_, s_, V, sd_);
-      const Real vi0 = V[0] + __ldg(a.geps + n), vi1 = V[1] + __ldg(a.geps + N + n),
-                 vi2 = V[2] + __ldg(a.geps + 2 * size_t(N) + n);
-      Unroll<0, Q>::run([&](auto qc) {
+      const Real vi0 = V[0] + gx, vi1 = V[1] + gy, vi2 = V[2] + gz;
+      const bool counts = !(link >> 31);
+      Unroll<1, Q>::run([&](auto qc) {
         constexpr int q = decltype(qc)::value;
         constexpr Real wu = kPair ? Real(1) : wq<Real>(q), wf = kPair ? wq<Real>(q) : Real(1);
-        const int cls = solute_class<q>(g, link, a.s_wall, a.s_inlet, a.s_outlet);
-        Real v;
-        if (cls == PULL_CELL) {
-          v = ld_h(qc, q, src_delta<q>(g));
-        } else if (cls == PULL_BOUNCE) {
-          v = ld_h(qc, opp(q), 0);
-        } else if (cls == PULL_INLET) {
+        if ((hin >> q) & 1u) {
           // entering through an inlet face: h^eq at C_in with the cell's bare
           // streamed velocity plus D grad(eps)/eps
           const Real cv = Real(cx(q)) * vi0 + Real(cy(q)) * vi1 + Real(cz(q)) * vi2;
-          v = wu * __ldg(a.eps + n) * a.C_in * (Real(1) + Real(3) * cv);
-          const Real f = wf * (v - ld_h(qc, opp(q), 0));
-          if (!(link >> 31)) fin_acc += f;
-        } else {
+          const Real v = wu * eps * a.C_in * (Real(1) + Real(3) * cv);
+          const Real f = wf * (v - hh[q]);
+          if (counts) fin_acc += f;
+          hh[q] = v;
+        } else if ((hout >> q) & 1u) {
           // outlet: the cell's own post-collision value (zero gradient)
-          v = ld_h(qc, q, 0);
-          const Real f = wf * (ld_h(qc, opp(q), 0) - v);
-          if (!(link >> 31)) fout_acc += f;
+          const Real f = wf * (ld_h(qc, opp(q), 0) - hh[q]);
+          if (counts) fout_acc += f;
         }
-        hh[q] = v;
       });
     }
   }
-  if (g.onface & open) statics();
   if (link >> 31) return;  // impermeable: never updated
   Real V[3];
   auto fv = [&](auto qc) { return d[decltype(qc)::value]; };
