@@ -30,7 +30,7 @@ static_assert(sizeof(BatchTable<float>) <= 32000 && sizeof(BatchTable<double>) <
               "batch table exceeds the kernel parameter space");
 
 template <class S, int KMODE, bool SOLUTE>
-__global__ void __launch_bounds__(STEP_BLOCK, step_blocks<typename S::Real>())
+__global__ void __launch_bounds__(STEP_BLOCK, sizeof(typename S::Real) == 8 ? 3 : 6)
     batched_step_kernel(const __grid_constant__ BatchTable<typename S::Real> tab) {
   using Real = typename S::Real;
   const unsigned total = tab.begin[tab.n];

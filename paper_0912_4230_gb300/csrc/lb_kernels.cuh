@@ -1303,14 +1303,24 @@ __device__ __forceinline__ CellIndex cell_index(const StepArgs<Real> &a, unsigne
 // thread): measured on GB300 at 128^3 this is 1.1x faster than the
 // unconstrained build (112 registers), since the kernel is bound by loads in
 // flight, and a little faster than 256-thread blocks at the same occupancy.
-// FP64 populations take twice the registers, and the FP64 pipe is busy with a
-// few warps: three blocks (168 registers) instead of six with spills.
-template <class Real>
+// Resident 128-thread blocks per SM of the per-cell kernel (registers a thread).
+// The kernel is bound by loads in flight, so warps are traded against registers
+// that keep a cell's ~48 loads together. Measured on GB300, ms per step with 4 /
+// 5 / 6 / 7 blocks: 128^3 FP32 diagonal 0.1086 / 0.1067 / 0.1077 / 0.1135,
+// Forchheimer 0.1139 / 0.1077 / 0.1254 / 0.1161, 117x83x101 with 10 % solid cells
+// 0.0905 / 0.0886 / 0.0938 / 0.0986, 256x192x64 with pressure faces 0.1655 /
+// 0.1690 / 0.1734 / 0.1775, three species 0.2265 / 0.2237 / 0.2162 / 0.2256,
+// 256^3 FP16 0.706 / 0.682 / 0.614 / 0.612; the batched kernel takes 6 (15
+// lattices FP32 0.266 / 0.281 / 0.243 / 0.260). FP64 populations take twice the
+// registers, and its pipe is busy with a few warps.
+template <class S, bool SOLUTE, int FEAT>
 constexpr int step_blocks() {
-  return sizeof(Real) == 8 ? 3 : 6;
+  if (sizeof(typename S::Real) == 8) return 3;
+  if (S::kShift || !SOLUTE || (FEAT & FEAT_SPEC)) return 6;
+  return (FEAT & FEAT_OPEN) ? 4 : 5;
 }
 template <class S, int KMODE, bool SOLUTE, int FEAT>
-__global__ void __launch_bounds__(STEP_BLOCK, step_blocks<typename S::Real>()) step_kernel(const StepArgs<typename S::Real> a) {
+__global__ void __launch_bounds__(STEP_BLOCK, step_blocks<S, SOLUTE, FEAT>()) step_kernel(const StepArgs<typename S::Real> a) {
   using Real = typename S::Real;
   const CellIndex c = cell_index(a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y,
                                  blockDim.x, threadIdx.x, threadIdx.y, blockDim.x);
