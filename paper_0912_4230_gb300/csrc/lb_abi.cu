@@ -68,15 +68,16 @@ struct lb_ctx {
   int S = 0;                // solute species (0 without the solute lattice)
   void *spec = nullptr;     // S > 1: per-species 1/tau_D, C_in, D_s/D_0 (24 Real)
   void *face = nullptr;  // per-face values of pressure / velocity faces (30 Real)
-  // CUDA graphs: two steps (both buffer parities) captured once on a private
+  // CUDA graphs: step pairs (both buffer parities) captured once on a private
   // stream and replayed while the launch configuration holds (lb_step), and
   // the same for a batch led by this context, keyed by its members' serial
-  // numbers and parities and the work list (lb_step_batch)
+  // numbers and parities (lb_step_batch)
   bool graphs = true;
   uint64_t serial = 0;
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t g_step = nullptr;
-  cudaGraphExec_t g_batch = nullptr;
+  cudaGraphExec_t g_many = nullptr;  // GRAPH_PAIRS step pairs, for long calls on small lattices
+  cudaGraphExec_t g_batch = nullptr, g_batch_many = nullptr;
   std::vector<uint64_t> g_batch_key;
   long long t = 0;
   long long n_live = 0;
@@ -161,8 +162,10 @@ void dev_free(lb_ctx *c, void *p) {
 
 void drop_graphs(lb_ctx *c) {
   if (c->g_step) cudaGraphExecDestroy(c->g_step);
+  if (c->g_many) cudaGraphExecDestroy(c->g_many);
   if (c->g_batch) cudaGraphExecDestroy(c->g_batch);
-  c->g_step = c->g_batch = nullptr;
+  if (c->g_batch_many) cudaGraphExecDestroy(c->g_batch_many);
+  c->g_step = c->g_many = c->g_batch = c->g_batch_many = nullptr;
   c->g_batch_key.clear();
 }
 
@@ -516,11 +519,19 @@ bool graph_safe(const lb_ctx *c) {
   return c->graphs && c->prm.visc_law != 2 && c->prm.check_every <= 1;
 }
 
-// Capture two steps, issued by step(stream) with the lattices' t and parity
-// advanced in between (enqueue restores nothing: the caller's step function
-// reads c->t / c->cur), on the leader's private stream, and instantiate.
+// Step pairs in the graph of a long call. One graph follows another ~1.2 us
+// later than a kernel its predecessor inside a graph: with 1 / 8 / 16 pairs a
+// 32x32x45 FP32 lattice steps in 6.16 / 4.93 / 4.81 us, the FP64 channel in 10.27 /
+// 9.05 / 8.93, the free-surface drop in 39.2 / 37.9 / 37.8.
+constexpr int GRAPH_PAIRS = 8;
+
+// Capture pairs of steps, issued by step(stream) with the lattices' t and
+// parity advanced in between (enqueue restores nothing: the caller's step
+// function reads c->t / c->cur), on the leader's private stream, and
+// instantiate.
 template <class StepFn, class AdvanceFn>
-int capture_two(lb_ctx *lead, cudaGraphExec_t *out, StepFn &&step, AdvanceFn &&advance) {
+int capture_pairs(lb_ctx *lead, cudaGraphExec_t *out, int pairs, StepFn &&step,
+                  AdvanceFn &&advance) {
   if (!lead->cap_stream &&
       cudaStreamCreateWithFlags(&lead->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
@@ -530,10 +541,13 @@ int capture_two(lb_ctx *lead, cudaGraphExec_t *out, StepFn &&step, AdvanceFn &&a
     cudaGetLastError();
     return LB_ECUDA;
   }
-  int rc = step(lead->cap_stream);
-  advance(+1);
-  if (rc == LB_OK) rc = step(lead->cap_stream);
-  advance(-1);
+  int rc = LB_OK;
+  for (int p = 0; p < pairs; ++p) {
+    if (rc == LB_OK) rc = step(lead->cap_stream);
+    advance(+1);
+    if (rc == LB_OK) rc = step(lead->cap_stream);
+    advance(-1);
+  }
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(lead->cap_stream, &g);
   if (rc == LB_OK && e == cudaSuccess && g &&
@@ -548,8 +562,8 @@ int capture_two(lb_ctx *lead, cudaGraphExec_t *out, StepFn &&step, AdvanceFn &&a
 }
 
 template <class StepFn>
-int capture_pair(lb_ctx *c, cudaGraphExec_t *out, StepFn &&step) {
-  return capture_two(c, out, step, [&](int d) {
+int capture_steps(lb_ctx *c, cudaGraphExec_t *out, int pairs, StepFn &&step) {
+  return capture_pairs(c, out, pairs, step, [&](int d) {
     c->t += d;
     c->cur = 1 - c->cur;
   });
@@ -1008,16 +1022,19 @@ int lb_step(lb_ctx *c, int64_t n) {
     // the graph, starting from buffer parity 0
     const int64_t pairs = (n - i - 1) / 2;
     if (pairs > 0 && c->cur == 0 && graph_safe(c)) {
-      if (!c->g_step && capture_pair(c, &c->g_step, [&](cudaStream_t s) {
-            return enqueue_step(c, s, false);
-          }) != LB_OK)
-        c->graphs = false;  // not capturable here: plain launches from now on
-      if (c->g_step) {
-        for (int64_t p = 0; p < pairs; ++p) CK(c, cudaGraphLaunch(c->g_step, c->stream));
-        c->t += 2 * pairs;
-        i += 2 * pairs;
-        continue;
+      auto one = [&](cudaStream_t s) { return enqueue_step(c, s, false); };
+      int64_t done = 0;
+      if (pairs >= 2 * GRAPH_PAIRS) {
+        if (!c->g_many) capture_steps(c, &c->g_many, GRAPH_PAIRS, one);  // (or leave it to pairs)
+        for (; c->g_many && done + GRAPH_PAIRS <= pairs; done += GRAPH_PAIRS)
+          CK(c, cudaGraphLaunch(c->g_many, c->stream));
       }
+      if (done < pairs && !c->g_step && capture_steps(c, &c->g_step, 1, one) != LB_OK)
+        c->graphs = false;  // not capturable here: plain launches from now on
+      for (; c->g_step && done < pairs; ++done) CK(c, cudaGraphLaunch(c->g_step, c->stream));
+      c->t += 2 * done;
+      i += 2 * done;
+      if (done) continue;
     }
     const int rc = enqueue_step(c, c->stream, i == n - 1);
     if (rc != LB_OK) return rc;
@@ -1030,7 +1047,7 @@ int lb_step(lb_ctx *c, int64_t n) {
 
 int lb_debug_graphs(const lb_ctx *c) {
   if (!c) return LB_EINVAL;
-  return (c->g_step ? 1 : 0) | (c->g_batch ? 2 : 0);
+  return (c->g_step || c->g_many ? 1 : 0) | (c->g_batch || c->g_batch_many ? 2 : 0);
 }
 
 int lb_set_graphs(lb_ctx *c, int32_t enable) {
@@ -1115,19 +1132,23 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   int64_t k = 0;
   const int64_t pairs = steps > 0 ? (steps - 1) / 2 : 0;
   if (safe && pairs > 0) {
-    if (!c0->g_batch || c0->g_batch_key != key) {
+    if (c0->g_batch_key != key) {
       if (c0->g_batch) cudaGraphExecDestroy(c0->g_batch);
-      c0->g_batch = nullptr;
-      c0->g_batch_key.clear();
-      if (capture_two(c0, &c0->g_batch, [&](cudaStream_t st) { return one_step(st, false); },
-                      advance) == LB_OK)
-        c0->g_batch_key = key;
+      if (c0->g_batch_many) cudaGraphExecDestroy(c0->g_batch_many);
+      c0->g_batch = c0->g_batch_many = nullptr;
+      c0->g_batch_key = key;
     }
-    if (c0->g_batch) {
-      for (int64_t p = 0; p < pairs; ++p) CK(c0, cudaGraphLaunch(c0->g_batch, s));
-      for (int i = 0; i < n; ++i) ctxs[i]->t += 2 * pairs;
-      k = 2 * pairs;
+    auto one = [&](cudaStream_t st) { return one_step(st, false); };
+    int64_t done = 0;
+    if (pairs >= 2 * GRAPH_PAIRS) {
+      if (!c0->g_batch_many) capture_pairs(c0, &c0->g_batch_many, GRAPH_PAIRS, one, advance);
+      for (; c0->g_batch_many && done + GRAPH_PAIRS <= pairs; done += GRAPH_PAIRS)
+        CK(c0, cudaGraphLaunch(c0->g_batch_many, s));
     }
+    if (done < pairs && !c0->g_batch) capture_pairs(c0, &c0->g_batch, 1, one, advance);
+    for (; c0->g_batch && done < pairs; ++done) CK(c0, cudaGraphLaunch(c0->g_batch, s));
+    for (int i = 0; i < n; ++i) ctxs[i]->t += 2 * done;
+    k = 2 * done;
   }
   for (; k < steps; ++k) {
     const int rc = one_step(s, k == steps - 1);
