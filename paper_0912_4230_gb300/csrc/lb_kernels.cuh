@@ -244,17 +244,39 @@ __device__ __forceinline__ Real tau_of(const StepArgs<Real> &a, Real C) {
   return a.tau;
 }
 
+// c_q . (a0, a1, a2) by additions of the axes that q has (a product with a zero
+// component is an instruction the compiler may not drop; in FP64 it holds the
+// pipe for 64 cycles).
+template <int q, class Real>
+__device__ __forceinline__ Real dot_c(Real a0, Real a1, Real a2) {
+  if constexpr (cx(q) != 0) {
+    const Real s = cx(q) > 0 ? a0 : -a0;
+    if constexpr (cy(q) != 0) return cy(q) > 0 ? add_rn(s, a1) : sub_rn(s, a1);
+    if constexpr (cz(q) != 0) return cz(q) > 0 ? add_rn(s, a2) : sub_rn(s, a2);
+    return s;
+  } else if constexpr (cy(q) != 0) {
+    const Real s = cy(q) > 0 ? a1 : -a1;
+    if constexpr (cz(q) != 0) return cz(q) > 0 ? add_rn(s, a2) : sub_rn(s, a2);
+    return s;
+  } else if constexpr (cz(q) != 0) {
+    return cz(q) > 0 ? a2 : -a2;
+  } else {
+    return Real(0);
+  }
+}
+
 // Reciprocal in the collision type: one correctly rounded reciprocal
 // instruction sequence in FP32, exact division in FP64.
 __device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 
 // Reciprocal of a quantity of order one (density, porosity, relaxation time,
-// 1 + drag): the hardware's approximation and Newton-Raphson steps, r <- r + r
-// (1 - x r), one in FP32 (from 1 ulp) and two in FP64 (from 2^-20), without
-// the range checks and slow path of the exact reciprocal. FP64 arithmetic is
-// 1/64 of FP32's rate on this chip, so a reciprocal of 5 instead of ~10
-// instructions counts there.
+// 1 + drag): the hardware's approximation and a Newton-Raphson step, r <- r +
+// r e, e = 1 - x r, in FP32 (from 1 ulp) or the third-order step r + r (e + e^2)
+// in FP64 (from 2^-20 to beyond 2^-53), without the range checks and slow path
+// of the exact reciprocal. An FP64 instruction holds its pipe for 64 cycles a
+// warp on this chip (measured, whatever the active lanes), so 3 instead of ~10
+// count there.
 __device__ __forceinline__ float rcp1(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -263,8 +285,8 @@ __device__ __forceinline__ float rcp1(float x) {
 __device__ __forceinline__ double rcp1(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 
 // Inside an iteration that corrects its own errors (the Forchheimer Newton
@@ -348,17 +370,25 @@ __device__ __forceinline__ void velocity_solve_kv(KV kv, Real eps, Real nu, cons
   } else if (KMODE == KM_DIAG) {
     const Real kx = kv(0), ky = kv(1), kz = kv(2);
     const Real hs = Real(0.5) * en;
+    if constexpr (sizeof(Real) == 8) {
+      // one reciprocal for the three (k <= 1e45, so the product is finite)
+      const Real e0 = en * kx, e1 = en * ky, e2 = en * kz;
+      const Real lx = fma(Real(0.5), e0, Real(1)), ly = fma(Real(0.5), e1, Real(1)),
+                 lz = fma(Real(0.5), e2, Real(1));
+      const Real lxy = lx * ly, i3 = rcp1(lxy * lz), iz = i3 * lz;
+      Vp[0] = r0 * (iz * ly);
+      Vp[1] = r1 * (iz * lx);
+      Vp[2] = r2 * (i3 * lxy);
+      Fe[0] = fma(-e0, Vp[0], eps * G[0]);
+      Fe[1] = fma(-e1, Vp[1], eps * G[1]);
+      Fe[2] = fma(-e2, Vp[2], eps * G[2]);
+      return;
+    }
     const Real lx = Real(1) + hs * kx, ly = Real(1) + hs * ky, lz = Real(1) + hs * kz;
     if constexpr (EXACT) {
       Vp[0] = r0 * rcp(lx);
       Vp[1] = r1 * rcp(ly);
       Vp[2] = r2 * rcp(lz);
-    } else if constexpr (sizeof(Real) == 8) {
-      // one FP64 reciprocal for the three (k <= 1e45, so the product is finite)
-      const Real lxy = lx * ly, i3 = rcp1(lxy * lz), iz = i3 * lz;
-      Vp[0] = r0 * (iz * ly);
-      Vp[1] = r1 * (iz * lx);
-      Vp[2] = r2 * (i3 * lxy);
     } else {
       Vp[0] = r0 * rcp1(lx);
       Vp[1] = r1 * rcp1(ly);
@@ -446,11 +476,11 @@ struct FluidCollide {
   template <int q>
   __device__ __forceinline__ Real br() const {
     if (q == 0) return K0;
-    const Real cu = Real(cx(q)) * Vp[0] + Real(cy(q)) * Vp[1] + Real(cz(q)) * Vp[2];
-    const Real cF = Real(cx(q)) * Fe[0] + Real(cy(q)) * Fe[1] + Real(cz(q)) * Fe[2];
+    const Real cu = dot_c<q>(Vp[0], Vp[1], Vp[2]);
+    const Real cF = dot_c<q>(Fe[0], Fe[1], Fe[2]);
     Real b = cu * (B3 + B45 * cu + P9 * cF) + (P3 * cF + K);
     if (st) {
-      const Real cs = Real(cx(q)) * F[0] + Real(cy(q)) * F[1] + Real(cz(q)) * F[2];
+      const Real cs = dot_c<q>(F[0], F[1], F[2]);
       b += S2 * cs * cs;
     }
     return b;
@@ -459,10 +489,10 @@ struct FluidCollide {
   // + P9 cF) [+ S2 (c.F)^2] and B3 cu + P3 cF (cu = c_q.V', cF = c_q.F_e)
   template <int q>
   __device__ __forceinline__ void even_odd(Real cu, Real &ev, Real &od) const {
-    const Real cF = Real(cx(q)) * Fe[0] + Real(cy(q)) * Fe[1] + Real(cz(q)) * Fe[2];
+    const Real cF = dot_c<q>(Fe[0], Fe[1], Fe[2]);
     ev = fma(cu, fma(B45, cu, P9 * cF), K);
     if (st) {
-      const Real cs = Real(cx(q)) * F[0] + Real(cy(q)) * F[1] + Real(cz(q)) * F[2];
+      const Real cs = dot_c<q>(F[0], F[1], F[2]);
       ev = fma(S2 * cs, cs, ev);
     }
     od = fma(B3, cu, P3 * cF);
@@ -472,10 +502,10 @@ struct FluidCollide {
   __device__ __forceinline__ Real feq_dev() const {
     constexpr Real w = wq<Real>(q);
     if (q == 0) return w * (drho - rho * Real(1.5) * ie * uu) + (st ? stc * w * Fn : Real(0));
-    const Real cu = Real(cx(q)) * Vp[0] + Real(cy(q)) * Vp[1] + Real(cz(q)) * Vp[2];
+    const Real cu = dot_c<q>(Vp[0], Vp[1], Vp[2]);
     Real e = w * (drho + rho * (Real(3) * cu + Real(4.5) * ie * cu * cu - Real(1.5) * ie * uu));
     if (st) {
-      const Real cs = Real(cx(q)) * F[0] + Real(cy(q)) * F[1] + Real(cz(q)) * F[2];
+      const Real cs = dot_c<q>(F[0], F[1], F[2]);
       e += w * stc * (cs * cs * iFn - Fn);
     }
     return e;
@@ -722,7 +752,7 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
   using D = Lat<Real, true>;
   const unsigned N = a.N;
   const Real rho = Real(1) + drho;
-  const Real C = sC * ie;
+  const Real C = SOLUTE ? sC * ie : Real(0);
   const Real tau = tau_of(a, C);
   const Real nu = a.visc_law == 0 ? a.nu0 : (tau - Real(0.5)) * Real(1.0 / 3.0);
   FluidCollide<Real> fc;
@@ -802,8 +832,8 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
   } else {
     constexpr Real w = wq<Real>(1);
     const Real itau = a.visc_law == 0 ? a.itau : rcp1(tau), omt = Real(1) - itau;
-    const Real it = w * itau, r3 = Real(3) * (it * rho), r15 = Real(0.5) * r3;
-    const Real p3 = Real(3) * w * (rho * fma(Real(-0.5), itau, Real(1)));
+    const Real it = w * itau, r3 = (Real(3) * it) * rho, r15 = Real(0.5) * r3;
+    const Real p3 = (Real(3) * w * fma(Real(-0.5), itau, Real(1))) * rho;
     const Real ie3 = Real(3) * ie;
     Real K, Wv[3], X[3], VY = Real(0);
 #pragma unroll
@@ -842,7 +872,7 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
       const D vx = along<q>(VX, D{});
       Real ev = fma(vx.lo(), vx.hi(), K);
       if constexpr (TENS) {
-        const Real cs = Real(cx(q)) * F[0] + Real(cy(q)) * F[1] + Real(cz(q)) * F[2];
+        const Real cs = dot_c<q>(F[0], F[1], F[2]);
         ev = fma(S2 * cs, cs, ev);
       }
       L e = L::mk(ev, so.e);
@@ -925,28 +955,43 @@ __device__ __noinline__ Pops<typename S::Real> open_face_rules(
   using Real = typename S::Real;
   using T = typename S::T;
   const unsigned N = a.N;
-  Real r = Real(0), j0 = Real(0), j1 = Real(0), j2 = Real(0);
-  Unroll<0, Q>::run([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    Real v;  // the own f~_q - w_q
-    if constexpr (S::kShift) {
+  Real r = Real(0), u0, u1, u2, ie;
+  if constexpr (S::kShift) {
+    Real j0 = Real(0), j1 = Real(0), j2 = Real(0);
+    Unroll<0, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      Real v;  // the own f~_q - w_q
       if (a.paired)
         v = wq<Real>(q) * (S::ld2(static_cast<const typename S::T2 *>(a.f_in) + size_t(q) * N + n).x +
                            ld_ref2(a.rf_in + n).x);
       else
         v = S::template ld_f<q>(static_cast<const T *>(a.f_in) + size_t(q) * N + n) +
             wq<Real>(q) * __ldg(a.rf_in + n);
-    } else {
-      v = S::template ld_f<q>(static_cast<const T *>(a.f_in) + size_t(q) * N + n);
-    }
-    r += v;
-    if (cx(q)) j0 += Real(cx(q)) * v;
-    if (cy(q)) j1 += Real(cy(q)) * v;
-    if (cz(q)) j2 += Real(cz(q)) * v;
-  });
-  const Real rho = Real(1) + r, irho = rcp(rho);
-  const Real u0 = j0 * irho, u1 = j1 * irho, u2 = j2 * irho;
-  const Real ie = rcp(eps);
+      r += v;
+      if (cx(q)) j0 += Real(cx(q)) * v;
+      if (cy(q)) j1 += Real(cy(q)) * v;
+      if (cz(q)) j2 += Real(cz(q)) * v;
+    });
+    const Real irho = rcp(Real(1) + r);
+    u0 = j0 * irho;
+    u1 = j1 * irho;
+    u2 = j2 * irho;
+    ie = rcp(eps);
+  } else {
+    Real u[3], s_;
+    Lat<Real, false> sd_[Q];
+    moments<S, false>(
+        [&](auto qc) {
+          constexpr int q = decltype(qc)::value;
+          return S::template ld_f<q>(static_cast<const T *>(a.f_in) + size_t(q) * N + n);
+        },
+        [&](auto) { return Real(0); }, r, s_, u, sd_);
+    u0 = u[0];
+    u1 = u[1];
+    u2 = u[2];
+    ie = rcp1(eps);
+  }
+  const Real rho = Real(1) + r;
   const Real uu = u0 * u0 + u1 * u1 + u2 * u2;
   Unroll<0, Q>::run([&](auto qc) {
     constexpr int q = decltype(qc)::value;
@@ -957,13 +1002,12 @@ __device__ __noinline__ Pops<typename S::Real> open_face_rules(
       const int fi = crossed_face<q>(g, a.f_press);
       const Real rbm1 = fma(eps, __ldg(a.face + fi), Real(-1)) + eps * __ldg(a.face + 24 + fi);
       const Real rb = Real(1) + rbm1;
-      const Real cu = Real(cx(q)) * u0 + Real(cy(q)) * u1 + Real(cz(q)) * u2;
+      const Real cu = dot_c<q>(u0, u1, u2);
       const Real e = wq<Real>(q) * (rbm1 + rb * (Real(4.5) * ie * cu * cu - Real(1.5) * ie * uu));
       v = Real(2) * e - own;
     } else if ((fvel >> q) & 1u) {
       const Real *uf = a.face + 6 + 3 * crossed_face<q>(g, a.f_vel);
-      const Real cub = Real(cx(q)) * __ldg(uf) + Real(cy(q)) * __ldg(uf + 1) +
-                       Real(cz(q)) * __ldg(uf + 2);
+      const Real cub = dot_c<q>(__ldg(uf), __ldg(uf + 1), __ldg(uf + 2));
       v = own + Real(6) * wq<Real>(q) * rho * cub;
     }
     d.v[q] = S::kShift ? v * Real(inv_wq(q)) : v;
@@ -1125,7 +1169,7 @@ __device__ __forceinline__ void update_cell(const StepArgs<typename S::Real> &a,
         if ((hin >> q) & 1u) {
           // entering through an inlet face: h^eq at C_in with the cell's bare
           // streamed velocity plus D grad(eps)/eps
-          const Real cv = Real(cx(q)) * vi0 + Real(cy(q)) * vi1 + Real(cz(q)) * vi2;
+          const Real cv = dot_c<q>(vi0, vi1, vi2);
           const Real v = wu * eps * a.C_in * (Real(1) + Real(3) * cv);
           const Real f = wf * (v - hh[q]);
           if (counts) fin_acc += f;
@@ -1199,7 +1243,7 @@ __device__ __forceinline__ void species_update(const StepArgs<typename S::Real> 
       } else if (cls == PULL_BOUNCE) {
         v = S::template ld_h<opp(q)>(hb + int(opp(q) * N)) + own;
       } else if (cls == PULL_INLET) {
-        const Real cv = Real(cx(q)) * vi0 + Real(cy(q)) * vi1 + Real(cz(q)) * vi2;
+        const Real cv = dot_c<q>(vi0, vi1, vi2);
         v = wq<Real>(q) * eps * C_in * (Real(1) + Real(3) * cv);
         fin_acc += v - (S::template ld_h<opp(q)>(hb + int(opp(q) * N)) + own);
       } else {
@@ -1216,7 +1260,7 @@ __device__ __forceinline__ void species_update(const StepArgs<typename S::Real> 
     Real hsum = Real(0);
     Unroll<1, Q>::run([&](auto qc) {
       constexpr int q = decltype(qc)::value;
-      const Real cv = Real(cx(q)) * vs0 + Real(cy(q)) * vs1 + Real(cz(q)) * vs2;
+      const Real cv = dot_c<q>(vs0, vs1, vs2);
       const Real heq = wq<Real>(q) * sC * (Real(1) + Real(3) * cv);
       hsum += heq;
       const Real h = hh[q];
@@ -1482,7 +1526,7 @@ __global__ void __launch_bounds__(BLOCK) init_kernel(const StepArgs<typename S::
     Real hsum = Real(0);
     Unroll<0, Q>::run([&](auto qc) {
       constexpr int q = decltype(qc)::value;
-      const Real cv = Real(cx(q)) * vs0 + Real(cy(q)) * vs1 + Real(cz(q)) * vs2;
+      const Real cv = dot_c<q>(vs0, vs1, vs2);
       hs[q] = wq<Real>(q) * eps * C * (Real(1) + Real(3) * cv);
       hsum += hs[q];
     });
@@ -1514,7 +1558,7 @@ __global__ void __launch_bounds__(BLOCK) init_kernel(const StepArgs<typename S::
     Real hsum = Real(0);
     Unroll<0, Q>::run([&](auto qc) {
       constexpr int q = decltype(qc)::value;
-      const Real cv = Real(cx(q)) * vs0 + Real(cy(q)) * vs1 + Real(cz(q)) * vs2;
+      const Real cv = dot_c<q>(vs0, vs1, vs2);
       hs[q] = wq<Real>(q) * eps * C * (Real(1) + Real(3) * cv);
       hsum += hs[q];
     });
