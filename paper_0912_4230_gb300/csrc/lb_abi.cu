@@ -96,6 +96,7 @@ struct lb_ctx {
   uint8_t *type = nullptr, *flag = nullptr;
   void *mass = nullptr, *lam = nullptr, *rho_post = nullptr, *mom = nullptr;
   uint32_t *flagged = nullptr, *near = nullptr;  // cells that convert, and with their neighbours
+  uint32_t *cells = nullptr;                     // liquid and interface cells
   // free surface: active-tile lists (parity of the epoch), tile stamps, counters
   uint32_t *tiles[2] = {nullptr, nullptr};
   unsigned *stamp = nullptr;
@@ -453,6 +454,7 @@ FsArgs<Real> fs_args(lb_ctx *c, const StepArgs<Real> &a) {
   fa.flag = c->flag;
   fa.flagged = c->flagged;
   fa.near = c->near;
+  fa.cells = c->cells;
   fa.rho_post = static_cast<Real *>(c->rho_post);
   fa.mom = static_cast<Real *>(c->mom);
   fa.cnt = c->fs_cnt;
@@ -633,7 +635,7 @@ int lb_bytes_required(const lb_domain *dom, const lb_params *prm, int32_t k_rows
   const size_t twice[] = {L.f, L.h, L.rf, L.rh, L.fs_list, L.fs_tiles};
   const size_t once[] = {L.spec, L.eps, L.link, L.fields, L.partials, L.state, L.geps,
                          L.rhohat, L.face, L.fs_type, L.fs_mass, L.fs_lam, L.fs_rho, L.fs_mom,
-                         L.fs_flag, L.fs_stamp, L.fs_cnt, L.kinv, L.flux_slots,
+                         L.fs_flag, L.fs_list, L.fs_stamp, L.fs_cnt, L.kinv, L.flux_slots,
                          L.batch_share};
   size_t total = 0;
   for (size_t b : twice) total += 2 * granule(b);
@@ -797,6 +799,7 @@ int lb_create(const lb_domain *dom, const float *porosity, const float *K6, cons
     c->flag = static_cast<uint8_t *>(dev_alloc(c, L.fs_flag));
     c->flagged = static_cast<uint32_t *>(dev_alloc(c, L.fs_list));
     c->near = static_cast<uint32_t *>(dev_alloc(c, L.fs_list));
+    c->cells = static_cast<uint32_t *>(dev_alloc(c, L.fs_list));
     c->ntx = (unsigned(dom->nx) + FS_TX - 1) / FS_TX;
     c->nty = (unsigned(dom->ny) + FS_TY - 1) / FS_TY;
     c->ntz = (unsigned(dom->nz) + FS_TZ - 1) / FS_TZ;
@@ -806,15 +809,15 @@ int lb_create(const lb_domain *dom, const float *porosity, const float *K6, cons
     c->stamp = static_cast<unsigned *>(dev_alloc(c, L.fs_stamp));
     c->fs_cnt = static_cast<FsCount *>(dev_alloc(c, L.fs_cnt));
     if (!c->type || !c->mass || !c->lam || !c->rho_post || !c->mom || !c->flag || !c->flagged ||
-        !c->near || !c->tiles[0] || !c->tiles[1] || !c->stamp || !c->fs_cnt)
+        !c->near || !c->cells || !c->tiles[0] || !c->tiles[1] || !c->stamp || !c->fs_cnt)
       return bail(fail(c, LB_ENOMEM, "free surface"));
-    // persistent grid of the tile passes: enough resident blocks to cover
-    // the list of a typical step in one round
+    // grid of the passes over the listed cells: the resident blocks
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return bail(fail(c, LB_ECUDA, "device attributes"));
-    c->fs_grid = unsigned(std::min<size_t>(ntiles, size_t(FS_BLOCKS_PER_SM) * unsigned(sms)));
+    c->fs_grid = unsigned(std::min<size_t>((N + FS_BLOCK - 1) / FS_BLOCK,
+                                           size_t(FS_BLOCKS_PER_SM) * unsigned(sms)));
   }
   // inputs -> device (caller pointers may be host or device)
   const size_t in_bytes = N * 4 + (K6 ? 6 * N * 4 : 0) + N + 64;
@@ -987,6 +990,7 @@ int lb_init(lb_ctx *c, const float *rho0, const float *u0, const float *C0,
     const Layout L = layout_of(c->dom, c->prm, *c->ops, 0, false);
     CK(c, cudaMemsetAsync(c->flag, 0, L.fs_flag, c->stream));
     CK(c, cudaMemsetAsync(c->stamp, 0, L.fs_stamp, c->stream));
+    CK(c, cudaMemsetAsync(c->rho_post, 0, L.fs_rho, c->stream));
     CK(c, cudaMemsetAsync(c->fs_cnt, 0, sizeof(FsCount), c->stream));
   } else if (c->prm.A != 0.0) {
     CK(c, rhohat_init(c->N, c->link, d_rho, nullptr, c->prm.wall_rho, c->rhohat, c->ops->fp64,

@@ -305,10 +305,11 @@ enum : uint8_t { FS_NONE = 0, FS_FILL = 1, FS_EMPTYING = 2, FS_NEWCELL = 4, FS_C
 // Counters of the free surface, on the device, so that a step's launches are
 // the same every time: steps taken since lb_init (read by a step's first pass,
 // advanced by its second) and the step in progress, the cells flagged in this
-// step, the cells near a conversion (this and the previous step, by parity),
-// the tiles of the current and the next list (by parity of the epoch).
+// step and the new interface cells, the cells near a conversion (this and the previous step, by parity),
+// the tiles and the cells of the current and the next list (by parity of the
+// epoch).
 struct FsCount {
-  unsigned step, now, n_flag, n_near[2], n_tiles[2];
+  unsigned step, now, n_flag, n_new, n_near[2], n_tiles[2], n_cells[2];
 };
 
 template <class Real>
@@ -321,13 +322,15 @@ struct FsArgs {
                          // emptied holds the excess mass of each receiver
   Real *rhohat_w;        // colour-gradient field written by the mass exchange
   uint8_t *flag;         // (N rounded up to whole words)
-  uint32_t *flagged;     // cells that fill or empty in this step
+  uint32_t *flagged;     // cells that fill or empty in this step; from its end, new cells
   uint32_t *near;        // converted cells and their neighbours
   Real *rho_post;        // post-collision density of each live cell (new interface cells:
-                         // of their initial populations)
+                         // of their initial populations); minus (1 + the epoch in which it
+                         // emptied) of a cell that has been live
   Real *mom;             // rho, V'_x, V'_y, V'_z (4 x N) of each live cell that pulls
                          // from an empty cell, written by the step pass
   FsCount *cnt;
+  uint32_t *cells;       // liquid and interface cells (fs_cell_loop)
   // Active tiles of FS_TX x FS_TY x FS_TZ cells: the tiles holding a cell
   // within one link of a liquid or interface cell (wrapped), by parity of the
   // epoch, and per tile 1 + the latest epoch whose list holds it.
@@ -336,14 +339,14 @@ struct FsArgs {
   unsigned ntx, nty, ntz;
   FastDiv by_ntx, by_nty;
 };
-// steps that one tile list serves before it is built afresh
+// steps that one cell list serves before it is built afresh
 constexpr unsigned FS_EPOCH = 16;
 // the launches over the converting cells: a thread per cell
-constexpr unsigned FS_LIST_BLOCK = 64, FS_LIST_GRID = 128;
+constexpr unsigned FS_LIST_BLOCK = 64, FS_LIST_GRID = 304;
 constexpr unsigned FS_TX = 32, FS_TY = 1, FS_TZ = 2;
-// the tile passes run one block of FS_BLOCK threads per tile (one thread a
-// cell), with as many blocks per SM as its 2048 threads and 32 blocks allow
+// threads per block: a tile's cells when lists are built, listed cells in the
+// passes, with as many blocks per SM as the stream/collide pass holds
 constexpr unsigned FS_BLOCK = FS_TX * FS_TY * FS_TZ;
-constexpr unsigned FS_BLOCKS_PER_SM = 2048 / FS_BLOCK < 32 ? 2048 / FS_BLOCK : 32;
+constexpr unsigned FS_BLOCKS_PER_SM = 12;
 
 }  // namespace lbgb

@@ -3,32 +3,36 @@
 // populations coming from empty cells, and the re-typing of cells whose
 // liquid fraction leaves [0, 1].
 //
-// One step is two passes over the active tiles (tiles holding a cell within
-// one link of a liquid or interface cell; every cell outside them is empty
-// with nothing to do) and three launches over the few cells that convert:
+// One step is two passes over the list of liquid and interface cells and three
+// launches over the few cells that convert:
 //   fs_mass      liquid-mass exchange, colour-gradient field
 //   fs_step      stream/collide; lists the interface cells that fill or empty
 //   fs_convert   re-types the listed cells and their neighbours
 //   fs_newcell   populations of new interface cells, excess mass
-//   fs_finish    receives the excess mass; liquid fraction, tiles of new cells
+//   fs_finish    receives the excess mass; liquid fraction, the list's upkeep
 // Each needs its neighbours' results of the one before. A drop of radius 24
 // converts ~100 of its 70 000 cells a step: as passes over all active tiles the
 // conversions took 36 us of a 192x192x128 step (of 55 us), as launches over
-// lists about 10 us (of 39).
+// lists about 10 us. Over the cells of active tiles (32x1x2) the two passes ran
+// 4 500 warps, in which two lanes of five were live, in two rounds of an SM's
+// resident warps; over the listed cells they are 2 100 full warps in one round:
+// 37.9 -> 32.9 us a step (with a warp per new cell).
 #pragma once
 
 #include "lb_kernels.cuh"
 
 namespace lbgb {
 
+static_assert(FS_BLOCK == FS_LIST_BLOCK, "fs_finish scans a tile per block");
 static_assert(FS_BLOCK % 32 == 0 && FS_BLOCK >= 27,
               "whole warps per tile, and a thread for each of the 27 tiles around it");
-// With FP32 storage the stream/collide pass keeps 24 warps per SM resident
-// (at most 85 registers a thread): on the falling drop 3 % faster than at 96
-// registers (20 warps), and no spills. FP64 takes what it needs.
+// With FP32 storage the stream/collide pass takes at most 102 registers (20
+// warps per SM): a drop of 70 000 cells is 14 warps an SM, and 80 or 128 registers
+// were no faster (38.8 / 38.3 / 38.3 us a step with 768 / 640 / 512 threads). FP64
+// takes what it needs.
 template <class Real>
 constexpr unsigned fs_step_blocks() {
-  return sizeof(Real) == 4 ? 768 / FS_BLOCK : 1;
+  return sizeof(Real) == 4 ? 640 / FS_BLOCK : 1;
 }
 
 // Tiles needed by the next step around one cell, as a mask over the 27
@@ -50,10 +54,11 @@ __device__ __forceinline__ unsigned fs_tile_mask(unsigned lx, unsigned ly, unsig
   return m;
 }
 
-// The tile list that step c runs over. A list serves FS_EPOCH steps: tiles of
-// new interface cells are appended as they appear, and its last step stamps the
-// next list from the cells that are live then (a tile that has emptied stays
-// listed until then; its cells do nothing).
+// The list of cells serves FS_EPOCH steps: new interface cells are appended as
+// they appear, cells that empty stay as entries without effect, and the last
+// step of the epoch builds the list afresh from the cells that are live then,
+// row by row of the active tiles (appended cells would scatter a warp's
+// accesses ever more). The tiles' list is kept the same way.
 __device__ __forceinline__ unsigned fs_epoch(unsigned c) { return c / FS_EPOCH; }
 __device__ __forceinline__ bool fs_rebuilds(unsigned c) { return c % FS_EPOCH == FS_EPOCH - 1; }
 
@@ -62,6 +67,16 @@ template <class Real>
 __device__ __forceinline__ void fs_add_tile(const FsArgs<Real> &s, unsigned t, unsigned e) {
   if (atomicExch(s.stamp + t, e + 1u) != e + 1u)
     s.tiles[e & 1u][atomicAdd(&s.cnt->n_tiles[e & 1u], 1u)] = t;
+}
+
+// The tile at offset k (0 .. 26, as in fs_tile_mask) of tile (bx, by, bz), wrapped.
+template <class Real>
+__device__ __forceinline__ unsigned fs_tile_near(const FsArgs<Real> &s, unsigned bx, unsigned by,
+                                                 unsigned bz, unsigned k) {
+  const unsigned mx = (bx + s.ntx + k % 3 - 1) % s.ntx;
+  const unsigned my = (by + s.nty + (k / 3) % 3 - 1) % s.nty;
+  const unsigned mz = (bz + s.ntz + k / 9 - 1) % s.ntz;
+  return mx + s.ntx * (my + s.nty * mz);
 }
 
 // Adds the tiles of the block-wide OR of the cells' masks around tile (bx, by,
@@ -78,66 +93,59 @@ __device__ __forceinline__ void fs_stamp_tiles(const FsArgs<Real> &s, unsigned b
   if ((threadIdx.x & 31u) == 0 && mask) atomicOr(&block_mask, mask);
   __syncthreads();
   const unsigned k = threadIdx.x;
-  if (k < 27 && ((block_mask >> k) & 1u)) {
-    const unsigned mx = (bx + s.ntx + k % 3 - 1) % s.ntx;
-    const unsigned my = (by + s.nty + (k / 3) % 3 - 1) % s.nty;
-    const unsigned mz = (bz + s.ntz + k / 9 - 1) % s.ntz;
-    fs_add_tile(s, mx + s.ntx * (my + s.nty * mz), e);
-  }
+  if (k < 27 && ((block_mask >> k) & 1u)) fs_add_tile(s, fs_tile_near(s, bx, by, bz, k), e);
   __syncthreads();  // block_mask is reset for the next tile only after every read
 }
 
-// Cells of step c's active tiles: block b takes list entries b, b +
-// gridDim.x, ...; thread k is cell (k % FS_TX, (k / FS_TX) % FS_TY, k /
-// (FS_TX FS_TY)) of the tile. cell(n, lx, ly, lz) runs for cells inside the
-// lattice; with MARK it returns the cell's tile mask (fs_tile_mask), and when
-// step c rebuilds the list the tiles of the block's masks are added to the next
-// one (the trip count is uniform in the block, so every thread reaches the
-// barriers).
-template <bool MARK, class Real, class F>
-__device__ __forceinline__ void fs_tile_loop(const FsArgs<Real> &s, unsigned c, F &&cell) {
-  const unsigned e = fs_epoch(c), cnt = s.cnt->n_tiles[e & 1u];
-  const uint32_t *list = s.tiles[e & 1u];
+// The live cells of tile (thread k is cell (k % FS_TX, (k / FS_TX) % FS_TY, k /
+// (FS_TX FS_TY)) of it; every thread of the block calls) go to the cell list of
+// epoch e, the tiles within one link of them to its tile list.
+template <class Real>
+__device__ __forceinline__ void fs_scan_tile(const FsArgs<Real> &s, unsigned tile, unsigned e) {
   const unsigned tx = threadIdx.x % FS_TX, ty = (threadIdx.x / FS_TX) % FS_TY,
                  tz = threadIdx.x / (FS_TX * FS_TY);
-  for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const unsigned tile = list[i];
-    const unsigned r = s.by_ntx.div(tile), bx = tile - r * s.ntx, bz = s.by_nty.div(r),
-                   by = r - bz * s.nty;
-    const unsigned x = bx * FS_TX + tx, y = by * FS_TY + ty, z = bz * FS_TZ + tz;
-    unsigned mask = 0u;
-    if (x < s.a.nx && y < s.a.ny && z < s.a.nz) mask = cell(x, y, z, tx, ty, tz);
-    if (MARK && fs_rebuilds(c)) fs_stamp_tiles(s, bx, by, bz, mask, e + 1u);
-  }
+  const unsigned r = s.by_ntx.div(tile), bx = tile - r * s.ntx, bz = s.by_nty.div(r),
+                 by = r - bz * s.nty;
+  const unsigned x = bx * FS_TX + tx, y = by * FS_TY + ty, z = bz * FS_TZ + tz;
+  const unsigned n = x + s.a.nx * (y + s.a.ny * z);
+  bool live = x < unsigned(s.a.nx) && y < unsigned(s.a.ny) && z < unsigned(s.a.nz);
+  if (live) live = !(s.a.link && (s.a.link[n] >> 31)) && s.type[n] != CELL_EMPTY;
+  fs_stamp_tiles(s, bx, by, bz, fs_tile_mask(tx, ty, tz, live, live), e);
+  const unsigned row = __ballot_sync(0xffffffffu, live), lane = threadIdx.x & 31u;
+  unsigned at = 0;
+  if (lane == 0 && row) at = atomicAdd(&s.cnt->n_cells[e & 1u], unsigned(__popc(row)));
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if (live) s.cells[at + __popc(row & ((1u << lane) - 1u))] = n;
 }
 
-// After initialisation: one block per tile stamps the tiles the first step
-// needs around its liquid and interface cells.
+// After initialisation: one block per tile lists the first step's cells.
 template <class Real>
 __global__ void __launch_bounds__(FS_BLOCK) fs_seed_kernel(const FsArgs<Real> s) {
-  const unsigned tile = blockIdx.x;
-  const unsigned bx = tile % s.ntx, r = tile / s.ntx, by = r % s.nty, bz = r / s.nty;
-  const unsigned tx = threadIdx.x % FS_TX, ty = (threadIdx.x / FS_TX) % FS_TY,
-                 tz = threadIdx.x / (FS_TX * FS_TY);
-  const unsigned x = bx * FS_TX + tx, y = by * FS_TY + ty, z = bz * FS_TZ + tz;
-  unsigned mask = 0u;
-  if (x < s.a.nx && y < s.a.ny && z < s.a.nz) {
-    const unsigned n = x + s.a.nx * (y + s.a.ny * z);
-    const uint32_t link = s.a.link ? s.a.link[n] : 0u;
-    const bool live = !(link >> 31) && s.type[n] != CELL_EMPTY;
-    mask = fs_tile_mask(tx, ty, tz, live, live);
+  fs_scan_tile(s, blockIdx.x, 0u);
+}
+
+// cell(n, x, y, z) for the live cells listed for step c, a thread each.
+template <class Real, class F>
+__device__ __forceinline__ void fs_cell_loop(const FsArgs<Real> &s, unsigned c, F &&cell) {
+  const unsigned cnt = s.cnt->n_cells[fs_epoch(c) & 1u];
+  for (unsigned i = blockIdx.x * FS_BLOCK + threadIdx.x; i < cnt; i += gridDim.x * FS_BLOCK) {
+    const unsigned n = s.cells[i];
+    const unsigned yz = s.a.by_nx.div(n), x = n - yz * s.a.nx, z = s.a.by_ny.div(yz),
+                   y = yz - z * s.a.ny;
+    cell(n, x, y, z);
   }
-  fs_stamp_tiles(s, bx, by, bz, mask, 0u);
 }
 
 // Flowchart step g, Eqs. eq:massmacro, eq:massevol, eq:deltamass:
 // m(x, t+1) = m(x, t) + sum_q w (f~_opp(q)(x + c_q) - f~_q(x)), with w = 1 when
 // either cell is liquid, (lambda(x) + lambda(x + c_q))/2 between two
 // interface cells, and no exchange with empty or solid cells. The colour
-// gradient field is the new liquid mass (0 in empty, wall_rho in solid cells).
+// gradient field is the new liquid mass (it holds 0 in empty cells and wall_rho
+// in solid ones from the initialisation and the conversions).
 // The types of all neighbours are loaded together, then the populations of
 // nine directions at a time, whatever the types (every address is a cell): one
-// wait each instead of one per direction.
+// wait each instead of one per direction (all 36 populations at once, at 128
+// registers, were slower: 12.5 instead of 11.4 us).
 template <class S>
 __global__ void __launch_bounds__(FS_BLOCK, sizeof(typename S::Real) == 4 ? 12 : 6)
     fs_mass_kernel(const FsArgs<typename S::Real> s) {
@@ -154,25 +162,21 @@ __global__ void __launch_bounds__(FS_BLOCK, sizeof(typename S::Real) == 4 ? 12 :
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       s.cnt->now = c;
       s.cnt->n_flag = 0u;
+      s.cnt->n_new = 0u;
       s.cnt->n_near[c & 1u] = 0u;
-      if (c % FS_EPOCH == 0) s.cnt->n_tiles[(fs_epoch(c) + 1u) & 1u] = 0u;
+      if (c % FS_EPOCH == 0) {
+        s.cnt->n_tiles[(fs_epoch(c) + 1u) & 1u] = 0u;
+        s.cnt->n_cells[(fs_epoch(c) + 1u) & 1u] = 0u;
+      }
     }
   }
-  fs_tile_loop<false>(s, c, [&](unsigned x, unsigned y, unsigned z, unsigned, unsigned,
-                                unsigned) -> unsigned {
-    const unsigned n = x + a.nx * (y + a.ny * z), N = a.N;
+  fs_cell_loop(s, c, [&](unsigned n, unsigned x, unsigned y, unsigned z) {
+    const unsigned N = a.N;
     const uint32_t link = a.link ? __ldg(a.link + n) : 0u;
     const uint8_t t = s.type[n];
     const Real lx = s.lam[n];
     Real m = s.m[n];
-    if (link >> 31) {
-      s.rhohat_w[n] = a.wall_rho;
-      return 0u;
-    }
-    if (t == CELL_EMPTY) {
-      s.rhohat_w[n] = Real(0);
-      return 0u;
-    }
+    if (t == CELL_EMPTY) return;
     const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
     const T *fin = static_cast<const T *>(a.f_in);
     // directions that exchange, and those to an interface cell
@@ -211,7 +215,6 @@ __global__ void __launch_bounds__(FS_BLOCK, sizeof(typename S::Real) == 4 ? 12 :
     part(std::integral_constant<int, 10>{});
     s.m[n] = m;
     s.rhohat_w[n] = m;
-    return 0u;
   });
 }
 
@@ -223,7 +226,7 @@ __global__ void __launch_bounds__(FS_BLOCK, sizeof(typename S::Real) == 4 ? 12 :
 // and surface tension; then lambda = m / rho, and the cells that fill or empty
 // are flagged and listed. Populations, colour-gradient field and types of the
 // neighbours are loaded together; the populations whose source turns out
-// empty are replaced.
+// empty, solid or a wall are replaced.
 template <class S>
 __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
     fs_step_kernel(const FsArgs<typename S::Real> s) {
@@ -234,23 +237,17 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
   const unsigned N = a.N;
   const unsigned c = s.cnt->now;
   if (blockIdx.x == 0 && threadIdx.x == 0) s.cnt->step = c + 1u;  // read by the next step's first pass
-  fs_tile_loop<true>(s, c, [&](unsigned x, unsigned y, unsigned z, unsigned lx, unsigned ly,
-                               unsigned lz) -> unsigned {
-  const unsigned n = x + a.nx * (y + a.ny * z);
+  fs_cell_loop(s, c, [&](unsigned n, unsigned x, unsigned y, unsigned z) {
   const uint32_t link = a.link ? __ldg(a.link + n) : 0u;
   const uint8_t t = s.type[n];
-  if ((link >> 31) || t == CELL_EMPTY) return 0u;
   const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
   const T *__restrict__ fin = static_cast<const T *>(a.f_in);
   T *__restrict__ fout = static_cast<T *>(a.f_out);
   const Real eps = __ldg(a.eps + n);
-  const uint32_t bounce = bounce_mask(link, g.onface & a.f_wall);
   Real d[Q];
   Unroll<0, Q>::run([&](auto qc) {
     constexpr int q = decltype(qc)::value;
-    const bool b = (bounce >> q) & 1u;
-    d[q] = S::template ld_f<q>(fin + size_t(b ? opp(q) : q) * N + (long long)n +
-                               (b ? 0 : src_delta<q>(g)));
+    d[q] = S::template ld_f<q>(fin + size_t(q) * N + (long long)n + src_delta<q>(g));
   });
   // sources that are empty cells
   uint32_t from_gas = 0;
@@ -258,11 +255,18 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
     constexpr int q = decltype(qc)::value;
     if (s.type[(long long)n + src_delta<q>(g)] == CELL_EMPTY) from_gas |= 1u << q;
   });
-  from_gas &= ~bounce;
   FluidCollide<Real> fc;
   fc.F[0] = fc.F[1] = fc.F[2] = Real(0);
   if (a.A != Real(0)) colour_gradient(a.rhohat, n, g, a.f_wall, a.wall_rho, fc.F);
   const Real mass = s.m[n];
+  if (t == CELL_EMPTY) return;
+  const uint32_t bounce = bounce_mask(link, g.onface & a.f_wall);
+  from_gas &= ~bounce;
+  if (bounce)
+    Unroll<1, Q>::run([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      if ((bounce >> q) & 1u) d[q] = S::template ld_f<opp(q)>(fin + size_t(opp(q)) * N + n);
+    });
   // f^eq_q - w_q at gas density 1 and the cell's own V' (time t), formed per
   // direction from u, 1/eps and u.u (a 19-value array held the kernel at 128
   // registers)
@@ -284,7 +288,7 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
     const Real guu = gu0 * gu0 + gu1 * gu1 + gu2 * gu2;
     auto ge = [&](auto qc) {
       constexpr int q = decltype(qc)::value;
-      const Real cu = Real(cx(q)) * gu0 + Real(cy(q)) * gu1 + Real(cz(q)) * gu2;
+      const Real cu = dot_c<q>(gu0, gu1, gu2);
       return wq<Real>(q) * (Real(3) * cu + Real(4.5) * gie * cu * cu - Real(1.5) * gie * guu);
     };
     Unroll<1, Q>::run([&](auto qc) {
@@ -351,17 +355,9 @@ __global__ void __launch_bounds__(FS_BLOCK, fs_step_blocks<typename S::Real>())
       s.flagged[atomicAdd(&s.cnt->n_flag, 1u)] = n;
     }
   }
-  // the tiles the next list needs: every cell within one link of this one
-  return fs_rebuilds(c) ? fs_tile_mask(lx, ly, lz, true, true) : 0u;
   });
 }
 
-// Sets bits of a cell's flag byte; returns the byte before.
-template <class Real>
-__device__ __forceinline__ unsigned fs_flag_or(const FsArgs<Real> &s, unsigned n, unsigned bits) {
-  const unsigned sh = 8u * (n & 3u);
-  return (atomicOr(reinterpret_cast<unsigned *>(s.flag) + (n >> 2), bits << sh) >> sh) & 0xffu;
-}
 // Component `axis` of c_q for the direction q = lane (0 beyond Q), from the
 // table packed in two bits each.
 __device__ __forceinline__ int fs_lane_c(unsigned lane, int axis) {
@@ -375,6 +371,36 @@ __device__ __forceinline__ int fs_lane_c(unsigned lane, int axis) {
   const unsigned long long p = axis == 0 ? px : axis == 1 ? py : pz;
   return lane < Q ? int((p >> (2 * lane)) & 3u) - 1 : 0;
 }
+
+// The neighbour n + c_q of a cell for the direction q = lane of a warp (lane 0:
+// the cell itself); there: it exists and is not solid.
+struct FsLane {
+  unsigned y;
+  bool there;
+};
+template <class Real>
+__device__ __forceinline__ FsLane fs_lane(const FsArgs<Real> &s, unsigned n, unsigned x, unsigned y,
+                                          unsigned z, unsigned lane) {
+  const StepArgs<Real> &a = s.a;
+  const int dx = fs_lane_c(lane, 0), dy = fs_lane_c(lane, 1), dz = fs_lane_c(lane, 2);
+  const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
+  const unsigned ahead = (dx > 0 ? 2u : 0u) | (dx < 0 ? 1u : 0u) | (dy > 0 ? 8u : 0u) |
+                         (dy < 0 ? 4u : 0u) | (dz > 0 ? 32u : 0u) | (dz < 0 ? 16u : 0u);
+  FsLane l;
+  l.y = n + unsigned((dx > 0 ? g.dxp : (dx < 0 ? g.dxm : 0)) +
+                     (dy > 0 ? g.dyp : (dy < 0 ? g.dym : 0)) +
+                     (dz > 0 ? g.dzp : (dz < 0 ? g.dzm : 0)));
+  l.there = lane < Q && !(ahead & g.onface & a.f_wall) && !(a.link && (a.link[l.y] >> 31));
+  return l;
+}
+
+// Sets bits of a cell's flag byte; returns the byte before.
+template <class Real>
+__device__ __forceinline__ unsigned fs_flag_or(const FsArgs<Real> &s, unsigned n, unsigned bits) {
+  const unsigned sh = 8u * (n & 3u);
+  return (atomicOr(reinterpret_cast<unsigned *>(s.flag) + (n >> 2), bits << sh) >> sh) & 0xffu;
+}
+
 // a cell's settled flag: filled, emptied, or neither
 __device__ __forceinline__ bool fs_settled(unsigned b) {
   return (b & FS_FILL) || ((b & FS_EMPTYING) && !(b & FS_CANCELLED));
@@ -412,23 +438,17 @@ template <class Real>
 __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_convert_kernel(const FsArgs<Real> s) {
   const StepArgs<Real> &a = s.a;
   const unsigned c = s.cnt->now, k = s.cnt->n_flag, lane = threadIdx.x & 31u;
-  const int dx = fs_lane_c(lane, 0), dy = fs_lane_c(lane, 1), dz = fs_lane_c(lane, 2);
   for (unsigned i = (blockIdx.x * FS_LIST_BLOCK + threadIdx.x) >> 5; i < k;
        i += gridDim.x * FS_LIST_BLOCK >> 5) {
     const unsigned n = s.flagged[i];
     const bool fill = s.flag[n] & FS_FILL;
     // this lane's neighbour n + c_lane (lane 0: the cell itself)
     const unsigned yz = a.by_nx.div(n), x = n - yz * a.nx, z = a.by_ny.div(yz), y = yz - z * a.ny;
-    const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
-    const unsigned ahead = (dx > 0 ? 2u : 0u) | (dx < 0 ? 1u : 0u) | (dy > 0 ? 8u : 0u) |
-                           (dy < 0 ? 4u : 0u) | (dz > 0 ? 32u : 0u) | (dz < 0 ? 16u : 0u);
-    const unsigned b = n + unsigned((dx > 0 ? g.dxp : (dx < 0 ? g.dxm : 0)) +
-                                    (dy > 0 ? g.dyp : (dy < 0 ? g.dym : 0)) +
-                                    (dz > 0 ? g.dzp : (dz < 0 ? g.dzm : 0)));
-    bool there = lane < Q && !(ahead & g.onface & a.f_wall);
-    const unsigned fb = there ? s.flag[b] : 0u;
-    const uint8_t tb = there ? s.type[b] : uint8_t(CELL_INTERFACE);
-    if (there && a.link && (a.link[b] >> 31)) there = false;
+    const FsLane l = fs_lane(s, n, x, y, z, lane);
+    const unsigned b = l.y;
+    const bool there = l.there;
+    const unsigned fb = s.flag[b];
+    const uint8_t tb = s.type[b];
     if (!fill && __any_sync(0xffffffffu, there && lane > 0 && (fb & FS_FILL))) {
       if (lane == 0) fs_flag_or(s, n, FS_CANCELLED);
       continue;
@@ -440,14 +460,73 @@ __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_convert_kernel(const FsArgs<
       fresh = fill && tb == CELL_EMPTY;
       if (fresh || (!fill && tb == CELL_LIQUID)) s.type[b] = CELL_INTERFACE;
     }
-    const bool first =
-        there && !(fs_flag_or(s, b, FS_CLAIMED | (fresh ? unsigned(FS_NEWCELL) : 0u)) & FS_CLAIMED);
+    const unsigned was =
+        there ? fs_flag_or(s, b, FS_CLAIMED | (fresh ? unsigned(FS_NEWCELL) : 0u)) : 0u;
+    const bool first = there && !(was & FS_CLAIMED);
     const unsigned won = __ballot_sync(0xffffffffu, first);
     unsigned at = 0;
     if (lane == 0 && won) at = atomicAdd(&s.cnt->n_near[c & 1u], unsigned(__popc(won)));
     at = __shfl_sync(0xffffffffu, at, 0);
     if (first) s.near[at + __popc(won & ((1u << lane) - 1u))] = b;
+    // new cells also from the end of the flagged list (the two are disjoint):
+    // the flag of the first to mark it tells which thread lists it
+    if (fresh && !(was & FS_NEWCELL)) s.flagged[a.N - 1u - atomicAdd(&s.cnt->n_new, 1u)] = b;
   }
+}
+
+// A new interface cell, by a warp (lane q its neighbour and its population in
+// direction q; as a thread's serial code the launch took 11 us for a few dozen
+// cells): f = f^eq(mean rho, mean V') of its liquid and interface neighbours that
+// are not new themselves. Sums run in the order of q.
+template <class S>
+__device__ __forceinline__ void fs_new_cell(const FsArgs<typename S::Real> &s, unsigned n,
+                                            unsigned lane, unsigned e, bool rebuilds) {
+  using Real = typename S::Real;
+  const StepArgs<Real> &a = s.a;
+  const unsigned N = a.N, all = 0xffffffffu;
+  const unsigned yz = a.by_nx.div(n), x = n - yz * a.nx, z = a.by_ny.div(yz), y = yz - z * a.ny;
+  const FsLane l = fs_lane(s, n, x, y, z, lane);
+  // density and V' of each neighbour as its collision in this step left them
+  // (its post-collision populations carry the same moments: the collision
+  // conserves mass, and without Darcy drag their momentum is rho (V' + eps G / 2))
+  const Real m0 = s.mom[l.y], m1 = s.mom[size_t(N) + l.y], m2 = s.mom[2 * size_t(N) + l.y],
+             m3 = s.mom[3 * size_t(N) + l.y];
+  const bool in = l.there && lane > 0 && s.type[l.y] != CELL_EMPTY && !(s.flag[l.y] & FS_NEWCELL);
+  const unsigned old = __ballot_sync(all, in);
+  Real rs = Real(0), u0 = Real(0), u1 = Real(0), u2 = Real(0);
+  for (unsigned b = old; b; b &= b - 1u) {
+    const int q = __ffs(b) - 1;
+    rs += __shfl_sync(all, m0, q);
+    u0 += __shfl_sync(all, m1, q);
+    u1 += __shfl_sync(all, m2, q);
+    u2 += __shfl_sync(all, m3, q);
+  }
+  const int cnt = __popc(old);
+  const Real ic = Real(1) / Real(cnt > 0 ? cnt : 1);
+  const Real r = cnt > 0 ? rs * ic : Real(1);
+  const Real u[3] = {u0 * ic, u1 * ic, u2 * ic};
+  const Real eps = a.eps[n];
+  const Real ie = Real(1) / eps, uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  const int dx = fs_lane_c(lane, 0), dy = fs_lane_c(lane, 1), dz = fs_lane_c(lane, 2);
+  const Real cu = Real(dx) * u[0] + Real(dy) * u[1] + Real(dz) * u[2];
+  const Real w = lane == 0 ? wq<Real>(0) : (dx * dx + dy * dy + dz * dz == 1 ? wq<Real>(5) : wq<Real>(1));
+  const Real dev =
+      w * ((r - Real(1)) + r * (Real(3) * cu + Real(4.5) * ie * cu * cu - Real(1.5) * ie * uu));
+  if (lane < Q) static_cast<typename S::T *>(a.f_out)[size_t(lane) * N + n] = dev;
+  Real rp = Real(0);
+  for (int q = 0; q < Q; ++q) rp += __shfl_sync(all, dev, q);
+  if (lane == 0) {
+    // it joins the cell list, unless it emptied in this epoch and is listed
+    if (!rebuilds && s.rho_post[n] != -Real(e + 1u))
+      s.cells[atomicAdd(&s.cnt->n_cells[e & 1u], 1u)] = n;
+    s.rho_post[n] = Real(1) + rp;  // the density of the stored populations, for lambda
+    if (a.fields) write_fields(a.fields, N, n, r, u, Real(0), (a.tau - Real(0.5)) / Real(3));
+  }
+  // the tiles within one link of it join the tile list
+  const unsigned mask = fs_tile_mask(x % FS_TX, y % FS_TY, z % FS_TZ, true, true);
+  if ((mask >> lane) & 1u)
+    fs_add_tile(s, fs_tile_near(s, x / FS_TX, y / FS_TY, z / FS_TZ, lane),
+                rebuilds ? e + 1u : e);
 }
 
 // New interface cells take f = f^eq(mean rho, mean V') of their liquid and
@@ -455,62 +534,32 @@ __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_convert_kernel(const FsArgs<
 // equilibrium, no mass); filled and emptied cells hand their excess mass (m -
 // rho, or m) in equal shares to the neighbours that are interface cells after
 // the re-typing (they keep it when there are none). The share waits in the
-// converted cell's liquid fraction, which only interface cells use.
+// converted cell's liquid fraction, which only interface cells use; an emptied
+// cell's density, which only liquid and interface cells use, notes the epoch.
+// The tiles around new interface cells join the tile list (the next one when
+// this step builds it).
 template <class S>
 __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_newcell_kernel(const FsArgs<typename S::Real> s) {
   using Real = typename S::Real;
   using T = typename S::T;
   const StepArgs<Real> &a = s.a;
   const unsigned N = a.N;
-  const unsigned c = s.cnt->now, k = s.cnt->n_near[c & 1u];
-  for (unsigned i = blockIdx.x * FS_LIST_BLOCK + threadIdx.x; i < k; i += gridDim.x * FS_LIST_BLOCK) {
-  const unsigned n = s.near[i];
-  const unsigned f = s.flag[n];
-  if (!(f & FS_NEWCELL) && !fs_settled(f)) continue;
-  const uint32_t link = a.link ? a.link[n] : 0u;
-  const unsigned yz = a.by_nx.div(n), x = n - yz * a.nx, z = a.by_ny.div(yz), y = yz - z * a.ny;
-  const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
-  if (f & FS_NEWCELL) {
-    // density and V' of each neighbour as its collision in this step left
-    // them (its post-collision populations carry the same moments: the
-    // collision conserves mass, and without Darcy drag their momentum is
-    // rho (V' + eps G / 2)); the loads of all neighbours are in flight together
-    const uint32_t old = fs_neighbors_that(n, g, link, a.f_wall, [&](unsigned y) {
-      return s.type[y] != CELL_EMPTY && !(s.flag[y] & FS_NEWCELL);
-    });
-    Real rs = Real(0), u0 = Real(0), u1 = Real(0), u2 = Real(0);
-    const int cnt = __popc(old);
-    Unroll<1, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      const unsigned y = unsigned((long long)n + ahead_delta<q>(g));
-      const Real m0 = s.mom[y], m1 = s.mom[size_t(N) + y], m2 = s.mom[2 * size_t(N) + y],
-                 m3 = s.mom[3 * size_t(N) + y];
-      const bool in = (old >> q) & 1u;
-      rs = in ? rs + m0 : rs;
-      u0 = in ? u0 + m1 : u0;
-      u1 = in ? u1 + m2 : u1;
-      u2 = in ? u2 + m3 : u2;
-    });
-    const Real ic = Real(1) / Real(cnt > 0 ? cnt : 1);
-    const Real r = cnt > 0 ? rs * ic : Real(1);
-    const Real u[3] = {u0 * ic, u1 * ic, u2 * ic};
-    const Real eps = a.eps[n];
-    const Real ie = Real(1) / eps, uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    T *fout = static_cast<T *>(a.f_out);
-    Real rp = Real(0);
-    Unroll<0, Q>::run([&](auto qc) {
-      constexpr int q = decltype(qc)::value;
-      const Real cu = Real(cx(q)) * u[0] + Real(cy(q)) * u[1] + Real(cz(q)) * u[2];
-      const Real dev = wq<Real>(q) * ((r - Real(1)) +
-                                      r * (Real(3) * cu + Real(4.5) * ie * cu * cu -
-                                           Real(1.5) * ie * uu));
-      S::template st_f<q>(fout + size_t(q) * N + n, dev);
-      rp += dev;
-    });
-    s.rho_post[n] = Real(1) + rp;  // the density of the stored populations, for lambda
-    if (a.fields) write_fields(a.fields, N, n, r, u, Real(0), (a.tau - Real(0.5)) / Real(3));
-    continue;
+  const unsigned c = s.cnt->now;
+  if (!(blockIdx.x & 1u)) {  // the even blocks take the new cells
+    const unsigned lane = threadIdx.x & 31u, k = s.cnt->n_new, e = fs_epoch(c);
+    for (unsigned i = ((blockIdx.x >> 1) * FS_LIST_BLOCK + threadIdx.x) >> 5; i < k;
+         i += (gridDim.x >> 1) * FS_LIST_BLOCK >> 5)
+      fs_new_cell<S>(s, s.flagged[N - 1u - i], lane, e, fs_rebuilds(c));
+    return;
   }
+  const unsigned k = s.cnt->n_flag;
+  for (unsigned i = (blockIdx.x >> 1) * FS_LIST_BLOCK + threadIdx.x; i < k;
+       i += (gridDim.x >> 1) * FS_LIST_BLOCK) {
+  const unsigned n = s.flagged[i];
+  const uint32_t link = a.link ? a.link[n] : 0u;
+  const CellGeo g = cell_geo(n, a.nx, a.ny, a.nz);
+  const unsigned f = s.flag[n];
+  if (!fs_settled(f)) continue;  // cancelled
   const int cnt = __popc(fs_neighbors_that(
       n, g, link, a.f_wall, [&](unsigned y) { return s.type[y] == CELL_INTERFACE; }));
   // a filled cell keeps m = rho: its post-collision density in the collision
@@ -523,13 +572,16 @@ __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_newcell_kernel(const FsArgs<
     s.m[n] = m - excess;
   }
   s.lam[n] = share;
-  if (!(f & FS_FILL)) zero_fields(s.fields, N, n);  // emptied
+  if (!(f & FS_FILL)) {  // emptied; its entry in this epoch's list stays
+    zero_fields(s.fields, N, n);
+    s.rhohat_w[n] = Real(0);
+    s.rho_post[n] = -Real(fs_epoch(c) + 1u);
+  }
   }
 }
 
 // Excess mass arrives at the interface cells near a conversion; their lambda =
-// m / rho; the tiles around new interface cells join the list (the next one
-// when this step builds it).
+// m / rho. The last step of an epoch builds both lists.
 template <class S>
 __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_finish_kernel(const FsArgs<typename S::Real> s) {
   using Real = typename S::Real;
@@ -539,7 +591,6 @@ __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_finish_kernel(const FsArgs<t
   for (unsigned i = blockIdx.x * FS_LIST_BLOCK + threadIdx.x; i < k; i += gridDim.x * FS_LIST_BLOCK) {
     const unsigned n = s.near[i];
     const uint8_t t = s.type[n];
-    const unsigned own = s.flag[n];
     const uint32_t link = a.link ? a.link[n] : 0u;
     const unsigned yz = a.by_nx.div(n), x = n - yz * a.nx, z = a.by_ny.div(yz), y = yz - z * a.ny;
     const CellGeo g = cell_geo_xyz(x, y, z, a.nx, a.ny, a.nz);
@@ -554,25 +605,11 @@ __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_finish_kernel(const FsArgs<t
     });
     s.m[n] = m;
     s.lam[n] = m / rho_post;
-    if (own & FS_NEWCELL) {
-      const unsigned bx = x / FS_TX, by = y / FS_TY, bz = z / FS_TZ;
-      // most of the tiles are listed: look at all of them together first, the
-      // atomics of the others run one after another
-      const unsigned mask = fs_tile_mask(x % FS_TX, y % FS_TY, z % FS_TZ, true, true);
-      unsigned missing = 0;
-      auto tile = [&](int j) {
-        const int mx = int(bx) + j % 3 - 1, my = int(by) + (j / 3) % 3 - 1, mz = int(bz) + j / 9 - 1;
-        const int X = int(s.ntx), Y = int(s.nty), Z = int(s.ntz);
-        return unsigned((mx < 0 ? mx + X : (mx >= X ? mx - X : mx)) +
-                        X * ((my < 0 ? my + Y : (my >= Y ? my - Y : my)) +
-                             Y * (mz < 0 ? mz + Z : (mz >= Z ? mz - Z : mz))));
-      };
-      Unroll<0, 27>::run([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        if (s.stamp[tile(j)] != e + 1u) missing |= 1u << j;
-      });
-      for (missing &= mask; missing; missing &= missing - 1u) fs_add_tile(s, tile(__ffs(missing) - 1), e);
-    }
+  }
+  if (fs_rebuilds(c)) {
+    const uint32_t *list = s.tiles[fs_epoch(c) & 1u];
+    const unsigned tiles = s.cnt->n_tiles[fs_epoch(c) & 1u];
+    for (unsigned i = blockIdx.x; i < tiles; i += gridDim.x) fs_scan_tile(s, list[i], e);
   }
 }
 
