@@ -489,7 +489,7 @@ struct FluidCollide {
   // + P9 cF) [+ S2 (c.F)^2] and B3 cu + P3 cF (cu = c_q.V', cF = c_q.F_e)
   template <int q>
   __device__ __forceinline__ void even_odd(Real cu, Real &ev, Real &od) const {
-    const Real cF = dot_c<q>(Fe[0], Fe[1], Fe[2]);
+    const Real cF = Real(cx(q)) * Fe[0] + Real(cy(q)) * Fe[1] + Real(cz(q)) * Fe[2];
     ev = fma(cu, fma(B45, cu, P9 * cF), K);
     if (st) {
       const Real cs = dot_c<q>(F[0], F[1], F[2]);
@@ -1354,12 +1354,13 @@ __device__ __forceinline__ CellIndex cell_index(const StepArgs<Real> &a, unsigne
 // Forchheimer 0.1139 / 0.1077 / 0.1254 / 0.1161, 117x83x101 with 10 % solid cells
 // 0.0905 / 0.0886 / 0.0938 / 0.0986, 256x192x64 with pressure faces 0.1655 /
 // 0.1690 / 0.1734 / 0.1775, three species 0.2265 / 0.2237 / 0.2162 / 0.2256,
-// 256^3 FP16 0.706 / 0.682 / 0.614 / 0.612; the batched kernel takes 6 (15
+// 256^3 FP16 0.706 / 0.682 / 0.628 / 0.607; the batched kernel takes 6 (15
 // lattices FP32 0.266 / 0.281 / 0.243 / 0.260). FP64 populations take twice the
 // registers, and its pipe is busy with a few warps.
 template <class S, bool SOLUTE, int FEAT>
 constexpr int step_blocks() {
   if (sizeof(typename S::Real) == 8) return 3;
+  if (S::kShift && SOLUTE && !(FEAT & FEAT_SPEC)) return 7;
   if (S::kShift || !SOLUTE || (FEAT & FEAT_SPEC)) return 6;
   return (FEAT & FEAT_OPEN) ? 4 : 5;
 }
