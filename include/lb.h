@@ -210,11 +210,11 @@ int lb_step(lb_ctx *ctx, int64_t n);
 /* CUDA graphs for lb_step and lb_step_batch (no counterpart in the paper;
  * default on). While a lattice's launches repeat exactly from one step pair
  * to the next (no time-dependent viscosity law, check_every 0 or 1; the free
- * surface keeps its tile lists and stamps on the device, so it qualifies),
- * the calls capture two steps, one of each buffer parity, into a
- * graph once and replay it for all but the last step of the call, which is
- * launched directly and exports the fields; the steps compute exactly what
- * direct launches compute. A batch graph is kept by the batch's first
+ * surface keeps its lists and counters on the device, so it qualifies),
+ * the calls capture pairs of steps, one of each buffer parity (one pair, and
+ * for long calls eight), into graphs once and replay them for all but the last
+ * step of the call, which is launched directly and exports the fields; the
+ * steps compute exactly what direct launches compute. A batch graph is kept by the batch's first
  * context for its members in that order and parity. enable = 0 drops the
  * context's graphs and launches every step directly. Synchronises the
  * context's stream. */
@@ -239,11 +239,10 @@ int lb_debug_graphs(const lb_ctx *ctx);
 int lb_autotune(lb_ctx *ctx, int32_t reps, int32_t *choice);
 
 /* Advance several lattices by the same n steps (continuous batching; no
- * counterpart in the paper). Per step, a lattice whose per-cell launch alone
- * fills the GPU (at least 6 blocks per SM), or that has pressure or velocity
- * faces, takes that launch; the smaller
- * lattices share one persistent launch per 64 lattices over a work list of
- * their cell blocks, their arguments travelling in the launch's parameters.
+ * counterpart in the paper). Per step, the lattices share one persistent
+ * launch per 64 of them over their concatenated blocks of cells, their
+ * arguments travelling in the launch's parameters; a lattice with pressure or
+ * velocity faces or several solute species takes its own per-cell launch.
  * Each lattice computes exactly what lb_step(n) with the per-cell kernel
  * computes.
  * All contexts: same storage, same permeability mode (none / diagonal / full),
@@ -311,9 +310,8 @@ void lb_destroy(lb_ctx *ctx);
  * allocate for a lattice of this domain and these parameters, each block
  * counted in 256-byte granules as the packed arena hands them out, with the
  * larger of the creation and initialisation staging blocks (the first is
- * released before the second is taken) and the lattice's share of a batch
- * work list (8 bytes per block of its per-cell launch, held by the first
- * context of an lb_step_batch call). Computed from the same layout that
+ * released before the second is taken) and an allowance for
+ * lb_step_batch (8 bytes per block of a per-cell launch by rows). Computed from the same layout that
  * lb_create allocates by; host arithmetic only, no device is touched.
  *   k_rows   rows of K^-1 kept: 0 (K NULL), 3 (a diagonal tensor field) or
  *            6 (a full tensor field; also the bound when unknown);

@@ -803,7 +803,6 @@ int lb_create(const lb_domain *dom, const float *porosity, const float *K6, cons
     c->ntx = (unsigned(dom->nx) + FS_TX - 1) / FS_TX;
     c->nty = (unsigned(dom->ny) + FS_TY - 1) / FS_TY;
     c->ntz = (unsigned(dom->nz) + FS_TZ - 1) / FS_TZ;
-    const size_t ntiles = size_t(c->ntx) * c->nty * c->ntz;
     c->tiles[0] = static_cast<uint32_t *>(dev_alloc(c, L.fs_tiles));
     c->tiles[1] = static_cast<uint32_t *>(dev_alloc(c, L.fs_tiles));
     c->stamp = static_cast<unsigned *>(dev_alloc(c, L.fs_stamp));
@@ -1009,7 +1008,7 @@ int lb_init(lb_ctx *c, const float *rho0, const float *u0, const float *C0,
     in.type = c->fs ? c->type : nullptr;
     CK(c, c->ops->init(c->kmode, c->solute, args, &in, c->nblk, c->stream));
     if (c->S > 1) CK(c, c->ops->species_init(args, d_u, d_C, c->nblk, c->stream));
-    if (c->fs) {  // the first step's active tiles
+    if (c->fs) {  // the first step's lists
       const FsArgs<Real> fa = fs_args(c, a);
       CK(c, c->ops->fs_seed(&fa, fs_tile_count(c), c->stream));
     }

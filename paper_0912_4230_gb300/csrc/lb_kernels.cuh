@@ -832,8 +832,12 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
   } else {
     constexpr Real w = wq<Real>(1);
     const Real itau = a.visc_law == 0 ? a.itau : rcp1(tau), omt = Real(1) - itau;
-    const Real it = w * itau, r3 = (Real(3) * it) * rho, r15 = Real(0.5) * r3;
-    const Real p3 = (Real(3) * w * fma(Real(-0.5), itau, Real(1))) * rho;
+    // (FP64 multiplies by rho last, so the factors of a constant tau are uniform;
+    // in FP32 their rounding, the same in every cell, doubled the error of u)
+    const Real it = w * itau, pf = fma(Real(-0.5), itau, Real(1));
+    constexpr bool last = sizeof(Real) == 8;
+    const Real r3 = last ? (Real(3) * it) * rho : Real(3) * (it * rho), r15 = Real(0.5) * r3;
+    const Real p3 = last ? (Real(3) * w * pf) * rho : Real(3) * w * (rho * pf);
     const Real ie3 = Real(3) * ie;
     Real K, Wv[3], X[3], VY = Real(0);
 #pragma unroll

@@ -54,7 +54,7 @@ struct StorageOps {
                           cudaStream_t s);
   cudaError_t (*totals)(PopView f, PopView h, const uint32_t *link, unsigned N, double *partials,
                         unsigned nblk, cudaStream_t s);
-  // one free-surface step, FsArgs<Real>*: two passes over the active tiles
+  // one free-surface step, FsArgs<Real>*: two passes over the listed live cells
   // (grid blocks each) and three launches over the converting cells; fs_seed
   // lists the first step's tiles after initialisation (one block per tile).
   // NULL when the storage format has no free-surface build

@@ -17,7 +17,7 @@
 // the per-cell path (update_cell) with its own global loads; the staged
 // values of such cells are not used. Every staged address is the wrapped
 // pull source of a cell inside the lattice, so it is in bounds for any cell.
-// The arithmetic of a cell is the per-cell kernel's (fluid_moments and
+// The arithmetic of a cell is the per-cell kernel's (moments and
 // collide_tail), so both kernels give the same results.
 #pragma once
 
