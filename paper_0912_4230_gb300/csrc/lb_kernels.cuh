@@ -1357,14 +1357,15 @@ __device__ __forceinline__ CellIndex cell_index(const StepArgs<Real> &a, unsigne
 // 5 / 6 / 7 blocks: 128^3 FP32 diagonal 0.1086 / 0.1067 / 0.1077 / 0.1135,
 // Forchheimer 0.1139 / 0.1077 / 0.1254 / 0.1161, 117x83x101 with 10 % solid cells
 // 0.0905 / 0.0886 / 0.0938 / 0.0986, 256x192x64 with pressure faces 0.1655 /
-// 0.1690 / 0.1734 / 0.1775, three species 0.2265 / 0.2237 / 0.2162 / 0.2256,
-// 256^3 FP16 0.706 / 0.682 / 0.628 / 0.607; the batched kernel takes 6 (15
+// 0.1690 / 0.1734 / 0.1775, three species 0.2249 / 0.2215 / 0.2223 / 0.2242,
+// 256^3 FP16 0.706 / 0.682 / 0.628 / 0.607, BF16 0.731 / 0.675 / 0.633 / 0.709
+// (0.681 before the packed collision); the batched kernel takes 6 (15
 // lattices FP32 0.266 / 0.281 / 0.243 / 0.260). FP64 populations take twice the
 // registers, and its pipe is busy with a few warps.
 template <class S, bool SOLUTE, int FEAT>
 constexpr int step_blocks() {
   if (sizeof(typename S::Real) == 8) return 3;
-  if (S::kShift && SOLUTE && !(FEAT & FEAT_SPEC)) return 7;
+  if (std::is_same<S, StoreF16>::value && SOLUTE && FEAT == 0) return 7;
   if (S::kShift || !SOLUTE || (FEAT & FEAT_SPEC)) return 6;
   return (FEAT & FEAT_OPEN) ? 4 : 5;
 }
