@@ -66,7 +66,7 @@ def _other_workloads():
         # free surface: algorithmic bytes counted per updated (liquid or interface) cell
         "drop": (lambda r: W.drop(seed=r), "fp32", 171,
                  "free-surface drop 192x192x128 (R 24, 40 cells above a solid wall), A 1e-3, "
-                 "FP32, five passes over the active tiles per step; roofline per updated cell"),
+                 "FP32, five launches over the live and converting cells per step; roofline per updated cell"),
     }
 
 
