@@ -270,8 +270,9 @@ __device__ __forceinline__ Real dot_c(Real a0, Real a1, Real a2) {
 __device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 
-// Reciprocal of a quantity of order one (density, porosity, relaxation time,
-// 1 + drag): the hardware's approximation and a Newton-Raphson step, r <- r +
+// Reciprocal of a normal number below 2^126 (density, porosity, relaxation time,
+// 1 + drag, a determinant below 2^120; beyond, the approximation is flushed to 0
+// and the correction of an infinity is not a number): the hardware's approximation and a Newton-Raphson step, r <- r +
 // r e, e = 1 - x r, in FP32 (from 1 ulp) or the third-order step r + r (e + e^2)
 // in FP64 (from 2^-20 to beyond 2^-53), without the range checks and slow path
 // of the exact reciprocal. An FP64 instruction holds its pipe for 64 cycles a
@@ -304,6 +305,32 @@ __device__ __forceinline__ float sqrt_iter(float x) {
   return r;
 }
 __device__ __forceinline__ double sqrt_iter(double x) { return sqrt(x); }
+
+// Lambda V' = r where the determinant leaves the range of FP32 (nearly tight
+// cells, K below ~1e-13 in every direction): with S = diag(s_i), s_i the power
+// of two that brings s_i^2 l_ii into [1, 4), V' = S (S Lambda S)^-1 S r, whose
+// determinant is at most 64. Scaling by powers of two rounds nothing.
+template <class Real>
+__device__ __forceinline__ void tight_solve(Real l00, Real l11, Real l22, Real l01, Real l12,
+                                            Real l02, Real r0, Real r1, Real r2, Real (&Vp)[3]) {
+  const auto half_scale = [](Real l) { return scalbn(Real(1), -(ilogb(l) / 2)); };
+  const Real s0 = half_scale(l00), s1 = half_scale(l11), s2 = half_scale(l22);
+  l00 = l00 * s0 * s0;
+  l11 = l11 * s1 * s1;
+  l22 = l22 * s2 * s2;
+  l01 = l01 * s0 * s1;
+  l12 = l12 * s1 * s2;
+  l02 = l02 * s0 * s2;
+  r0 *= s0;
+  r1 *= s1;
+  r2 *= s2;
+  const Real c00 = l11 * l22 - l12 * l12, c01 = l02 * l12 - l01 * l22, c02 = l01 * l12 - l02 * l11;
+  const Real c11 = l00 * l22 - l02 * l02, c12 = l01 * l02 - l00 * l12, c22 = l00 * l11 - l01 * l01;
+  const Real idet = Real(1) / (l00 * c00 + l01 * c01 + l02 * c02);
+  Vp[0] = s0 * ((c00 * r0 + c01 * r1 + c02 * r2) * idet);
+  Vp[1] = s1 * ((c01 * r0 + c11 * r1 + c12 * r2) * idet);
+  Vp[2] = s2 * ((c02 * r0 + c12 * r1 + c22 * r2) * idet);
+}
 
 // V' = Lambda^-1 (V + eps G / 2), Lambda = I + (eps nu / 2) K^-1, and
 // F^ext = -eps nu K^-1 V' + eps G (Eqs. forcement, expandV, expandVsub).
@@ -407,13 +434,20 @@ __device__ __forceinline__ void velocity_solve_kv(KV kv, Real eps, Real nu, cons
     const Real c00 = l11 * l22 - l12 * l12, c01 = l02 * l12 - l01 * l22, c02 = l01 * l12 - l02 * l11;
     const Real c11 = l00 * l22 - l02 * l02, c12 = l01 * l02 - l00 * l12, c22 = l00 * l11 - l01 * l01;
     const Real det = l00 * c00 + l01 * c01 + l02 * c02;
-    const Real idet = EXACT ? Real(1) / det : rcp1(det);
-    Vp[0] = (c00 * r0 + c01 * r1 + c02 * r2) * idet;
-    Vp[1] = (c01 * r0 + c11 * r1 + c12 * r2) * idet;
-    Vp[2] = (c02 * r0 + c12 * r1 + c22 * r2) * idet;
-    Fe[0] = -en * (kxx * Vp[0] + kxy * Vp[1] + kzx * Vp[2]) + eps * G[0];
-    Fe[1] = -en * (kxy * Vp[0] + kyy * Vp[1] + kyz * Vp[2]) + eps * G[1];
-    Fe[2] = -en * (kzx * Vp[0] + kyz * Vp[1] + kzz * Vp[2]) + eps * G[2];
+    // Lambda >= 1, so det bounds every cofactor; a sum that overflows may end at
+    // either infinity or not a number. (FP64 stays in range: k <= 1e45.)
+    if (sizeof(Real) == 4 && !(fabs(det) < Real(0x1p120))) {
+      tight_solve(l00, l11, l22, l01, l12, l02, r0, r1, r2, Vp);
+      for (int i = 0; i < 3; ++i) Fe[i] = Real(2) * (Vp[i] - V[i]);  // V' = V + F^ext / 2
+    } else {
+      const Real idet = EXACT ? Real(1) / det : rcp1(det);
+      Vp[0] = (c00 * r0 + c01 * r1 + c02 * r2) * idet;
+      Vp[1] = (c01 * r0 + c11 * r1 + c12 * r2) * idet;
+      Vp[2] = (c02 * r0 + c12 * r1 + c22 * r2) * idet;
+      Fe[0] = -en * (kxx * Vp[0] + kxy * Vp[1] + kzx * Vp[2]) + eps * G[0];
+      Fe[1] = -en * (kxy * Vp[0] + kyy * Vp[1] + kyz * Vp[2]) + eps * G[1];
+      Fe[2] = -en * (kzx * Vp[0] + kyz * Vp[1] + kzz * Vp[2]) + eps * G[2];
+    }
   }
 }
 
