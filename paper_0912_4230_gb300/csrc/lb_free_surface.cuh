@@ -35,18 +35,23 @@ constexpr unsigned fs_step_blocks() {
   return sizeof(Real) == 4 ? 640 / FS_BLOCK : 1;
 }
 
-// Tiles needed by the next step around one cell, as a mask over the 27
-// tile offsets (bit (dx+1) + 3(dy+1) + 9(dz+1)): the cell's own tile when
-// `self`, and with `halo` also the tiles holding its D3Q19 neighbours (a
-// neighbour lies in another tile only when the cell is on that tile face).
-__device__ __forceinline__ unsigned fs_tile_mask(unsigned lx, unsigned ly, unsigned lz, bool self,
-                                                 bool halo) {
-  if (!self && !halo) return 0u;
-  unsigned m = 1u << 13;
-  if (!halo) return m;
-  const int x0 = lx == 0 ? -1 : 0, x1 = lx == FS_TX - 1 ? 1 : 0;
-  const int y0 = ly == 0 ? -1 : 0, y1 = ly == FS_TY - 1 ? 1 : 0;
-  const int z0 = lz == 0 ? -1 : 0, z1 = lz == FS_TZ - 1 ? 1 : 0;
+// Tiles needed by the next step around cell (x, y, z), as a mask over the 27
+// tile offsets (bit (dx+1) + 3(dy+1) + 9(dz+1)): the cell's own tile and the
+// tiles holding its D3Q19 neighbours. A neighbour lies in another tile only
+// when the cell is on that face of its tile; the last tile of a row may be
+// partial and ends at the lattice's last cell, whose neighbour across the
+// periodic seam lies in the first tile.
+template <class Real>
+__device__ __forceinline__ unsigned fs_tile_mask(const FsArgs<Real> &s, unsigned x, unsigned y,
+                                                 unsigned z) {
+  const auto lo = [](unsigned v, unsigned tile) { return v % tile == 0 ? -1 : 0; };
+  const auto hi = [](unsigned v, unsigned tile, int n) {
+    return v % tile == tile - 1 || v + 1 == unsigned(n) ? 1 : 0;
+  };
+  const int x0 = lo(x, FS_TX), x1 = hi(x, FS_TX, s.a.nx);
+  const int y0 = lo(y, FS_TY), y1 = hi(y, FS_TY, s.a.ny);
+  const int z0 = lo(z, FS_TZ), z1 = hi(z, FS_TZ, s.a.nz);
+  unsigned m = 0u;
   for (int dz = z0; dz <= z1; ++dz)
     for (int dy = y0; dy <= y1; ++dy)
       for (int dx = x0; dx <= x1; ++dx)
@@ -110,7 +115,7 @@ __device__ __forceinline__ void fs_scan_tile(const FsArgs<Real> &s, unsigned til
   const unsigned n = x + s.a.nx * (y + s.a.ny * z);
   bool live = x < unsigned(s.a.nx) && y < unsigned(s.a.ny) && z < unsigned(s.a.nz);
   if (live) live = !(s.a.link && (s.a.link[n] >> 31)) && s.type[n] != CELL_EMPTY;
-  fs_stamp_tiles(s, bx, by, bz, fs_tile_mask(tx, ty, tz, live, live), e);
+  fs_stamp_tiles(s, bx, by, bz, live ? fs_tile_mask(s, x, y, z) : 0u, e);
   const unsigned row = __ballot_sync(0xffffffffu, live), lane = threadIdx.x & 31u;
   unsigned at = 0;
   if (lane == 0 && row) at = atomicAdd(&s.cnt->n_cells[e & 1u], unsigned(__popc(row)));
@@ -523,7 +528,7 @@ __device__ __forceinline__ void fs_new_cell(const FsArgs<typename S::Real> &s, u
     if (a.fields) write_fields(a.fields, N, n, r, u, Real(0), (a.tau - Real(0.5)) / Real(3));
   }
   // the tiles within one link of it join the tile list
-  const unsigned mask = fs_tile_mask(x % FS_TX, y % FS_TY, z % FS_TZ, true, true);
+  const unsigned mask = fs_tile_mask(s, x, y, z);
   if ((mask >> lane) & 1u)
     fs_add_tile(s, fs_tile_near(s, x / FS_TX, y / FS_TY, z / FS_TZ, lane),
                 rebuilds ? e + 1u : e);
