@@ -306,21 +306,23 @@ __device__ __forceinline__ float sqrt_iter(float x) {
 }
 __device__ __forceinline__ double sqrt_iter(double x) { return sqrt(x); }
 
-// Lambda V' = r where the determinant leaves the range of FP32 (nearly tight
-// cells, K below ~1e-13 in every direction): with S = diag(s_i), s_i the power
-// of two that brings s_i^2 l_ii into [1, 4), V' = S (S Lambda S)^-1 S r, whose
-// determinant is at most 64. Scaling by powers of two rounds nothing.
-template <class Real>
-__device__ __forceinline__ void tight_solve(Real l00, Real l11, Real l22, Real l01, Real l12,
-                                            Real l02, Real r0, Real r1, Real r2, Real (&Vp)[3]) {
+// Lambda V' = r, Lambda = 1 + hs K^-1, where the determinant leaves the range of
+// FP32 (nearly tight cells, K below ~1e-13 in every direction): with S = diag(s_i),
+// s_i the power of two that brings s_i^2 l_ii into [1, 4), V' = S (S Lambda S)^-1
+// S r, whose determinant is at most 64. Scaling by powers of two rounds nothing.
+// again(i) loads row i of K^-1 anew: kept in registers for this rare branch, the
+// rows cost a 256^3 FP16 solve 1.8 % in spills (25.50 to 25.95 ms; 25.76 so).
+template <class Real, class KV>
+__device__ __forceinline__ void tight_solve(KV again, Real hs, Real r0, Real r1, Real r2,
+                                            Real (&Vp)[3]) {
   const auto half_scale = [](Real l) { return scalbn(Real(1), -(ilogb(l) / 2)); };
+  Real l00 = Real(1) + hs * again(0), l11 = Real(1) + hs * again(1), l22 = Real(1) + hs * again(2);
   const Real s0 = half_scale(l00), s1 = half_scale(l11), s2 = half_scale(l22);
   l00 = l00 * s0 * s0;
   l11 = l11 * s1 * s1;
   l22 = l22 * s2 * s2;
-  l01 = l01 * s0 * s1;
-  l12 = l12 * s1 * s2;
-  l02 = l02 * s0 * s2;
+  const Real l01 = hs * again(3) * s0 * s1, l12 = hs * again(4) * s1 * s2,
+             l02 = hs * again(5) * s0 * s2;
   r0 *= s0;
   r1 *= s1;
   r2 *= s2;
@@ -335,7 +337,7 @@ __device__ __forceinline__ void tight_solve(Real l00, Real l11, Real l22, Real l
 // V' = Lambda^-1 (V + eps G / 2), Lambda = I + (eps nu / 2) K^-1, and
 // F^ext = -eps nu K^-1 V' + eps G (Eqs. forcement, expandV, expandVsub).
 // kv(r) returns row r of the cell's K^-1 (diagonal: xx, yy, zz; full: xx, yy,
-// zz, xy, yz, zx).
+// zz, xy, yz, zx); again(r) loads it anew, and as row 6 the porosity.
 //
 // KM_FORCH adds the Forchheimer drag of the porous-flow model the paper builds
 // on (the paper names the term without an equation): F^ext = -eps nu K^-1 V'
@@ -346,8 +348,8 @@ __device__ __forceinline__ void tight_solve(Real l00, Real l11, Real l22, Real l
 // closed form of an isotropic medium with the r^2-weighted a and b; three
 // iterations in FP32 and four in FP64 reach the root to rounding for K from
 // 1e-4 to 1e2, 100:1 anisotropy and cF up to 20.
-template <int KMODE, bool EXACT = false, class Real, class KV>
-__device__ __forceinline__ void velocity_solve_kv(KV kv, Real eps, Real nu, const Real (&V)[3],
+template <int KMODE, bool EXACT = false, class Real, class KV, class KA>
+__device__ __forceinline__ void velocity_solve_kv(KV kv, KA again, Real eps, Real nu, const Real (&V)[3],
                                                   const Real (&G)[3], Real cF, Real (&Vp)[3],
                                                   Real (&Fe)[3]) {
   const Real r0 = V[0] + Real(0.5) * eps * G[0];
@@ -434,19 +436,24 @@ __device__ __forceinline__ void velocity_solve_kv(KV kv, Real eps, Real nu, cons
     const Real c00 = l11 * l22 - l12 * l12, c01 = l02 * l12 - l01 * l22, c02 = l01 * l12 - l02 * l11;
     const Real c11 = l00 * l22 - l02 * l02, c12 = l01 * l02 - l00 * l12, c22 = l00 * l11 - l01 * l01;
     const Real det = l00 * c00 + l01 * c01 + l02 * c02;
+    const Real idet = EXACT ? Real(1) / det : rcp1(det);
+    Vp[0] = (c00 * r0 + c01 * r1 + c02 * r2) * idet;
+    Vp[1] = (c01 * r0 + c11 * r1 + c12 * r2) * idet;
+    Vp[2] = (c02 * r0 + c12 * r1 + c22 * r2) * idet;
+    Fe[0] = -en * (kxx * Vp[0] + kxy * Vp[1] + kzx * Vp[2]) + eps * G[0];
+    Fe[1] = -en * (kxy * Vp[0] + kyy * Vp[1] + kyz * Vp[2]) + eps * G[1];
+    Fe[2] = -en * (kzx * Vp[0] + kyz * Vp[1] + kzz * Vp[2]) + eps * G[2];
     // Lambda >= 1, so det bounds every cofactor; a sum that overflows may end at
     // either infinity or not a number. (FP64 stays in range: k <= 1e45.)
     if (sizeof(Real) == 4 && !(fabs(det) < Real(0x1p120))) {
-      tight_solve(l00, l11, l22, l01, l12, l02, r0, r1, r2, Vp);
-      for (int i = 0; i < 3; ++i) Fe[i] = Real(2) * (Vp[i] - V[i]);  // V' = V + F^ext / 2
-    } else {
-      const Real idet = EXACT ? Real(1) / det : rcp1(det);
-      Vp[0] = (c00 * r0 + c01 * r1 + c02 * r2) * idet;
-      Vp[1] = (c01 * r0 + c11 * r1 + c12 * r2) * idet;
-      Vp[2] = (c02 * r0 + c12 * r1 + c22 * r2) * idet;
-      Fe[0] = -en * (kxx * Vp[0] + kxy * Vp[1] + kzx * Vp[2]) + eps * G[0];
-      Fe[1] = -en * (kxy * Vp[0] + kyy * Vp[1] + kyz * Vp[2]) + eps * G[1];
-      Fe[2] = -en * (kzx * Vp[0] + kyz * Vp[1] + kzz * Vp[2]) + eps * G[2];
+      // V' = V + F^ext / 2 = r + (F^ext - eps G) / 2. (A product shared with the
+      // lines above would change which of their operations the compiler fuses,
+      // so eps is loaded too.)
+      tight_solve(again, hs, r0, r1, r2, Vp);
+      const Real e = again(6);
+      Fe[0] = Real(2) * (Vp[0] - r0) + e * G[0];
+      Fe[1] = Real(2) * (Vp[1] - r1) + e * G[1];
+      Fe[2] = Real(2) * (Vp[2] - r2) + e * G[2];
     }
   }
 }
@@ -456,8 +463,8 @@ __device__ __forceinline__ void velocity_solve(const Real *__restrict__ kinv, un
                                                unsigned n, Real eps, Real nu, const Real (&V)[3],
                                                const Real (&G)[3], Real (&Vp)[3],
                                                Real (&Fe)[3]) {
-  velocity_solve_kv<KMODE>([&](int r) { return __ldg(kinv + size_t(r) * N + n); }, eps, nu, V, G,
-                           Real(0), Vp, Fe);
+  auto row = [&](int r) { return r < 6 ? __ldg(kinv + size_t(r) * N + n) : eps; };
+  velocity_solve_kv<KMODE>(row, row, eps, nu, V, G, Real(0), Vp, Fe);
 }
 
 // Colour gradient F = sum_q rhohat(x + c_q) c_q (Eq. macros); a step out
@@ -791,7 +798,8 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
   const Real nu = a.visc_law == 0 ? a.nu0 : (tau - Real(0.5)) * Real(1.0 / 3.0);
   FluidCollide<Real> fc;
   Real(&Vp)[3] = fc.Vp, (&Fe)[3] = fc.Fe, (&F)[3] = fc.F;
-  velocity_solve_kv<KMODE, S::kShift>(kv, eps, nu, V, a.G, a.forch, Vp, Fe);
+  auto again = [&](int r) { return __ldcg(r < 6 ? a.kinv + size_t(r) * N + n : a.eps + n); };
+  velocity_solve_kv<KMODE, S::kShift>(kv, again, eps, nu, V, a.G, a.forch, Vp, Fe);
   Real Fn = Real(0);
   bool st = false;
   F[0] = F[1] = F[2] = Real(0);
