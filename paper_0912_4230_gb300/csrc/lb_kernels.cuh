@@ -77,6 +77,11 @@ struct Lat {
   __device__ __forceinline__ static Lat sub(Lat a, Lat b) {
     return mk(sub_rn(a.f, b.f), SOLUTE ? sub_rn(a.h, b.h) : Real(0));
   }
+  // gap = e.h - h/2, and the values af f + e.f, e.h - ah gap
+  __device__ __forceinline__ static Lat relax(Lat v, Lat e, Real af, Real ah, Real &gap) {
+    gap = SOLUTE ? ::fma(Real(-0.5), v.h, e.h) : Real(0);
+    return mk(::fma(af, v.f, e.f), SOLUTE ? ::fma(-ah, gap, e.h) : Real(0));
+  }
 };
 template <>
 struct Lat<float, true> {
@@ -110,6 +115,11 @@ struct Lat<float, true> {
     Lat r;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
+  }
+  __device__ __forceinline__ static Lat relax(Lat v, Lat e, float af, float ah, float &gap) {
+    const Lat t = fma(mk(af, -0.5f), v, e);
+    gap = t.hi();
+    return mk(t.lo(), fmaf(-ah, gap, e.hi()));
   }
 };
 
@@ -729,20 +739,23 @@ __device__ __forceinline__ float div_third(float x) {
 }
 
 // Solute collision of one lattice (Eq. equild, BGK) for itd = 1/tau_D, per
-// cell. Weighted rows: with e = itd sC / 36 and H = 3 e V*, h~_q = (1 - itd) h_q
-// + (e + c_q.H) for the diagonals, twice the bracket for the axes, and the
-// rest direction takes itd sC - 24 e, so the equilibrium adds no solute beyond
-// one rounding.
+// cell. With e = sC / 36 and H = 3 itd e V*, the sum s and the difference d of a
+// pair of opposite diagonals become twice e - (1 - itd) (e - s/2) and (1 - itd)/2 d +
+// c_q.H (axes: twice e and c_q.H), and the rest direction gives up what the 18
+// others gained, 2 itd sum (e - s/2). Roundings then scale with the distance from
+// the equilibrium, and a cell keeps its solute to those of the gains. Formed as
+// (1 - itd) s/2 + itd e, every collision lost ~1e-8 of the solute in FP32 (tau_D
+// 0.6, 0.75), and C was 3e-7 .. 5e-7 from the 64-bit result after 60 steps; now
+// 7e-8 .. 9e-8, and FP64 populations of a random medium 2.7e-16 instead of 5.2e-16.
 template <class Real>
 struct SoluteRows {
-  Real e, H[3], rest;
+  Real e, H[3];
   __device__ __forceinline__ void fold(Real sC, Real itd, Real v0, Real v1, Real v2) {
-    e = mul_rn(mul_rn(itd, wq<Real>(1)), sC);
-    const Real e3 = mul_rn(Real(3), e);
+    e = mul_rn(wq<Real>(1), sC);
+    const Real e3 = mul_rn(Real(3), mul_rn(itd, e));
     H[0] = mul_rn(e3, v0);
     H[1] = mul_rn(e3, v1);
     H[2] = mul_rn(e3, v2);
-    rest = fma(Real(-24), e, mul_rn(itd, sC));
   }
 };
 
@@ -904,6 +917,7 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
       ho = static_cast<T *>(a.h_out) + n;
     }
     const Real omd = Real(1) - itd;
+    Real gained = Real(0);  // by the moving solute, over 2 itd
     const L om = L::mk(omt, omd), half = L::mk(Real(0.5) * omt, Real(0.5) * omd);
     const L W2[3] = {L::mk(Wv[0], so.H[0]), L::mk(Wv[1], so.H[1]), L::mk(Wv[2], so.H[2])};
     const D VX[3] = {D::mk(Vp[0], X[0]), D::mk(Vp[1], X[1]), D::mk(Vp[2], X[2])};
@@ -921,7 +935,7 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
         const Real cs = dot_c<q>(F[0], F[1], F[2]);
         ev = fma(S2 * cs, cs, ev);
       }
-      L e = L::mk(ev, so.e);
+      L e = L::mk(ev, so.e);  // solute: the equilibrium itself
       if constexpr (inv_wq(q) == 18) {  // weight 2/36
         od = L::add(od, od);
         e = L::add(e, e);
@@ -929,7 +943,9 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
       const auto qq = std::integral_constant<int, q>{};
       const auto oo = std::integral_constant<int, o>{};
       if constexpr (SOLUTE) {
-        e = L::fma(half, sd[k], e);
+        Real gap;
+        e = L::relax(sd[k], e, half.lo(), omd, gap);
+        gained = k == 0 ? gap : add_rn(gained, gap);
         od = L::fma(half, sd[9 + k], od);
         store(qq, L::add(e, od));
         store(oo, L::sub(e, od));
@@ -938,8 +954,10 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
         store(oo, L::fma(om, L::mk(fv(oo), Real(0)), L::sub(e, od)));
       }
     });
+    const L r0 = sd[18];
     store(std::integral_constant<int, 0>{},
-          L::fma(om, sd[18], L::mk(mul_rn(Real(12), K0), so.rest)));
+          L::fma(L::mk(omt, Real(-2) * itd), L::mk(r0.lo(), gained),
+                 L::mk(mul_rn(Real(12), K0), r0.hi())));
   }
   if (a.fields) write_fields(a.fields, N, n, rho, Vp, C, nu);
   if constexpr (VOUT) {
@@ -1333,6 +1351,7 @@ __device__ __forceinline__ void species_update(const StepArgs<typename S::Real> 
     SoluteRows<Real> so;
     so.fold(sC, itd, vel[3] + gx, vel[4] + gy, vel[5] + gz);
     const Real om = Real(1) - itd, half = Real(0.5) * om;
+    Real gained = Real(0);
     Unroll<0, 9>::run([&](auto kc) {
       constexpr int k = decltype(kc)::value, q = pair_first(k), o = opp(q);
       Real od = along<q>(so.H, Lat1<Real>{}), e = so.e;
@@ -1340,12 +1359,14 @@ __device__ __forceinline__ void species_update(const StepArgs<typename S::Real> 
         od = add_rn(od, od);
         e = add_rn(e, e);
       }
-      e = fma(half, hh[q], e);
+      const Real gap = fma(Real(-0.5), hh[q], e);
+      gained = k == 0 ? gap : add_rn(gained, gap);
+      e = fma(-om, gap, e);
       od = fma(half, dif[k], od);
       S::template st_h<q>(ho + int(q * N), add_rn(e, od));
       S::template st_h<o>(ho + int(o * N), sub_rn(e, od));
     });
-    S::template st_h<0>(ho, fma(om, hh[0], so.rest));
+    S::template st_h<0>(ho, fma(Real(-2) * itd, gained, hh[0]));
   }
   if (a.fields) a.fields[(5 + size_t(sp)) * N + n] = float(sC * rcp(eps));
 }
