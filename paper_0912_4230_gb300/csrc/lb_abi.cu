@@ -379,7 +379,14 @@ void fill_args(const lb_ctx *c, StepArgs<Real> &a) {
   for (int i = 0; i < 3; ++i) a.G[i] = Real(c->prm.G[i]);
   a.tau = Real(c->prm.tau);
   a.itau = Real(1.0 / c->prm.tau);
-  a.nu0 = (a.tau - Real(0.5)) * Real(1.0 / 3.0);
+  if (c->prm.visc_law == 1) {
+    a.nu0 = Real((c->prm.tau0 - 0.5) / 3.0);
+    a.dnu = Real((c->prm.tau1 - c->prm.tau0) / 3.0);
+  } else if (c->ops->elt_bytes == 2) {
+    a.nu0 = (a.tau - Real(0.5)) * Real(1.0 / 3.0);  // as the 16-bit kernels form it
+  } else {
+    a.nu0 = Real((c->prm.tau - 0.5) / 3.0);
+  }
   a.tau0 = Real(c->prm.tau0);
   a.tau1 = Real(c->prm.tau1);
   a.beta = Real(c->prm.beta);

@@ -273,7 +273,8 @@ struct StepArgs {
                          // [24, 30) 3 x pressure minus its rounding to Real
   Real G[3];
   Real tau, tau0, tau1, beta;
-  Real itau, nu0;       // 1/tau and nu of the constant law
+  Real itau;            // 1/tau of the constant law
+  Real nu0, dnu;        // nu of law 0; law 1: nu0 + dnu C (formed in FP64)
   Real nu_t;            // law 2: nu_g (1 + a e^{alpha t}) at this step's t
   int visc_law;
   Real A, wall_rho;

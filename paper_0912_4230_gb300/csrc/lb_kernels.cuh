@@ -254,6 +254,19 @@ __device__ __forceinline__ Real tau_of(const StepArgs<Real> &a, Real C) {
   return a.tau;
 }
 
+// Viscosity from the law, not from the relaxation time: tau - 1/2 loses the
+// leading digits of a rounded tau (2.4e-7 of nu at tau 0.6 in FP32, and as much of
+// the velocity wherever the drag holds the flow).
+template <class Real>
+__device__ __forceinline__ Real nu_of(const StepArgs<Real> &a, Real C) {
+  if (a.visc_law == 1) {
+    const Real cl = C < Real(0) ? Real(0) : (C > Real(1) ? Real(1) : C);
+    return fma(a.dnu, cl, a.nu0);
+  }
+  if (a.visc_law == 2) return a.nu_t * exp(a.beta * (Real(1) - C));
+  return a.nu0;
+}
+
 // c_q . (a0, a1, a2) by additions of the axes that q has (a product with a zero
 // component is an instruction the compiler may not drop; in FP64 it holds the
 // pipe for 64 cycles).
@@ -808,7 +821,9 @@ __device__ __forceinline__ void collide_tail(const StepArgs<typename S::Real> &a
   const Real rho = Real(1) + drho;
   const Real C = SOLUTE ? sC * ie : Real(0);
   const Real tau = tau_of(a, C);
-  const Real nu = a.visc_law == 0 ? a.nu0 : (tau - Real(0.5)) * Real(1.0 / 3.0);
+  // (16-bit storage keeps the order of operations that its results are compared by)
+  const Real nu = !S::kShift ? nu_of(a, C)
+                             : (a.visc_law == 0 ? a.nu0 : (tau - Real(0.5)) * Real(1.0 / 3.0));
   FluidCollide<Real> fc;
   Real(&Vp)[3] = fc.Vp, (&Fe)[3] = fc.Fe, (&F)[3] = fc.F;
   auto again = [&](int r) { return __ldcg(r < 6 ? a.kinv + size_t(r) * N + n : a.eps + n); };
