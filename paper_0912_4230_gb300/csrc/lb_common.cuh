@@ -326,8 +326,8 @@ struct FsArgs {
   uint32_t *flagged;     // cells that fill or empty in this step; from its end, new cells
   uint32_t *near;        // converted cells and their neighbours
   Real *rho_post;        // post-collision density of each live cell (new interface cells:
-                         // of their initial populations); minus (1 + the epoch in which it
-                         // emptied) of a cell that has been live
+                         // of their initial populations); of a cell that has been live
+                         // the mark of the epoch in which it emptied (fs_mark)
   Real *mom;             // rho, V'_x, V'_y, V'_z (4 x N) of each live cell that pulls
                          // from an empty cell, written by the step pass
   FsCount *cnt;
@@ -342,6 +342,24 @@ struct FsArgs {
 };
 // steps that one cell list serves before it is built afresh
 constexpr unsigned FS_EPOCH = 16;
+// A mark of epoch e in place of a density: the negative number whose bits are e +
+// 1, another for every epoch of the step counter (2^28) in either type. (As the
+// number -(e + 1), FP32 marks of neighbouring epochs coincide from 2^24 on, 2^28
+// steps, and a new cell is taken to be listed already.)
+__host__ __device__ inline float fs_mark(unsigned e, float) {
+  union {
+    unsigned u;
+    float f;
+  } v = {0x80000000u | (e + 1u)};
+  return v.f;
+}
+__host__ __device__ inline double fs_mark(unsigned e, double) {
+  union {
+    unsigned long long u;
+    double f;
+  } v = {0x8000000000000000ull | (e + 1u)};
+  return v.f;
+}
 // the launches over the converting cells: a thread per cell
 constexpr unsigned FS_LIST_BLOCK = 64, FS_LIST_GRID = 304;
 constexpr unsigned FS_TX = 32, FS_TY = 1, FS_TZ = 2;

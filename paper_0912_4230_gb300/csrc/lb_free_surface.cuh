@@ -522,7 +522,7 @@ __device__ __forceinline__ void fs_new_cell(const FsArgs<typename S::Real> &s, u
   for (int q = 0; q < Q; ++q) rp += __shfl_sync(all, dev, q);
   if (lane == 0) {
     // it joins the cell list, unless it emptied in this epoch and is listed
-    if (!rebuilds && s.rho_post[n] != -Real(e + 1u))
+    if (!rebuilds && s.rho_post[n] != fs_mark(e, Real(0)))
       s.cells[atomicAdd(&s.cnt->n_cells[e & 1u], 1u)] = n;
     s.rho_post[n] = Real(1) + rp;  // the density of the stored populations, for lambda
     if (a.fields) write_fields(a.fields, N, n, r, u, Real(0), (a.tau - Real(0.5)) / Real(3));
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(FS_LIST_BLOCK) fs_newcell_kernel(const FsArgs<
   if (!(f & FS_FILL)) {  // emptied; its entry in this epoch's list stays
     zero_fields(s.fields, N, n);
     s.rhohat_w[n] = Real(0);
-    s.rho_post[n] = -Real(fs_epoch(c) + 1u);
+    s.rho_post[n] = fs_mark(fs_epoch(c), Real(0));
   }
   }
 }
