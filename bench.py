@@ -570,6 +570,8 @@ def main():
                                 else "step_kernel (fluid and every solute species)"
                                 if species > 1 else
                                 "tma_step_kernel (row-pipelined)" if choice == 256 else
+                                f"step_kernel, cells in order, blocks of {choice - 2000} threads"
+                                if choice > 2000 else
                                 f"pipe_step_kernel (row-staged), rows of {choice - 1000} threads"
                                 if choice > 1000 else
                                 f"step_kernel, rows of {choice or 'default'} threads"),

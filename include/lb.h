@@ -225,15 +225,17 @@ int lb_set_graphs(lb_ctx *ctx, int32_t enable);
 int lb_debug_graphs(const lb_ctx *ctx);
 
 /* Pick the step kernel and its launch shape by timing (no counterpart in the
- * paper): the per-cell kernel with rows of 32, 64 or 128 threads per block,
+ * paper): the per-cell kernel with rows of 32, 64 or 128 threads per block or
+ * over the cells in the order of n (blocks of 32 or 128 threads),
  * the row-staged kernel with rows of 32, 64 or 128 threads (FP32/FP64
  * storage), and the row-pipelined kernel where the lattice allows it. Each
  * candidate runs reps side-effect-free launches (input buffer to output
  * buffer without swapping, no flux accumulation, no checks, no field export),
  * so the state and t are unchanged. The fastest is kept for later lb_step
  * calls. *choice (may be NULL) receives the row width for the per-cell
- * kernel, 1000 + the row width for the row-staged kernel, 256 for the
- * row-pipelined kernel, or 0 when nothing was tuned (free surface or surface
+ * kernel (in the order of n: the threads of a block, plus 2000 where nx is no
+ * multiple of 32, so that its warps are not those of any rows), 1000 + the row
+ * width for the row-staged kernel, 256 for the row-pipelined kernel, or 0 when nothing was tuned (free surface or surface
  * tension keep fixed launches). Results of a step do not depend on the choice
  * beyond the order of the FP64 flux sums. */
 int lb_autotune(lb_ctx *ctx, int32_t reps, int32_t *choice);

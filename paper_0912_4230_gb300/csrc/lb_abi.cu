@@ -1282,7 +1282,11 @@ int lb_autotune(lb_ctx *c, int32_t reps, int32_t *choice) {
     c->sgrid = dim3((c->dom.nx + w.bx - 1) / w.bx, (c->dom.ny + c->sblock.y - 1) / c->sblock.y,
                     c->dom.nz);
   }
-  if (choice) *choice = w.kind == ROWS ? 256 : (w.kind == STAGED ? 1000 + int(w.bx) : int(w.bx));
+  if (choice) {
+    *choice = w.kind == ROWS ? 256 : (w.kind == STAGED ? 1000 + int(w.bx) : int(w.bx));
+    // the linear mapping: where whole warps fill a row its warps are those of the rows
+    if (w.kind == LINEAR) *choice = (c->dom.nx % 32 ? 2000 : 0) + int(c->sblock.x);
+  }
   return LB_OK;
 }
 

@@ -182,8 +182,10 @@ def lb_step(ctx, n: int):
 
 def lb_autotune(ctx, reps: int = 5) -> int:
     """Time the candidate kernels and launch shapes and keep the fastest;
-    returns the choice (per-cell kernel: the row width; row-staged kernel:
-    1000 + the row width; 256 = row-pipelined; 0 = not tuned)."""
+    returns the choice (per-cell kernel: the row width, or 2000 + the threads
+    of a block over the cells in order where nx is no multiple of 32;
+    row-staged kernel: 1000 + the row width; 256 = row-pipelined; 0 = not
+    tuned)."""
     ch = c_int32()
     _check(load().lb_autotune(ctx, int(reps), ctypes.byref(ch)), ctx)
     return ch.value
