@@ -1084,9 +1084,13 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   // only the last wave of a whole step is partly filled. Large ones too: 15
   // lattices of 32^3 .. 128^3 (FP32) step in 0.244 ms; with those of at least 1,
   // 2, 4 or 8 waves in launches of their own 0.302, 0.285, 0.261, 0.252 ms.
+  // (Tuned rows of a width that is no multiple of a warp sum their fluxes over
+  // other warps than the concatenation does: such a lattice keeps its launch.)
   std::vector<int> alone, shared;
-  for (int i = 0; i < n; ++i)
-    (ctxs[i]->open_faces || ctxs[i]->S > 1 ? alone : shared).push_back(i);
+  for (int i = 0; i < n; ++i) {
+    const bool own_warps = !ctxs[i]->linear && ctxs[i]->dom.nx % 32 != 0;
+    (ctxs[i]->open_faces || ctxs[i]->S > 1 || own_warps ? alone : shared).push_back(i);
+  }
   if (shared.size() == 1) {  // nothing to share with
     alone.push_back(shared[0]);
     shared.clear();
@@ -1131,13 +1135,14 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
       ctxs[i]->cur = 1 - ctxs[i]->cur;
     }
   };
-  // the graph of a step pair is valid for this set of lattices in this order
-  // and these parities
+  // the graph of a step pair is valid for this set of lattices in this order,
+  // these parities and these launch shapes (lb_autotune changes a member's)
   bool safe = true;
   std::vector<uint64_t> key;
   for (int i = 0; i < n; ++i) {
     safe = safe && graph_safe(ctxs[i]);
     key.push_back(ctxs[i]->serial * 2 + uint64_t(ctxs[i]->cur));
+    key.push_back(uint64_t(ctxs[i]->sblock.x) * 2 + uint64_t(ctxs[i]->linear));
   }
   int64_t k = 0;
   const int64_t pairs = steps > 0 ? (steps - 1) / 2 : 0;
