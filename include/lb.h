@@ -245,7 +245,8 @@ int lb_autotune(lb_ctx *ctx, int32_t reps, int32_t *choice);
  * launch per 64 of them over their concatenated blocks of cells, their
  * arguments travelling in the launch's parameters; a lattice with pressure or
  * velocity faces, with several solute species, or tuned (lb_autotune) to rows
- * whose width is no multiple of 32 takes its own per-cell launch.
+ * whose warps are not 32 consecutive cells each in the order of n takes its
+ * own per-cell launch.
  * Each lattice computes exactly what lb_step(n) with the per-cell kernel
  * computes.
  * All contexts: same storage, same permeability mode (none / diagonal / full),

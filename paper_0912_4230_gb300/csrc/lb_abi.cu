@@ -1084,11 +1084,13 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   // only the last wave of a whole step is partly filled. Large ones too: 15
   // lattices of 32^3 .. 128^3 (FP32) step in 0.244 ms; with those of at least 1,
   // 2, 4 or 8 waves in launches of their own 0.302, 0.285, 0.261, 0.252 ms.
-  // (Tuned rows of a width that is no multiple of a warp sum their fluxes over
-  // other warps than the concatenation does: such a lattice keeps its launch.)
+  // (A lattice tuned to rows whose warps are not those of the concatenation, or
+  // not in its order, sums its fluxes otherwise: it keeps its launch.)
   std::vector<int> alone, shared;
   for (int i = 0; i < n; ++i) {
-    const bool own_warps = !ctxs[i]->linear && ctxs[i]->dom.nx % 32 != 0;
+    const dim3 g = ctxs[i]->sgrid, b = ctxs[i]->sblock;
+    const bool own_warps = !ctxs[i]->linear && (ctxs[i]->dom.nx % b.x || ctxs[i]->dom.ny % b.y ||
+                                                (g.x > 1 && b.y > 1));
     (ctxs[i]->open_faces || ctxs[i]->S > 1 || own_warps ? alone : shared).push_back(i);
   }
   if (shared.size() == 1) {  // nothing to share with

@@ -3,8 +3,8 @@
 // The launch's blocks are the concatenation of every lattice's cells in blocks
 // of STEP_BLOCK in the order of n, with the warps and flux slots of the per-cell
 // step kernel (cell_index), so each lattice computes exactly what its own launch
-// would; one whose launch was tuned to rows that leave lanes empty sums its fluxes
-// over other warps and is not taken in. The grid is a fixed number of resident blocks that walk the
+// would; one whose launch was tuned to rows with other warps or another order of
+// them is not taken in. The grid is a fixed number of resident blocks that walk the
 // concatenation with stride gridDim.x. The lattices' arguments and first blocks
 // travel in the launch's parameter space (__grid_constant__), and a block finds
 // its lattice there from its number alone: everything up to the arguments is
@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(STEP_BLOCK, sizeof(typename S::Real) == 8 ? 3 
     for (int step = BATCH_MAX / 2; step > 0; step /= 2)
       if (d + step < tab.n && tab.begin[d + step] <= vb) d += step;
     const StepArgs<Real> &a = tab.a[d];
-    const CellIndex c = cell_index(a, vb - tab.begin[d], 0, 0, STEP_BLOCK, threadIdx.x, 0);
+    const CellIndex c = cell_index(a, vb - tab.begin[d], 0, 0, 0, 0, STEP_BLOCK, threadIdx.x, 0);
     const uint32_t link = (c.in && a.link) ? __ldg(a.link + c.n) : 0u;
     Real fin_acc = Real(0), fout_acc = Real(0), drho = Real(0), sC = Real(0);
     bool open_face = false;

@@ -1387,10 +1387,7 @@ __device__ __forceinline__ void species_update(const StepArgs<typename S::Real> 
 }
 
 // The cell of thread `tid` of block (bx, by, bz) of a per-cell launch with
-// rows of `row` threads, and its warp's number: the flux slot, the same for every
-// width of the rows and, where nx is a multiple of 32, for the linear mapping, so
-// that the flux sums do not depend on the launch (a lane beyond the lattice is in
-// no cell on a face, and uses no slot).
+// rows of `row` threads, and its warp's number in the launch (its flux slot).
 // Two mappings. Rows: block (row, STEP_BLOCK/row), grid (ceil(nx/row),
 // ceil(ny/(STEP_BLOCK/row)), nz), a warp covers 32 consecutive x of one row
 // (nothing to divide). Linear (a.linear): the threads of the launch take the
@@ -1403,7 +1400,8 @@ struct CellIndex {
 };
 template <class Real>
 __device__ __forceinline__ CellIndex cell_index(const StepArgs<Real> &a, unsigned bx, unsigned by,
-                                                unsigned bz, unsigned row, unsigned tx, unsigned ty,
+                                                unsigned bz, unsigned gx, unsigned gy, unsigned row,
+                                                unsigned tx, unsigned ty,
                                                 unsigned threads = STEP_BLOCK) {
   CellIndex c;
   if (a.linear) {
@@ -1421,7 +1419,7 @@ __device__ __forceinline__ CellIndex cell_index(const StepArgs<Real> &a, unsigne
     c.z = bz;
     c.in = c.x < unsigned(a.nx) && c.y < unsigned(a.ny);
     c.n = c.x + unsigned(a.nx) * (c.y + unsigned(a.ny) * c.z);
-    c.warp = (c.y + unsigned(a.ny) * c.z) * ((unsigned(a.nx) + 31u) >> 5) + (c.x >> 5);
+    c.warp = ((bz * gy + by) * gx + bx) * (STEP_BLOCK / 32) + ((ty * row + tx) >> 5);
   }
   return c;
 }
@@ -1452,8 +1450,8 @@ constexpr int step_blocks() {
 template <class S, int KMODE, bool SOLUTE, int FEAT>
 __global__ void __launch_bounds__(STEP_BLOCK, step_blocks<S, SOLUTE, FEAT>()) step_kernel(const StepArgs<typename S::Real> a) {
   using Real = typename S::Real;
-  const CellIndex c = cell_index(a, blockIdx.x, blockIdx.y, blockIdx.z, blockDim.x, threadIdx.x,
-                                 threadIdx.y, blockDim.x);
+  const CellIndex c = cell_index(a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y,
+                                 blockDim.x, threadIdx.x, threadIdx.y, blockDim.x);
   const unsigned x = c.x, y = c.y, z = c.z, n = c.n, warp_gid = c.warp;
   const uint32_t link = (c.in && a.link) ? __ldg(a.link + n) : 0u;
   Real fin_acc = Real(0), fout_acc = Real(0), drho = Real(0), sC = Real(0);
