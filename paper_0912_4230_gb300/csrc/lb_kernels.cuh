@@ -1424,29 +1424,26 @@ __device__ __forceinline__ CellIndex cell_index(const StepArgs<Real> &a, unsigne
   return c;
 }
 
-// One time step for every non-solid cell (see update_cell; launch shapes at
-// cell_index). Six resident 128-thread blocks per SM (at most 85 registers a
-// thread): measured on GB300 at 128^3 this is 1.1x faster than the
-// unconstrained build (112 registers), since the kernel is bound by loads in
-// flight, and a little faster than 256-thread blocks at the same occupancy.
 // Resident 128-thread blocks per SM of the per-cell kernel (registers a thread).
 // The kernel is bound by loads in flight, so warps are traded against registers
 // that keep a cell's ~48 loads together. Measured on GB300, ms per step with 4 /
-// 5 / 6 / 7 blocks: 128^3 FP32 diagonal 0.1086 / 0.1067 / 0.1077 / 0.1135,
-// Forchheimer 0.1139 / 0.1077 / 0.1254 / 0.1161, 117x83x101 with 10 % solid cells
-// 0.0905 / 0.0886 / 0.0938 / 0.0986, 256x192x64 with pressure faces 0.1655 /
-// 0.1690 / 0.1734 / 0.1775, three species 0.2249 / 0.2215 / 0.2223 / 0.2242,
-// 256^3 FP16 0.706 / 0.682 / 0.628 / 0.607, BF16 0.731 / 0.675 / 0.633 / 0.709
-// (0.681 before the packed collision); the batched kernel takes 6 (15
-// lattices FP32 0.266 / 0.281 / 0.243 / 0.260). FP64 populations take twice the
-// registers, and its pipe is busy with a few warps.
+// 5 / 6 / 7 blocks: 128^3 FP32 diagonal 0.1064 / 0.1050 / 0.1091 / 0.1134,
+// Forchheimer 0.1134 / 0.1064 / 0.1144 / 0.1180, 117x83x101 with 10 % solid cells
+// 0.0908 / 0.0893 / 0.0963 / 0.1004, 256^3 with a full tensor 0.838 / 0.833 / 0.902
+// / 0.909, 256x192x64 with pressure faces 0.1663 / 0.1650 / 0.1731 / 0.1796, three
+// species 0.2249 / 0.2118 / 0.2249 / 0.2242 (6 took 0.2201 before); 256^3 FP16 with a
+// full tensor 0.725 / 0.666 / 0.616 / 0.616, with a diagonal one 0.678 / 0.573 at 6 /
+// 7, BF16 0.754 / 0.740 / 0.640 / 0.702. The batched kernel takes 6 (15 lattices FP32
+// 0.269 / 0.286 / 0.245 / 0.256, 24 of 32^3 FP16 0.0509 / 0.0514 / 0.0430 / 0.0445).
+// FP64 populations take twice the registers, and its pipe is busy with a few warps.
 template <class S, bool SOLUTE, int FEAT>
 constexpr int step_blocks() {
   if (sizeof(typename S::Real) == 8) return 3;
   if (std::is_same<S, StoreF16>::value && SOLUTE && FEAT == 0) return 7;
-  if (S::kShift || !SOLUTE || (FEAT & FEAT_SPEC)) return 6;
-  return (FEAT & FEAT_OPEN) ? 4 : 5;
+  return S::kShift || !SOLUTE ? 6 : 5;
 }
+// One time step for every non-solid cell (see update_cell; launch shapes at
+// cell_index).
 template <class S, int KMODE, bool SOLUTE, int FEAT>
 __global__ void __launch_bounds__(STEP_BLOCK, step_blocks<S, SOLUTE, FEAT>()) step_kernel(const StepArgs<typename S::Real> a) {
   using Real = typename S::Real;
