@@ -314,8 +314,8 @@ void lb_destroy(lb_ctx *ctx);
  * allocate for a lattice of this domain and these parameters, each block
  * counted in 256-byte granules as the packed arena hands them out, with the
  * larger of the creation and initialisation staging blocks (the first is
- * released before the second is taken) and an allowance for
- * lb_step_batch (8 bytes per block of a per-cell launch by rows). Computed from the same layout that
+ * released before the second is taken) and a margin of 8 bytes per block of
+ * a per-cell launch by rows, which no call takes. Computed from the same layout that
  * lb_create allocates by; host arithmetic only, no device is touched.
  *   k_rows   rows of K^-1 kept: 0 (K NULL), 3 (a diagonal tensor field) or
  *            6 (a full tensor field; also the bound when unknown);

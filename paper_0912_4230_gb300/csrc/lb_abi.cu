@@ -152,7 +152,7 @@ void dev_free(lb_ctx *c, void *p) {
   if (c->release_fn) {
     // A caller's allocator may hand the block out again at once (the packed
     // arena does), while launches already enqueued on the context's stream
-    // (a batch work list, a graph replay) may still read it; cudaFree waits
+    // (a graph replay) may still read it; cudaFree waits
     // by itself, a release callback does not.
     cudaStreamSynchronize(c->stream);
     c->release_fn(p, c->alloc_user);
@@ -225,9 +225,14 @@ void row_shape(const lb_domain &dom, dim3 *grid, dim3 *block) {
 }
 // ... over the cells in order of n (never more blocks than by rows, which hold
 // STEP_BLOCK cells or fewer each, so the flux slots cover it too).
-// Where all warps of the launch are resident at once (152 SMs of 24 warps; FP64
-// 12) blocks of one warp spread them evenly: 254 warps of FP64 work are 2 on
-// the busiest SM instead of 4.
+// Small launches take blocks of one warp, which spread the work evenly: 254 warps of
+// FP64 work are 2 on the busiest SM instead of 4. FP64 up to its resident warps (3
+// blocks of 4 on each of 152 SMs): a miscible lattice 41 cells wide takes, with blocks
+// of one warp / of four, 16.5 / 17.5 us a step at 1 warp an SM, 24.3 / 26.9 at 6, 26.7 /
+// 27.1 at 8, 37.1 / 37.5 at 12. In FP32 and 16-bit storage, bound by latency, the two
+// are within a few per cent, up to 24 warps an SM: 32x32x45 FP32 (9.5 warps) 5.07 / 5.24
+// us; 41 cells wide FP32 4.82 / 4.95 at 1, 5.85 / 5.84 at 9.4, 6.55 / 6.22 at 16, 8.8 /
+// 8.7 at 24; FP16 6.7 / 6.9 at 9.4, 7.5 / 6.9 at 16.
 void linear_shape(const lb_domain &dom, bool fp64, dim3 *grid, dim3 *block) {
   const size_t N = size_t(dom.nx) * dom.ny * dom.nz;
   const unsigned threads = N <= size_t(152) * 32 * (fp64 ? 12 : 24) ? 32 : STEP_BLOCK;
@@ -272,7 +277,7 @@ struct Layout {
   size_t kinv, flux_slots;
   size_t create_stage;   // inputs of lb_create, released before it returns
   size_t init_stage;     // inputs of lb_init, kept for later staging
-  size_t batch_share;    // allowance for lb_step_batch (8 bytes per block of a launch by rows)
+  size_t batch_share;    // a margin that no call takes (8 bytes per block of a launch by rows)
 };
 
 Layout layout_of(const lb_domain &dom, const lb_params &prm, const StorageOps &ops, int k_rows,
@@ -1079,7 +1084,9 @@ int step_batch_t(lb_ctx *const *ctxs, int n, int64_t steps) {
   int dev = 0, sms = 0;
   CK(c0, cudaGetDevice(&dev));
   CK(c0, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const unsigned wave = unsigned(6 * sms);  // resident blocks of the per-cell kernel
+  // at most the resident blocks of the batched kernel in 32- and 16-bit storage; FP64
+  // holds 3 an SM, and the rest follow as those end
+  const unsigned wave = unsigned(6 * sms);
   // the lattices share persistent launches, their blocks concatenated, so that
   // only the last wave of a whole step is partly filled. Large ones too: 15
   // lattices of 32^3 .. 128^3 (FP32) step in 0.244 ms; with those of at least 1,

@@ -364,7 +364,8 @@ __host__ __device__ inline double fs_mark(unsigned e, double) {
 constexpr unsigned FS_LIST_BLOCK = 64, FS_LIST_GRID = 304;
 constexpr unsigned FS_TX = 32, FS_TY = 1, FS_TZ = 2;
 // threads per block: a tile's cells when lists are built, listed cells in the
-// passes, with as many blocks per SM as the stream/collide pass holds
+// passes, on a grid of at most as many blocks per SM as the mass pass holds (the
+// stream/collide pass holds 10 in FP32; further blocks follow as those end)
 constexpr unsigned FS_BLOCK = FS_TX * FS_TY * FS_TZ;
 constexpr unsigned FS_BLOCKS_PER_SM = 12;
 

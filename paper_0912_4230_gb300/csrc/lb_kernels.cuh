@@ -317,12 +317,14 @@ __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 
 // Reciprocal of a normal number below 2^126 (density, porosity, relaxation time,
 // 1 + drag, a determinant below 2^120; beyond, the approximation is flushed to 0
-// and the correction of an infinity is not a number): the hardware's approximation and a Newton-Raphson step, r <- r +
-// r e, e = 1 - x r, in FP32 (from 1 ulp) or the third-order step r + r (e + e^2)
-// in FP64 (from 2^-20 to beyond 2^-53), without the range checks and slow path
-// of the exact reciprocal. An FP64 instruction holds its pipe for 64 cycles a
-// warp on this chip (measured, whatever the active lanes), so 3 instead of ~10
-// count there.
+// and the correction of an infinity is not a number): the hardware's approximation
+// and a Newton-Raphson step, r <- r + r e, e = 1 - x r, in FP32 (from 1 ulp) or the
+// third-order step r + r (e + e^2) in FP64 (from 2^-20 to beyond 2^-53), without
+// the range checks and slow path of the exact reciprocal. FP32 results are those of
+// the correctly rounded reciprocal for every argument from 2^-100 to 2^126; of
+// 1.3e9 random FP64 ones 0.03 % differ in the last bit. An FP64 instruction holds its
+// pipe for 64 cycles a warp on this chip (measured, whatever the active lanes), so 3
+// instead of ~10 count there.
 __device__ __forceinline__ float rcp1(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -537,7 +539,7 @@ __device__ __forceinline__ void colour_gradient(const Real *__restrict__ rh, uns
 // direction they are w_q b_q with
 //   b_q = K + cu (B3 + B45 cu + P9 cF) + P3 cF [+ S2 (c_q.F)^2],
 // cu = c_q.V', cF = c_q.F_e (K0 in place of K for the rest direction), taken
-// taken as scale (b_q - shift). Used by the initialisation (feq_dev), the
+// as scale (b_q - shift). Used by the initialisation (feq_dev), the
 // free surface and 16-bit storage; the FP32/FP64 porous step folds further
 // (collide_tail).
 template <class Real>
@@ -809,9 +811,9 @@ struct SoluteRows {
 // directions are formed from the sum s and the difference d of their old
 // values as E + O and E - O, E = (1 - 1/tau)/2 s + w (K + (c.V')(c.X)), O = (1 -
 // 1/tau)/2 d + w c.W: for a pair of diagonals of both lattices two packed
-// additions give the dot products, one fma and two packed fmas E and O, two
-// packed additions the new values: 7 instructions where the unfolded form took
-// ~26. Where the density is away from 1 (E much larger than O: a wood sample
+// additions give the dot products, one fma and two packed fmas E and O, two more
+// instructions the solute's part of E (SoluteRows), two packed additions the new
+// values: 9 instructions where the unfolded form took ~26. Where the density is away from 1 (E much larger than O: a wood sample
 // under pressure) the rounding of E drops out of the momentum: after 60 steps
 // at 256x192x64 FP32 u is 4.1e-6 from the 64-bit result, 1.0e-5 before. Without
 // the solute the flow is driven by a force at density 1 (O the larger part),

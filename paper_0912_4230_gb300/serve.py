@@ -29,7 +29,8 @@ def device_bytes(prob, storage: str = "fp32") -> int:
     """Device memory one lattice of this problem takes, as the library
     allocates it (lb_bytes_required: the library's own allocation layout,
     each block in the packed arena's 256-byte granules, the larger of the
-    creation and initialisation staging, and an allowance for batches). A permeability field keeps 6 rows of K^-1 when any cell has
+    creation and initialisation staging, and a margin). A permeability
+    field keeps 6 rows of K^-1 when any cell has
     an off-diagonal entry, else 3."""
     from . import lb
     kr = 0
