@@ -88,9 +88,13 @@ __global__ void fields_kernel(const SetupArgs a) {
     const double c12 = M[0][1] * M[0][2] - M[0][0] * M[1][2];
     const double c22 = M[0][0] * M[1][1] - M[0][1] * M[0][1];
     const double det = M[0][0] * c00 + M[0][1] * c01 + M[0][2] * c02;
-    ki[n] = Real(c00 / det);
-    ki[size_t(N) + n] = Real(c11 / det);
-    ki[2 * size_t(N) + n] = Real(c22 / det);
+    // A diagonal tensor in FP32 is as tight as it gets at 2^100: V' is below 1e-20 of
+    // what arrives, and 1 + eps nu k / 2 stays where its reciprocal is normal (K = 1e-38
+    // would lose the drag at nu > 2).
+    const double most = sizeof(Real) == 4 && a.kmode != KM_SPD ? 0x1p100 : 1e300;
+    ki[n] = Real(fmin(c00 / det, most));
+    ki[size_t(N) + n] = Real(fmin(c11 / det, most));
+    ki[2 * size_t(N) + n] = Real(fmin(c22 / det, most));
     if (a.kmode == KM_SPD) {
       ki[3 * size_t(N) + n] = Real(c01 / det);
       ki[4 * size_t(N) + n] = Real(c12 / det);

@@ -65,3 +65,14 @@ def test_full_tensor_of_nearly_tight_cells(K, storage):
 @pytest.mark.parametrize("along", [(1.0, 1.0, 1e12), (1.0, 1e-8, 1e8), (1e4, 1.0, 1.0)])
 def test_full_tensor_tight_along_some_axes(along):
     check(tight_medium(1e-18, along=along), "fp32")
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp64"])
+def test_diagonal_tensor_at_the_smallest_permeability(storage):
+    """K = 1.5e-38 at nu = 4.8: 1 + eps nu k / 2 is 0.5e38 .. 1.6e38, on both sides
+    of 2^126 (the reciprocal of more is subnormal)."""
+    p = W.random_medium(19, 7, 6, seed=11, spd=False, visc_law=0)
+    K6 = np.asarray(p.K6, np.float64).reshape(-1, 6).copy()
+    tight = np.random.default_rng(4).uniform(size=p.N) < 1 / 3
+    K6[tight, :3] = 1.5e-38
+    check(p.replace(K6=K6.astype(np.float32).ravel(), params=dict(p.params, tau=15.0)), storage)
